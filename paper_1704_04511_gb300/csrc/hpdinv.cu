@@ -33,25 +33,25 @@ namespace recon {
 namespace {
 
 constexpr int kThreads = 256;
-// The Lanczos kernel: four warps per CTA (so that up to four launches fit on an SM at once, as
-// when several solves start together), each warp holding up to kLancRows rows of a matrix.
+// The Lanczos kernel: four warps per CTA, which keep the SM's FP64 pipe busy (one instruction per
+// ~19 cycles, one per ~64 and warp), and up to four launches on an SM at once, as when several
+// solves start together.
 constexpr int kLancThreads = 128;
-constexpr int kLancRows = 8;
 constexpr int kB = 8;                        // tile edge
 constexpr int kTileT = kB * kB;              // elements of a tile = threads of a tile group
 constexpr int kGroups = kThreads / kTileT;   // tile groups per CTA
 constexpr int kChunk = 4;                    // off-diagonal tiles of one row handled per CTA pass
 constexpr int kMaxItems = 128;               // work items one CTA may own
 constexpr long long kSpinLimit = 1LL << 24;  // polls (~1 us each at most) before giving up
-// Lanczos steps (tridiagonal order) at most. lambda_max of a Gram of image series converges to
-// rounding by ~16 steps (a dominant top eigenvalue); Grams of random series, whose relative top
-// gap is ~0.2 %, by ~40 (plain Lanczos from the start vector below, checked in FP64 on the CPU).
+// Lanczos steps (tridiagonal order) at most: enough for lambda_max of random-series Grams, whose
+// relative top gap is ~0.2 % (checked in FP64 on the CPU).
 constexpr int kLanczosMax = 64;
+constexpr size_t kLancSmemMax = 200 * 1024;  // s <= 6400
 
 struct alignas(8) GridBar {
     unsigned int word;  // bit 31 flips when the last CTA arrives; bits 0-30 count arrivals
     int err;            // read with `word` in one 8-byte load
-    unsigned int pad[2];
+    unsigned int pad[2];  // the Lanczos kernel: published steps, stop request
 };
 static_assert(sizeof(GridBar) <= kCoopBarrierBytes, "grid barrier exceeds its scratch header");
 
@@ -269,11 +269,6 @@ RECON_DEV void report_batch(const SweepBatch& bt, int v) {
         for (int b = 0; b < bt.n; ++b)
             if (bt.m[b].err_out) *bt.m[b].err_out = v;
 }
-
-// Failure status of a batched Lanczos launch (thread 0 of CTA 0, every matrix); on success each
-// matrix's CTA writes 0 after its multisection.
-struct LancBatch;
-RECON_DEV void report_lanc(const LancBatch& bt, int v);
 
 struct SweepSmem {
     double2 D[kTileT];            // D_K
@@ -641,268 +636,339 @@ __global__ void hdiag_kernel(const double2* __restrict__ H, int N1, int N2, int 
     if (lane == 0) dsum[warp] = acc;
 }
 
-// ---- Lanczos estimate of lambda_max(G), FP64, m steps, then multisection on the tridiagonal.
-// One matrix of a batched Lanczos launch (by value in the kernel parameters).
+// ---- lambda_max(G) by Lanczos, FP64, to convergence (at most kLanczosMax steps).
+//
+// One grid barrier per step. Every worker CTA holds the whole vectors q_k and q_{k-1} in shared
+// memory; a step forms this CTA's rows of w = G q_k (two warps a row, G from L2), crosses the
+// barrier, reads all of w and continues the recurrence for every element itself, so that nothing
+// but w crosses between CTAs. The recurrence is the unnormalised one,
+//   q_{k+1} = 2^-e_k (G q_k - alpha_k q_k - gamma_k q_{k-1}),  alpha_k = <q_k, G q_k> / n_k,
+//   n_k = <q_k, q_k>,  beta_{k-1}^2 = (n_k / n_{k-1}) 4^e_{k-1},  gamma_k = (n_k / n_{k-1}) 2^e_{k-1},
+// with powers of two e_k that keep n_k near 1 (exact): no square root, and both sums come from one
+// reduction after the barrier. CTA 0 publishes (alpha_k, beta_{k-1}^2).
+//
+// The last CTA takes no part in the barriers: it takes the largest eigenvalue of the tridiagonal as
+// published so far, again and again, and asks CTA 0 to end the iteration once it has not grown by
+// 1e-15 of itself over two checks in a row (at least four steps). lambda_max of Grams of image
+// series stands after ~14-18 steps, that of random series with a 0.2 % top gap after ~40-50; a fixed
+// 64 steps with two barriers each took 805 us at s = 243 (12.6 us a step) on every first iteration.
+// The bound of a step is latency: the barrier, the dependent FP64 chains (64 cycles an operation)
+// and the FP64 issue of the redundant vector work. s = 243 series: 805 -> 168 us
+// (recon_weight with its own eps 1098 -> 461 us).
 struct LancMat {
-    const double2* G;      // s x s column-major, Hermitian
-    double2 *u, *vprev;    // Lanczos vectors (s each)
-    double* part;          // 4 x grid partial sums (alpha, beta; ping-pong)
-    double* ab;            // alpha_k, beta_k
-    double* lmax_out;      // device scalar
-    int* err_out;          // status word (may be null)
-    int s, m;              // order, steps (<= kLanczosMax)
+    const double2* G;   // s x s column-major, Hermitian
+    double2* w;         // G q of a step, two buffers of s
+    double* ab;         // alpha_k, beta_{k-1}^2
+    int* dec;           // CTA 0's decision after a step (two slots): 1 = the last one
+    double* lmax_out;   // device scalar
+    int* err_out;       // status word (may be null)
+    int s, m;           // order, steps at most
 };
-struct LancBatch {
-    int n, m_max;
-    LancMat mt[kMaxHpdBatch];
-};
+constexpr unsigned int kLancFin = 0x40000000u;  // published step count: the iteration has ended
 
-RECON_DEV void report_lanc(const LancBatch& bt, int v) {
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-        for (int b = 0; b < bt.n; ++b)
-            if (bt.mt[b].err_out) *bt.mt[b].err_out = v;
+// floor(log2(v)) of a positive normal number, and 2^e.
+RECON_DEV int exponent_of(double v) { return (int)((__double_as_longlong(v) >> 52) & 0x7ff) - 1023; }
+RECON_DEV double pow2i(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+
+// Two sums over a warp in one tree: lane 0 returns the sum of a, lane 16 that of b (every FP64
+// instruction of a warp costs the SM's FP64 pipe the same, however many lanes it is for).
+RECON_DEV double warp_sum_pair(double a, double b, int lane) {
+    const bool hi = (lane & 16) != 0;
+    double v = hi ? b : a;
+    v += __shfl_xor_sync(0xffffffffu, hi ? a : b, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
-// Several matrices per launch, two grid barriers per step for all of them. Row i of matrix b goes
-// to global warp i mod (warps of the grid), as in a launch of that matrix alone, and every sum is
-// taken in the same order, so each matrix's lambda_max is bitwise the one its own launch gives.
-__global__ void __launch_bounds__(kLancThreads, 4)
-lanczos_kernel(LancBatch bt, GridBar* gb, CoopFault fault) {
-    __shared__ double red[kMaxHpdBatch][kLancThreads / 32];
-    __shared__ double2 ys[kMaxHpdBatch][kLancRows][kLancThreads / 32];  // G v of the warp's rows (lane 0)
-    __shared__ double s_beta[kMaxHpdBatch], s_ib[kMaxHpdBatch], s_alpha[kMaxHpdBatch];
-    __shared__ int s_m[kMaxHpdBatch];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nw = gridDim.x * (kLancThreads / 32);
-    const int gw = warp * gridDim.x + blockIdx.x;  // rows spread over every SM (FP64 unit per SM)
-    const int n = bt.n;
-    // deterministic start vector, unnormalised: u_i = 1 + 0.5 sin(i) + i 0.25 i cos(3 i) / s
-    for (int b = 0; b < n; ++b) {
-        const LancMat& L = bt.mt[b];
-        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < L.s; i += gridDim.x * blockDim.x) {
-            L.u[i] = make_double2(1.0 + 0.5 * sin((double)i), 0.25 * cos(3.0 * i) * i / L.s);
-            L.vprev[i] = make_double2(0.0, 0.0);
-        }
-    }
-    if (!grid_barrier(gb, fault)) return report_lanc(bt, 1);
-    for (int b = warp; b < n; b += kLancThreads / 32) {
-        const LancMat& L = bt.mt[b];
-        double acc = 0.0;
-        for (int i = lane; i < L.s; i += 32) acc += L.u[i].x * L.u[i].x + L.u[i].y * L.u[i].y;
-        acc = warp_sum(acc);
-        if (lane == 0) {
-            s_beta[b] = sqrt(acc);
-            s_ib[b] = rcp_nr(s_beta[b]);
-            s_m[b] = L.m;
-        }
-    }
-    __syncthreads();
-    for (int k = 0; k < bt.m_max; ++k) {
-        // v_k = u / beta_{k-1};  w = G v_k - alpha_k v_k - beta_{k-1} v_{k-1};  beta_k = |w|
-        bool any = false;
-        for (int b = 0; b < n; ++b) {
-            const LancMat& L = bt.mt[b];
-            const bool act = k < s_m[b];
-            any = any || act;
-            double ap = 0.0;
-            if (act) {
-                const double ib = s_ib[b];
-                int nrow = 0;
-                for (int i = gw; i < L.s && nrow < kLancRows; i += nw, ++nrow) {
-                    // row i of the Hermitian G is the conjugate of column i (contiguous)
-                    double2 acc = make_double2(0.0, 0.0);
-                    const double2* gcol = L.G + (size_t)i * L.s;
-                    int j = lane;
-                    for (; j + 32 * 3 < L.s; j += 32 * 4) {  // four loads of each in flight
-                        double2 g[4], uj[4];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            g[q] = gcol[j + 32 * q];
-                            uj[q] = L.u[j + 32 * q];
-                        }
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            acc.x = fma(g[q].x, uj[q].x, acc.x);
-                            acc.x = fma(g[q].y, uj[q].y, acc.x);
-                            acc.y = fma(g[q].x, uj[q].y, acc.y);
-                            acc.y = fma(-g[q].y, uj[q].x, acc.y);
-                        }
-                    }
-                    for (; j < L.s; j += 32) {
-                        const double2 g = gcol[j], uj = L.u[j];
-                        acc.x = fma(g.x, uj.x, acc.x);
-                        acc.x = fma(g.y, uj.y, acc.x);
-                        acc.y = fma(g.x, uj.y, acc.y);
-                        acc.y = fma(-g.y, uj.x, acc.y);
-                    }
-                    acc.x = warp_sum(acc.x) * ib;
-                    acc.y = warp_sum(acc.y) * ib;
-                    if (lane == 0) ys[b][nrow][warp] = acc;
-                    const double2 vi = make_double2(L.u[i].x * ib, L.u[i].y * ib);
-                    ap += vi.x * acc.x + vi.y * acc.y;
-                }
-            }
-            if (lane == 0) red[b][warp] = ap;
-        }
-        if (!any) break;
-        __syncthreads();
-        if ((int)threadIdx.x < n && k < s_m[threadIdx.x]) {
-            const int b = threadIdx.x;
-            double t = 0.0;
-            for (int w = 0; w < kLancThreads / 32; ++w) t += red[b][w];
-            bt.mt[b].part[(size_t)(k & 1) * 2 * gridDim.x + blockIdx.x] = t;
-        }
-        if (!grid_barrier(gb, fault)) return report_lanc(bt, 1);
-        for (int b = warp; b < n; b += kLancThreads / 32) {
-            if (k >= s_m[b]) continue;
-            const double* pa = bt.mt[b].part + (size_t)(k & 1) * 2 * gridDim.x;
-            const double v = warp_sum(lane_sum(pa, lane, (int)gridDim.x));
-            if (lane == 0) s_alpha[b] = v;
-        }
-        __syncthreads();
-        for (int b = 0; b < n; ++b) {
-            const LancMat& L = bt.mt[b];
-            double bp = 0.0;
-            if (k < s_m[b] && lane == 0) {
-                const double alpha = s_alpha[b], beta = s_beta[b], ib = s_ib[b];
-                int nrow = 0;
-                for (int i = gw; i < L.s && nrow < kLancRows; i += nw, ++nrow) {
-                    const double2 vi = make_double2(L.u[i].x * ib, L.u[i].y * ib);
-                    const double2 vp = L.vprev[i], yi = ys[b][nrow][warp];
-                    const double2 un = make_double2(yi.x - alpha * vi.x - beta * vp.x,
-                                                    yi.y - alpha * vi.y - beta * vp.y);
-                    bp += un.x * un.x + un.y * un.y;
-                    L.vprev[i] = vi;
-                    L.u[i] = un;
-                }
-            }
-            if (lane == 0) red[b][warp] = bp;
-        }
-        __syncthreads();
-        if ((int)threadIdx.x < n && k < s_m[threadIdx.x]) {
-            const int b = threadIdx.x;
-            double t = 0.0;
-            for (int w = 0; w < kLancThreads / 32; ++w) t += red[b][w];
-            bt.mt[b].part[(size_t)(k & 1) * 2 * gridDim.x + gridDim.x + blockIdx.x] = t;
-        }
-        if (!grid_barrier(gb, fault)) return report_lanc(bt, 1);
-        for (int b = warp; b < n; b += kLancThreads / 32) {
-            if (k >= s_m[b]) continue;
-            const double* pb = bt.mt[b].part + (size_t)(k & 1) * 2 * gridDim.x + gridDim.x;
-            const double b2 = warp_sum(lane_sum(pb, lane, (int)gridDim.x));
-            if (lane == 0) {
-                const double bnew = sqrt(b2);
-                if ((int)blockIdx.x == b) {  // the CTA that reads them for the multisection
-                    bt.mt[b].ab[2 * k] = s_alpha[b];
-                    bt.mt[b].ab[2 * k + 1] = bnew;
-                }
-                const double al = s_alpha[b];
-                s_beta[b] = bnew;
-                s_ib[b] = rcp_nr(bnew);
-                if (!(bnew > 1e-300 * fabs(al) + 1e-300)) s_m[b] = k + 1;
-            }
-        }
-        __syncthreads();
-    }
-    // matrix b's tridiagonal on CTA b
-    if ((int)blockIdx.x >= n) return;
-    const LancMat& L = bt.mt[blockIdx.x];
-    const double* ab = L.ab;
-    const int m = s_m[blockIdx.x];
-    __shared__ double sh_lo, sh_hi;
-    // Largest eigenvalue of the m x m tridiagonal (alpha_k, beta_k) by multisection with Sturm
-    // counts (one CTA per matrix): FP32 rounds over the whole block to 1e-4 relative (FP32 counts are exact
-    // for x farther than ~m eps32 |T| from an eigenvalue), then FP64 rounds on three warps. The
-    // FP64 count follows the characteristic polynomials p_k = (alpha_k - x) p_{k-1} -
-    // beta_{k-1}^2 p_{k-2} (the number of sign changes of p_0 .. p_m is the number of eigenvalues
-    // below x), rescaled by exact powers of two when the exponent drifts: two dependent FP64
-    // operations per step instead of a reciprocal.
-    __shared__ int best;
-    __shared__ float sa32[kLanczosMax], sb32[kLanczosMax];
-    __shared__ double sa64[kLanczosMax], sb64[kLanczosMax];
-    for (int k = threadIdx.x; k < m; k += blockDim.x) {
-        const double a = ab[2 * k], b2 = k > 0 ? ab[2 * k - 1] * ab[2 * k - 1] : 0.0;
-        sa64[k] = a;
-        sb64[k] = b2;
-        sa32[k] = (float)a;
-        sb32[k] = (float)b2;
-    }
+// Barrier of the worker CTAs 0 .. n-1 of a larger grid (as grid_barrier).
+RECON_DEV bool worker_barrier(GridBar* gb, const CoopFault& fault, unsigned int n) {
+    __shared__ int ok_s;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double lo = 1e300, hi = -1e300;
-        for (int k = 0; k < m; ++k) {
-            const double r = (k > 0 ? fabs(ab[2 * k - 1]) : 0.0) + (k + 1 < m ? fabs(ab[2 * k + 1]) : 0.0);
-            lo = fmin(lo, ab[2 * k] - r);
-            hi = fmax(hi, ab[2 * k] + r);
+        int ok = !(fault.withhold > 0 && (int)blockIdx.x == fault.withhold);
+        if (ok) {
+            __threadfence();
+            const unsigned int inc = blockIdx.x == 0 ? 0x80000000u - (n - 1u) : 1u;
+            const unsigned int old = atom_add_acq_rel(&gb->word, inc);
+            if ((((old + inc) ^ old) & 0x80000000u) == 0u) ok = barrier_wait(gb, old, fault);
+            else __threadfence();
         }
-        const double pad = 1e-6 * fmax(fabs(lo), fabs(hi));
-        sh_lo = lo - pad;
-        sh_hi = hi + pad;
+        ok_s = ok;
     }
     __syncthreads();
+    return ok_s != 0;
+}
+
+// Number of eigenvalues of the tridiagonal (a_k, b_k = beta_{k-1}^2) below x: the sign changes of its
+// characteristic polynomials p_k = (a_k - x) p_{k-1} - b_k p_{k-2}, rescaled by exact powers of two
+// when the exponent drifts (two dependent FP64 operations per step instead of a reciprocal).
+RECON_DEV int sturm_count(const double* a, const double* b, int m, double x) {
+    double p0 = 1.0, p1 = a[0] - x;
+    if (p1 == 0.0) p1 = -1e-300;
+    int cnt = p1 < 0.0;
+    for (int k = 1; k < m; ++k) {
+        double p2 = fma(-b[k], p0, (a[k] - x) * p1);
+        if (p2 == 0.0) p2 = p1 < 0.0 ? 1e-300 : -1e-300;  // a zero counts as a change
+        cnt += (p2 < 0.0) != (p1 < 0.0);
+        p0 = p1;
+        p1 = p2;
+        const int ex = max((int)((__double_as_longlong(p0) >> 52) & 0x7ff),
+                           (int)((__double_as_longlong(p1) >> 52) & 0x7ff));
+        if (ex > 1023 + 480 || ex < 1023 - 480) {  // keep the larger one near 1
+            const double sc = __longlong_as_double((long long)(2046 - ex) << 52);
+            p0 *= sc;
+            p1 *= sc;
+        }
+    }
+    return cnt;
+}
+
+// Largest eigenvalue of the m x m tridiagonal in shared memory, by the whole CTA (uniform control
+// flow): multisection with one sample per thread. Without an earlier value (prev <= 0) from the
+// Gershgorin bounds, in FP32 down to 1e-4 relative (FP32 counts are exact for x farther than
+// ~m eps32 |T| from an eigenvalue) and FP64 from there; with one, which the eigenvalue cannot lie
+// below, from samples prev (1 + 2^-51 .. 2^-1.5) spread over the exponents.
+RECON_DEV double tri_max(const double* a, const double* b, int m, double prev) {
+    __shared__ double sh_lo, sh_hi;
+    __shared__ int best;
+    const int t = threadIdx.x, nthr = blockDim.x;
+    __syncthreads();  // a, b; the results of an earlier call are read
+    if (t == 0) {
+        double lo = 1e300, hi = -1e300;
+        for (int k = 0; k < m; ++k) {
+            // FP32 square roots, rounded up: only the bounds of the search
+            const double r = 1.000001 * ((k > 0 ? (double)sqrtf((float)b[k]) : 0.0) +
+                                         (k + 1 < m ? (double)sqrtf((float)b[k + 1]) : 0.0));
+            lo = fmin(lo, a[k] - r);
+            hi = fmax(hi, a[k] + r);
+        }
+        const double pad = 1e-6 * fmax(fabs(lo), fabs(hi));
+        sh_lo = prev > 0.0 ? prev : lo - pad;
+        sh_hi = hi + pad;
+    }
+    if (t == 0) best = -1;
+    __syncthreads();
+    if (prev > 0.0) {
+        const double x = fma(prev, (double)exp2f(-51.f + 0.39f * (float)t), prev);
+        if (sturm_count(a, b, m, x) < m) atomicMax(&best, t);
+        __syncthreads();
+        const int bt = best;
+        if (bt < 0) return prev;  // within 2^-51 of it
+        __syncthreads();
+        if (t == bt) sh_lo = x;
+        if (t == bt + 1) sh_hi = fmin(sh_hi, x);
+    }
     for (int round = 0; round < 24; ++round) {
-        const bool fp32 = (sh_hi - sh_lo) > 1e-4 * fabs(sh_hi);
-        const int nthr = fp32 ? (int)blockDim.x : 96;
+        __syncthreads();
         const double lo = sh_lo, hi = sh_hi;
-        int cnt = m;
-        if ((int)threadIdx.x < nthr) {
-            const double x = lo + (hi - lo) * (threadIdx.x + 1) / (double)(nthr + 1);
-            cnt = 0;
-            if (fp32) {
-                const float xf = (float)x;
-                float d = 1.f;
-                for (int k = 0; k < m; ++k) {
-                    d = (sa32[k] - xf) - (k > 0 ? sb32[k] * __frcp_rn(d) : 0.f);
-                    if (d == 0.f) d = -1e-30f;
-                    if (d < 0.f) ++cnt;
-                }
-            } else {
-                double p0 = 1.0, p1 = sa64[0] - x;
-                if (p1 == 0.0) p1 = -1e-300;
-                cnt = p1 < 0.0;
-                for (int k = 1; k < m; ++k) {
-                    double p2 = fma(-sb64[k], p0, (sa64[k] - x) * p1);
-                    if (p2 == 0.0) p2 = p1 < 0.0 ? 1e-300 : -1e-300;  // a zero counts as a change
-                    cnt += (p2 < 0.0) != (p1 < 0.0);
-                    p0 = p1;
-                    p1 = p2;
-                    const int ex = max((int)((__double_as_longlong(p0) >> 52) & 0x7ff),
-                                       (int)((__double_as_longlong(p1) >> 52) & 0x7ff));
-                    if (ex > 1023 + 480 || ex < 1023 - 480) {  // keep the larger one near 1
-                        const double sc = __longlong_as_double((long long)(2046 - ex) << 52);
-                        p0 *= sc;
-                        p1 *= sc;
-                    }
-                }
+        if (hi - lo <= 2e-16 * fabs(hi)) break;
+        const bool fp32 = (hi - lo) > 1e-4 * fabs(hi);
+        const double x = lo + (hi - lo) * (t + 1) / (double)(nthr + 1);
+        int cnt = 0;
+        if (fp32) {
+            const float xf = (float)x;
+            float d = 1.f;
+            for (int k = 0; k < m; ++k) {
+                d = ((float)a[k] - xf) - (k > 0 ? (float)b[k] * __frcp_rn(d) : 0.f);
+                if (d == 0.f) d = -1e-30f;
+                if (d < 0.f) ++cnt;
             }
+        } else {
+            cnt = sturm_count(a, b, m, x);
         }
         // the largest eigenvalue lies above the largest sample x with cnt < m
-        if (threadIdx.x == 0) best = -1;
+        if (t == 0) best = -1;
         __syncthreads();
-        if ((int)threadIdx.x < nthr && cnt < m) atomicMax(&best, (int)threadIdx.x);
+        if (cnt < m) atomicMax(&best, t);
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if (t == 0) {
             const double step = (hi - lo) / (double)(nthr + 1);
             const double nlo = lo + step * (best + 1);
             // FP32 counts near the root may be off by rounding: keep one step of margin
             sh_lo = fp32 ? fmax(lo, nlo - step) : nlo;
             sh_hi = fp32 ? fmin(hi, nlo + 2 * step) : nlo + step;
         }
+    }
+    __syncthreads();
+    return 0.5 * (sh_lo + sh_hi);
+}
+
+// The checking CTA (see above). It alone writes lmax_out and the status word, and hands the two
+// words it shares with CTA 0 (gb->pad: published steps, stop request) back zeroed, as the host
+// leaves them when it zeroes the scratch header.
+RECON_DEV void lanczos_check(const LancMat& L, GridBar* gb, const CoopFault& fault) {
+    __shared__ double sa[kLanczosMax], sb[kLanczosMax];
+    __shared__ unsigned int sh_seen;
+    __shared__ int sh_ok, sh_bad;
+    unsigned int seen = 0;
+    int calm = 0;
+    double theta = 0.0;
+    for (;;) {
+        if (threadIdx.x == 0) {
+            const unsigned int next = calm >= 2 ? kLancFin : (seen ? seen + 2u : 6u);
+            sh_ok = flag_wait(&gb->pad[0], next < (unsigned int)L.m || calm >= 2 ? next : kLancFin, gb, fault);
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(sh_seen) : "l"(&gb->pad[0]) : "memory");
+            sh_bad = 0;
+        }
         __syncthreads();
-        if (sh_hi - sh_lo <= 2e-16 * fabs(sh_hi)) break;
+        if (!sh_ok) {
+            if (threadIdx.x == 0 && L.err_out) *L.err_out = 1;
+            return;
+        }
+        const bool fin = sh_seen >= kLancFin;
+        const int m = (int)(fin ? sh_seen - kLancFin : sh_seen);
+        if (calm < 2) {
+            for (int k = threadIdx.x; k < m; k += blockDim.x) {
+                sa[k] = __ldcg(L.ab + 2 * k);
+                sb[k] = __ldcg(L.ab + 2 * k + 1);
+                if (!isfinite(sa[k]) || !isfinite(sb[k])) sh_bad = 1;
+            }
+            __syncthreads();
+            // a matrix that is not finite: reported as such by the value
+            const double th = (m < 1 || sh_bad) ? __longlong_as_double(0x7ff8000000000000LL)
+                                                : tri_max(sa, sb, m, theta);
+            calm = theta > 0.0 && th <= theta * (1.0 + 1e-15) ? calm + 1 : 0;
+            theta = th;
+            seen = (unsigned int)m;
+        }
+        __syncthreads();
+        if (fin) break;
+        if (calm >= 2 && threadIdx.x == 0)
+            *reinterpret_cast<volatile unsigned int*>(&gb->pad[1]) = 1u;
     }
     if (threadIdx.x == 0) {
-        L.lmax_out[0] = 0.5 * (sh_lo + sh_hi);
+        gb->pad[0] = 0u;
+        gb->pad[1] = 0u;
+        L.lmax_out[0] = theta;
         if (L.err_out) *L.err_out = 0;
     }
 }
 
+__global__ void __launch_bounds__(kLancThreads, 4)
+lanczos_kernel(LancMat L, GridBar* gb, CoopFault fault) {
+    const unsigned int nwork = gridDim.x - 1;
+    if (blockIdx.x == nwork) return lanczos_check(L, gb, fault);
+    extern __shared__ double2 vs[];  // q_k, q_{k-1}
+    __shared__ double2 part[kLancThreads / 64][2];
+    __shared__ double red[2][kLancThreads / 32];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int half = warp >> 1, idx = tid & 63;  // two warps a row, two rows at a time
+    const int s = L.s;
+    double2 *q = vs, *p = vs + s;
+    // deterministic start vector (values of an integer hash: exact, and cheap on the FP64 pipe)
+    for (int i = tid; i < s; i += kLancThreads) {
+        const float h = (float)((i * 40503 + 12345) & 1023) / 512.f - 1.f;
+        const float g = (float)((i * 30011 + 777) & 1023) / 512.f - 1.f;
+        q[i] = make_double2(1.0f + 0.5f * h, 0.25f * g * (float)i / (float)s);
+        p[i] = make_double2(0.0, 0.0);
+    }
+    __syncthreads();
+    double rn_prev = 0.0;
+    int e_prev = 0, k = 0;
+    for (; k < L.m; ++k) {
+        unsigned int stop = 0;
+        if (blockIdx.x == 0 && tid == 0)  // in flight while the rows are formed
+            asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(stop) : "l"(&gb->pad[1]) : "memory");
+        double2* w = L.w + (size_t)(k & 1) * s;
+        for (int r0 = blockIdx.x; r0 < s; r0 += 2 * nwork) {
+            const int row = r0 + half * nwork;
+            // row i of the Hermitian G is the conjugate of column i (contiguous)
+            double2 acc = make_double2(0.0, 0.0);
+            if (row < s) {
+                const double2* gcol = L.G + (size_t)row * s;
+                int j = idx;
+                for (; j + 64 * 3 < s; j += 64 * 4) {  // four loads in flight
+                    double2 g[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) g[u] = __ldg(gcol + j + 64 * u);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const double2 v = q[j + 64 * u];
+                        acc.x = fma(g[u].x, v.x, acc.x);
+                        acc.x = fma(g[u].y, v.y, acc.x);
+                        acc.y = fma(g[u].x, v.y, acc.y);
+                        acc.y = fma(-g[u].y, v.x, acc.y);
+                    }
+                }
+                for (; j < s; j += 64) {
+                    const double2 g = __ldg(gcol + j), v = q[j];
+                    acc.x = fma(g.x, v.x, acc.x);
+                    acc.x = fma(g.y, v.y, acc.x);
+                    acc.y = fma(g.x, v.y, acc.y);
+                    acc.y = fma(-g.y, v.x, acc.y);
+                }
+            }
+            const double v = warp_sum_pair(acc.x, acc.y, lane);
+            if (lane == 0) part[half][warp & 1].x = v;
+            if (lane == 16) part[half][warp & 1].y = v;
+            __syncthreads();
+            if (idx == 0 && row < s) w[row] = zadd(part[half][0], part[half][1]);
+            if (r0 + 2 * (int)nwork < s) __syncthreads();
+        }
+        if (blockIdx.x == 0 && tid == 0) L.dec[k & 1] = (int)stop;
+        // (the buffers of step k are written again at step k + 2, after barrier k + 1, which every
+        // CTA reaches only once it has read those of step k)
+        if (!worker_barrier(gb, fault, nwork)) return;
+        const int last = __ldcg(L.dec + (k & 1));
+        // alpha and n_k in one reduction
+        double a = 0.0, n = 0.0;
+        for (int i = tid; i < s; i += kLancThreads) {
+            const double2 wi = __ldcg(w + i), qi = q[i];
+            a = fma(qi.x, wi.x, a);
+            a = fma(qi.y, wi.y, a);
+            n = fma(qi.x, qi.x, n);
+            n = fma(qi.y, qi.y, n);
+        }
+        const double v = warp_sum_pair(a, n, lane);
+        if (lane == 0) red[0][warp] = v;
+        if (lane == 16) red[1][warp] = v;
+        __syncthreads();
+        double t = red[(lane >> 2) & 1][lane & 3];
+        t += __shfl_xor_sync(0xffffffffu, t, 1);
+        t += __shfl_xor_sync(0xffffffffu, t, 2);
+        a = __shfl_sync(0xffffffffu, t, 0);
+        n = __shfl_sync(0xffffffffu, t, 4);
+        if (!(n > 0.0)) break;  // an exhausted Krylov space, or a value that is not finite
+        const double rn = rcp_nr(n);
+        const double alpha = a * rn, ratio = n * rn_prev;
+        const double b2 = ratio * pow2i(2 * e_prev), gamma = ratio * pow2i(e_prev);
+        if (blockIdx.x == 0 && tid == 0) {
+            L.ab[2 * k] = alpha;
+            L.ab[2 * k + 1] = b2;
+            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&gb->pad[0]),
+                         "r"((unsigned int)(k + 1)) : "memory");
+        }
+        if (last) {
+            ++k;
+            break;
+        }
+        // the next vector's norm near 1: beta changes little from step to step
+        int e = exponent_of(n) / 2 + (b2 > 0.0 ? exponent_of(b2) / 2 : alpha != 0.0 ? exponent_of(fabs(alpha)) : 0);
+        e = min(max(e, -400), 400);
+        const double sc = pow2i(-e);
+        for (int i = tid; i < s; i += kLancThreads) {
+            const double2 wi = __ldcg(w + i), qi = q[i], pi = p[i];
+            p[i] = make_double2(sc * fma(-gamma, pi.x, fma(-alpha, qi.x, wi.x)),
+                                sc * fma(-gamma, pi.y, fma(-alpha, qi.y, wi.y)));
+        }
+        double2* sw = q;
+        q = p;
+        p = sw;
+        rn_prev = rn;
+        e_prev = e;
+        __syncthreads();
+    }
+    if (blockIdx.x == 0 && tid == 0)
+        asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&gb->pad[0]),
+                     "r"(kLancFin + (unsigned int)k) : "memory");
+}
 
-int coop_grid(const void* kern, int threads, int* grid) {
+int coop_grid(const void* kern, int threads, size_t smem, int* grid) {
     int dev = 0, sms = 0, per = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return -1;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads, 0) != cudaSuccess) return -1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads, smem) != cudaSuccess) return -1;
     if (per < 1) return -1;
     *grid = sms;  // one CTA per SM
     return 0;
@@ -913,11 +979,12 @@ int tiles_per_side(int s) { return (s + kB - 1) / kB; }
 // Cooperative launch (all CTAs co-resident, required by the grid barriers) through
 // cudaLaunchKernelEx so that it can be captured into a CUDA graph.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_coop(void (*kern)(KArgs...), int grid, int threads, cudaStream_t st,
+cudaError_t launch_coop(void (*kern)(KArgs...), int grid, int threads, size_t smem, cudaStream_t st,
                         Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -940,16 +1007,15 @@ size_t hpd_scratch_bytes(const Dims& d) {
     return kCoopBarrierBytes + 2 * nlt * kTileT * sizeof(double2) + 7 * kTileT * sizeof(double2) + 1024;
 }
 
-size_t lanczos_scratch_bytes(const Dims& d, int grid_max) {
-    return kCoopBarrierBytes + 2 * (size_t)d.s() * sizeof(double2) + 4 * (size_t)grid_max * sizeof(double) +
-           2 * kLanczosMax * sizeof(double) + 1024;
+size_t lanczos_scratch_bytes(const Dims& d) {
+    return kCoopBarrierBytes + 2 * (size_t)d.s() * sizeof(double2) + 2 * kLanczosMax * sizeof(double) + 256;
 }
 
 cudaError_t launch_hpd_inverse_batch(const HpdJob* jobs, int n, void* barrier_scratch,
                                      cudaStream_t st, CoopFault fault) {
     if (n < 1 || n > kMaxHpdBatch || !barrier_scratch) return cudaErrorInvalidValue;
     int grid = 0;
-    if (coop_grid((const void*)hpd_sweep_kernel, kThreads, &grid) || grid < 2 * n + 1)
+    if (coop_grid((const void*)hpd_sweep_kernel, kThreads, 0, &grid) || grid < 2 * n + 1)
         return cudaErrorInvalidConfiguration;
     SweepBatch bt = {};
     bt.n = n;
@@ -981,7 +1047,7 @@ cudaError_t launch_hpd_inverse_batch(const HpdJob* jobs, int n, void* barrier_sc
     // every work item must fit the per-CTA item table
     if (sweep_items(nts, n, grid - 2 * n, -1, nullptr, 0) > kMaxItems) return cudaErrorInvalidValue;
     GridBar* gb = reinterpret_cast<GridBar*>(barrier_scratch);
-    return launch_coop(hpd_sweep_kernel, grid, kThreads, st, bt, gb, fault);
+    return launch_coop(hpd_sweep_kernel, grid, kThreads, 0, st, bt, gb, fault);
 }
 
 cudaError_t launch_hpd_inverse(const Dims& d, double2* G, const double* eps, void* scratch,
@@ -998,44 +1064,33 @@ cudaError_t launch_hdiag(const Dims& d, const double2* H, double2* dsum, cudaStr
     return cudaGetLastError();
 }
 
-cudaError_t launch_lanczos_batch(const LanczosJob* jobs, int n, void* barrier_scratch,
-                                 cudaStream_t st, CoopFault fault) {
-    if (n < 1 || n > kMaxHpdBatch || !barrier_scratch) return cudaErrorInvalidValue;
-    int grid = 0;
-    if (coop_grid((const void*)lanczos_kernel, kLancThreads, &grid) || grid < n)
-        return cudaErrorInvalidConfiguration;
-    const int nw = grid * (kLancThreads / 32);
-    LancBatch bt = {};
-    bt.n = n;
-    for (int b = 0; b < n; ++b) {
-        const int s = jobs[b].s;
-        // each warp holds at most kLancRows rows of a matrix
-        if (s < 1 || s > kLancRows * nw || !jobs[b].G || !jobs[b].scratch || !jobs[b].lmax)
-            return cudaErrorInvalidValue;
-        unsigned char* p = reinterpret_cast<unsigned char*>(jobs[b].scratch) + kCoopBarrierBytes;
-        LancMat& L = bt.mt[b];
-        L.G = jobs[b].G;
-        L.u = reinterpret_cast<double2*>(p);
-        p += (size_t)s * sizeof(double2);
-        L.vprev = reinterpret_cast<double2*>(p);
-        p += (size_t)s * sizeof(double2);
-        L.part = reinterpret_cast<double*>(p);
-        p += 4 * (size_t)grid * sizeof(double);
-        L.ab = reinterpret_cast<double*>(p);
-        L.lmax_out = jobs[b].lmax;
-        L.err_out = jobs[b].err_out;
-        L.s = s;
-        L.m = s < kLanczosMax ? s : kLanczosMax;
-        if (L.m > bt.m_max) bt.m_max = L.m;
-    }
-    GridBar* gb = reinterpret_cast<GridBar*>(barrier_scratch);
-    return launch_coop(lanczos_kernel, grid, kLancThreads, st, bt, gb, fault);
-}
-
-cudaError_t launch_lanczos_lmax(const Dims& d, const double2* G, void* scratch, double* lmax,
+cudaError_t launch_lanczos_lmax(int s, const double2* G, void* scratch, double* lmax,
                                 int* err_flag_out, cudaStream_t st, CoopFault fault) {
-    const LanczosJob job{G, scratch, lmax, err_flag_out, d.s()};
-    return launch_lanczos_batch(&job, 1, scratch, st, fault);
+    // every CTA holds two vectors in shared memory
+    const size_t smem = 2 * (size_t)s * sizeof(double2);
+    if (s < 1 || smem > kLancSmemMax || !G || !scratch || !lmax) return cudaErrorInvalidValue;
+    if (smem > 40 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(lanczos_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    int grid = 0;
+    if (coop_grid((const void*)lanczos_kernel, kLancThreads, smem, &grid) || grid < 2)
+        return cudaErrorInvalidConfiguration;
+    unsigned char* p = reinterpret_cast<unsigned char*>(scratch) + kCoopBarrierBytes;
+    LancMat L = {};
+    L.G = G;
+    L.w = reinterpret_cast<double2*>(p);
+    p += 2 * (size_t)s * sizeof(double2);
+    L.ab = reinterpret_cast<double*>(p);
+    p += 2 * kLanczosMax * sizeof(double);
+    L.dec = reinterpret_cast<int*>(p);
+    L.lmax_out = lmax;
+    L.err_out = err_flag_out;
+    L.s = s;
+    L.m = s < kLanczosMax ? s : kLanczosMax;
+    GridBar* gb = reinterpret_cast<GridBar*>(scratch);
+    return launch_coop(lanczos_kernel, grid, kLancThreads, smem, st, L, gb, fault);
 }
 
 }  // namespace recon

@@ -177,7 +177,7 @@ struct CoopFault {
     long long polls = 0;
 };
 size_t hpd_scratch_bytes(const Dims& d);
-size_t lanczos_scratch_bytes(const Dims& d, int grid_max);
+size_t lanczos_scratch_bytes(const Dims& d);
 // G (s x s, column-major, Hermitian) is replaced by H = (G + eps I)^-1. The kernel writes
 // *err_flag_out itself (device int, may be NULL): 0 when it completed, 1 when a grid barrier
 // gave up. The same holds for launch_lanczos_lmax.
@@ -198,21 +198,10 @@ cudaError_t launch_hpd_inverse_batch(const HpdJob* jobs, int n, void* barrier_sc
                                      cudaStream_t st, CoopFault fault = {});
 // d_ab[delta] (summed diagonals) from an explicit H
 cudaError_t launch_hdiag(const Dims& d, const double2* H, double2* dsum, cudaStream_t st);
-// *lmax = largest eigenvalue of G (Lanczos, FP64)
-cudaError_t launch_lanczos_lmax(const Dims& d, const double2* G, void* scratch, double* lmax,
+// *lmax = largest eigenvalue of the s x s matrix G (Lanczos, FP64), 1 <= s <= 6400; scratch:
+// lanczos_scratch_bytes of its s.
+cudaError_t launch_lanczos_lmax(int s, const double2* G, void* scratch, double* lmax,
                                 int* err_flag_out, cudaStream_t st, CoopFault fault = {});
-// Several matrices in one cooperative launch (two grid barriers per step serve all): job b writes
-// lambda_max of its G (s_b x s_b) to its *lmax, using its scratch (lanczos_scratch_bytes of its
-// s). Bitwise the value of launching the matrix alone.
-struct LanczosJob {
-    const double2* G;
-    void* scratch;
-    double* lmax;
-    int* err_out;
-    int s;
-};
-cudaError_t launch_lanczos_batch(const LanczosJob* jobs, int n, void* barrier_scratch,
-                                 cudaStream_t st, CoopFault fault = {});
 
 // ---- coils (Eq. measurement-ij with receiver sensitivities C_c; d.nc coils, coil-major) ----
 // Pass A: p = r (first) or r + beta p (as launch_row_fwd_pupdate); t[c] = row-FFT(C_c * p).

@@ -437,15 +437,12 @@ int get_work(recon_ctx* c, const Dims& d, int n_cg, int n_iter, bool vectors, bo
         if (rc) return rc;
         GET("eigwork", (size_t)(w->lwork < 1 ? 1 : w->lwork) * sizeof(double2), eigwork, double2*);
     } else {
-        int dev = 0, sms = 0;
-        RC_CUDA(cudaGetDevice(&dev));
-        RC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         // the grid barriers of the cooperative kernels start zeroed (see kCoopBarrierBytes)
         unsigned long gen0 = c->ws_gen;
         GET("hpd", recon::hpd_scratch_bytes(d), hpd, void*);
         if (c->ws_gen != gen0) RC_CUDA(cudaMemsetAsync(w->hpd, 0, recon::kCoopBarrierBytes, c->stream));
         gen0 = c->ws_gen;
-        GET("lanc", recon::lanczos_scratch_bytes(d, sms), lanc, void*);
+        GET("lanc", recon::lanczos_scratch_bytes(d), lanc, void*);
         if (c->ws_gen != gen0) RC_CUDA(cudaMemsetAsync(w->lanc, 0, recon::kCoopBarrierBytes, c->stream));
     }
 #undef GET
@@ -493,7 +490,7 @@ int weight_step(recon_ctx* c, const Dims& d, const Twiddles& tw, Work& w, double
         if (!eps_mode_set) {
             if (eps_first) {
                 ProfScope ps(c, RECON_PROF_LANCZOS);
-                RC_CUDA(recon::launch_lanczos_lmax(d, w.G, w.lanc, w.lmax, w.kerr + 2 * it + 1, c->stream,
+                RC_CUDA(recon::launch_lanczos_lmax(d.s(), w.G, w.lanc, w.lmax, w.kerr + 2 * it + 1, c->stream,
                                                    w.fault));
             }
             ProfScope ps(c, RECON_PROF_EPS);
@@ -931,15 +928,14 @@ int iter_gram(recon_ctx* c, Solve& sv) {
 }
 
 // The FP64 weight of a group of solves (p = 0 sweep path) in shared launches on the active
-// stream: at n = 0 one Lanczos launch for every lambda_max, then one eps launch and one sweep
+// stream: at n = 0 a Lanczos launch for each lambda_max, then one eps launch and one sweep
 // launch for all. The group leader's scratch holds the barriers of the shared launches.
 int group_weight(recon_ctx* c, Solve* grp, int cnt, int n) {
     if (n == 0) {
-        recon::LanczosJob jobs[recon::kMaxHpdBatch];
-        for (int b = 0; b < cnt; ++b)
-            jobs[b] = {grp[b].w.G, grp[b].w.lanc, grp[b].w.lmax, grp[b].w.kerr + 2 * n + 1, grp[b].d.s()};
         ProfScope ps(c, RECON_PROF_LANCZOS);
-        RC_CUDA(recon::launch_lanczos_batch(jobs, cnt, grp[0].w.lanc, c->stream, grp[0].w.fault));
+        for (int b = 0; b < cnt; ++b)
+            RC_CUDA(recon::launch_lanczos_lmax(grp[b].d.s(), grp[b].w.G, grp[b].w.lanc, grp[b].w.lmax,
+                                               grp[b].w.kerr + 2 * n + 1, c->stream, grp[b].w.fault));
     }
     {
         const double* lmax[recon::kMaxHpdBatch];
@@ -1274,7 +1270,7 @@ int direct_weight(recon_ctx* c, const Dims& d, Work& w, DirectWork& dw, double p
     } else {
         if (!eps_set) {
             if (first)
-                RC_CUDA(recon::launch_lanczos_lmax(d, w.G, w.lanc, w.lmax, w.kerr + 2 * it + 1, c->stream,
+                RC_CUDA(recon::launch_lanczos_lmax(d.s(), w.G, w.lanc, w.lmax, w.kerr + 2 * it + 1, c->stream,
                                                    w.fault));
             RC_CUDA(recon::launch_eps(w.lmax, w.eps, first, frac, gamma, c->stream));
         }
