@@ -29,58 +29,154 @@ constexpr int kThreads = 256;
 constexpr int kVoxThreads = 128;
 constexpr int kJacobiSweeps = 16;
 
-// Per-pixel HLR-Voxel weight. eps_mode: 0 = eps_r = eps_in[px] (one eps per pixel); 1 = no
-// weight: the largest lambda_max(G_r) over the pixels goes to *lmax_max (FP64 bits, atomic max;
-// zero it first); 2 = eps_r = eps_in[0] (one eps for every pixel). G_out (may be null):
-// [npix][M][M] complex128 row-major; lmax_out (may be null): [npix].
+// G_r[a][b] = sum_j conj(x_{j+M-1-a}) x_{j+M-1-b} (j < k), upper triangle in FP64, the diagonal real.
+// Pairs of the same frame distance d = b - a sum the same products conj(x_n) x_{n-d} over ranges of n
+// shifted by a, so each product of the frames that all of them share (M-1 <= n <= T-M) is formed once
+// and added at the end: about M T products a pixel instead of M (M + 1) / 2 per window, on a pipe
+// that issues one FP64 instruction per ~19 cycles and SM.
 template <int M>
+RECON_DEV void voxel_gram(const float2* __restrict__ x, int T, size_t npix, size_t px,
+                          double2 (&A)[M][M]) {
+    double2 core[M], w[M];  // w[m] = x_{n-m}
+#pragma unroll
+    for (int a = 0; a < M; ++a) {
+        core[a] = w[a] = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int b = a; b < M; ++b) A[a][b] = make_double2(0.0, 0.0);
+    }
+    for (int n = 0; n < T; ++n) {
+        const float2 v = x[(size_t)n * npix + px];
+#pragma unroll
+        for (int m = M - 1; m > 0; --m) w[m] = w[m - 1];
+        w[0] = make_double2(v.x, v.y);
+        const bool inner = n >= M - 1 && n <= T - M;
+#pragma unroll
+        for (int d = 0; d < M; ++d) {
+            if (inner) {
+                if (d == 0) core[0].x = fma(w[0].x, w[0].x, fma(w[0].y, w[0].y, core[0].x));
+                else core[d] = zfmacj2(w[d], w[0], core[d]);
+                continue;
+            }
+#pragma unroll
+            for (int a = 0; a + d < M; ++a)
+                if (n >= M - 1 - a && n <= T - 1 - a) A[a][a + d] = zfmacj2(w[d], w[0], A[a][a + d]);
+        }
+    }
+#pragma unroll
+    for (int a = 0; a < M; ++a) {
+#pragma unroll
+        for (int b = a; b < M; ++b) A[a][b] = zadd(A[a][b], core[b - a]);
+        A[a][a].y = 0.0;
+    }
+}
+
+// The HLR-Voxel weight for p = 0 where neither G_r nor its eigenvalues are asked for: H_r =
+// (G_r + eps)^-1 by a Hermitian sweep of the M x M matrix in registers (its upper triangle; M pivots
+// of a Hermitian positive-definite matrix, no pivoting), one pixel a thread. The eigendecomposition
+// below takes ~90 us for this at 128x128x12, M = 3, all of it FP64 issue; this 12.7 us.
+template <int M>
+__global__ void __launch_bounds__(kVoxThreads)
+voxel_inverse_kernel(const float2* __restrict__ x, int T, size_t npix,
+                     const double* __restrict__ eps_in, int eps_each, float2* __restrict__ S) {
+    for (size_t px = (size_t)blockIdx.x * blockDim.x + threadIdx.x; px < npix;
+         px += (size_t)gridDim.x * blockDim.x) {
+        double2 A[M][M];
+        voxel_gram<M>(x, T, npix, px, A);
+        const double eps = eps_in[eps_each ? px : 0];
+#pragma unroll
+        for (int a = 0; a < M; ++a) A[a][a].x += eps;
+        // sweep of pivot k: A_ij -= A_ik A_kj / A_kk, A_ik /= A_kk, A_kk = -1 / A_kk; all of them
+        // leave -A^-1
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+            const double inv = rcp_nr(A[k][k].x);
+            double2 c[M];  // A_ik / A_kk
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                if (i == k) continue;
+                const double2 v = i < k ? A[i][k] : zconj(A[k][i]);
+                c[i] = make_double2(v.x * inv, v.y * inv);
+            }
+#pragma unroll
+            for (int i = 0; i < M; ++i)
+#pragma unroll
+                for (int j = i; j < M; ++j) {
+                    if (i == k || j == k) continue;
+                    const double2 akj = j < k ? zconj(A[j][k]) : A[k][j];
+                    if (i == j) A[i][i].x = fma(-c[i].x, akj.x, fma(c[i].y, akj.y, A[i][i].x));
+                    else A[i][j] = zfms(c[i], akj, A[i][j]);
+                }
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                if (i < k) A[i][k] = c[i];
+                if (i > k) A[k][i] = zconj(c[i]);
+            }
+            A[k][k].x = -inv;
+        }
+        int e = 0;  // S_ab = H_ba = conj(H_ab), H = -A
+#pragma unroll
+        for (int a = 0; a < M; ++a)
+#pragma unroll
+            for (int b = a; b < M; ++b, ++e)
+                S[(size_t)e * npix + px] =
+                    make_float2((float)-A[a][b].x, a == b ? 0.f : (float)A[a][b].y);
+    }
+}
+
+// Per-pixel HLR-Voxel weight by the eigendecomposition. eps_mode: 0 = eps_r = eps_in[px] (one eps
+// per pixel); 1 = no weight: the largest lambda_max(G_r) over the pixels goes to *lmax_max (FP64 bits,
+// atomic max; zero it first); 2 = eps_r = eps_in[0] (one eps for every pixel). G_out (may be null):
+// [npix][M][M] complex128 row-major; lmax_out (may be null): [npix]. In mode 1 (kVec = false) a
+// pixel whose trace is no larger than the maximum so far cannot raise it and is left out, and no
+// vectors are formed.
+template <int M, bool kVec>
 __global__ void __launch_bounds__(kVoxThreads)
 voxel_weight_kernel(const float2* __restrict__ x, int T, size_t npix, double p,
                     const double* __restrict__ eps_in, unsigned long long* __restrict__ lmax_max,
                     int eps_mode, float2* __restrict__ S, double2* __restrict__ G_out,
                     double* __restrict__ lmax_out) {
-    const int k = T - M + 1;
     for (size_t px = (size_t)blockIdx.x * blockDim.x + threadIdx.x; px < npix;
          px += (size_t)gridDim.x * blockDim.x) {
-        // G_r[a][b] = sum_j conj(x_{j+M-1-a}) x_{j+M-1-b}, window w[m] = x_{j+M-1-m}
-        double2 A[M][M], w[M];
+        double2 A[M][M];
+        voxel_gram<M>(x, T, npix, px, A);
 #pragma unroll
         for (int a = 0; a < M; ++a)
 #pragma unroll
-            for (int b = 0; b < M; ++b) A[a][b] = make_double2(0.0, 0.0);
-#pragma unroll
-        for (int m = 1; m < M; ++m) {
-            const float2 v = x[(size_t)(M - 1 - m) * npix + px];
-            w[m] = make_double2(v.x, v.y);
-        }
-        for (int j = 0; j < k; ++j) {
-            const float2 v = x[(size_t)(j + M - 1) * npix + px];
-            w[0] = make_double2(v.x, v.y);
-#pragma unroll
-            for (int a = 0; a < M; ++a)
-#pragma unroll
-                for (int b = a; b < M; ++b) A[a][b] = zfmacj2(w[b], w[a], A[a][b]);
-#pragma unroll
-            for (int m = M - 1; m > 0; --m) w[m] = w[m - 1];
-        }
-#pragma unroll
-        for (int a = 0; a < M; ++a) {
-            A[a][a].y = 0.0;
-#pragma unroll
             for (int b = a + 1; b < M; ++b) A[b][a] = zconj(A[a][b]);
-        }
         if (G_out) {
 #pragma unroll
             for (int a = 0; a < M; ++a)
 #pragma unroll
                 for (int b = 0; b < M; ++b) G_out[(px * M + a) * M + b] = A[a][b];
         }
+        if constexpr (!kVec) {
+            // trace / M <= lambda_max <= trace (a margin for the rounding of both)
+            double tr = 0.0;
+#pragma unroll
+            for (int a = 0; a < M; ++a) tr += A[a][a].x;
+            const unsigned act = __activemask();
+            double lb = tr;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const double other = __shfl_xor_sync(act, lb, o);
+                if (((act >> ((threadIdx.x & 31) ^ o)) & 1u) && other > lb) lb = other;
+            }
+            lb *= (1.0 - 1e-12) / M;
+            unsigned long long old = 0;
+            const int leader = __ffs(act) - 1;
+            if ((int)(threadIdx.x & 31) == leader)
+                old = atomicMax(lmax_max, (unsigned long long)__double_as_longlong(fmax(lb, 0.0)));
+            const double cur = fmax(__longlong_as_double((long long)__shfl_sync(act, old, leader)), lb);
+            if (tr * (1.0 + 1e-12) < cur) continue;
+        }
         // cyclic Jacobi: A <- J^H A J with J = diag(1, conj(e)) x real rotation on (p, q)
-        double2 V[M][M];
+        double2 V[kVec ? M : 1][kVec ? M : 1];
+        if constexpr (kVec) {
 #pragma unroll
-        for (int a = 0; a < M; ++a)
+            for (int a = 0; a < M; ++a)
 #pragma unroll
-            for (int b = 0; b < M; ++b) V[a][b] = make_double2(a == b ? 1.0 : 0.0, 0.0);
+                for (int b = 0; b < M; ++b) V[a][b] = make_double2(a == b ? 1.0 : 0.0, 0.0);
+        }
         for (int sweep = 0; sweep < kJacobiSweeps; ++sweep) {
             double off = 0.0, dg = 0.0;
 #pragma unroll
@@ -107,9 +203,11 @@ voxel_weight_kernel(const float2* __restrict__ x, int T, size_t npix, double p,
                         const double2 aip = A[i][pp], aiq = zmul(ec, A[i][qq]);
                         A[i][pp] = make_double2(c * aip.x - s * aiq.x, c * aip.y - s * aiq.y);
                         A[i][qq] = make_double2(s * aip.x + c * aiq.x, s * aip.y + c * aiq.y);
-                        const double2 vip = V[i][pp], viq = zmul(ec, V[i][qq]);
-                        V[i][pp] = make_double2(c * vip.x - s * viq.x, c * vip.y - s * viq.y);
-                        V[i][qq] = make_double2(s * vip.x + c * viq.x, s * vip.y + c * viq.y);
+                        if constexpr (kVec) {
+                            const double2 vip = V[i][pp], viq = zmul(ec, V[i][qq]);
+                            V[i][pp] = make_double2(c * vip.x - s * viq.x, c * vip.y - s * viq.y);
+                            V[i][qq] = make_double2(s * vip.x + c * viq.x, s * vip.y + c * viq.y);
+                        }
                     }
 #pragma unroll
                     for (int j = 0; j < M; ++j) {
@@ -127,12 +225,11 @@ voxel_weight_kernel(const float2* __restrict__ x, int T, size_t npix, double p,
 #pragma unroll
         for (int a = 1; a < M; ++a) lmax = fmax(lmax, A[a][a].x);
         if (lmax_out) lmax_out[px] = lmax;
-        if (eps_mode == 1) {
+        if constexpr (!kVec) {
             // lambda_max >= 0 (PSD Gram): the bit patterns of non-negative doubles order as the
             // values do
             atomicMax(lmax_max, (unsigned long long)__double_as_longlong(fmax(lmax, 0.0)));
-            continue;
-        }
+        } else {
         const double eps = eps_mode == 0 ? eps_in[px] : eps_in[0];
         double alpha[M];
 #pragma unroll
@@ -155,6 +252,7 @@ voxel_weight_kernel(const float2* __restrict__ x, int T, size_t npix, double p,
                 }
                 S[(size_t)e * npix + px] = make_float2((float)h.x, (float)h.y);
             }
+        }
     }
 }
 
@@ -382,10 +480,19 @@ cudaError_t launch_voxel_weight(const Dims& d, const float2* x, double p, const 
     const int grid = (int)((npix + kVoxThreads - 1) / kVoxThreads) < g
                          ? (int)((npix + kVoxThreads - 1) / kVoxThreads) : g;
     unsigned long long* mx = reinterpret_cast<unsigned long long*>(lmax_max);
+    // the inverse alone where it is all that is wanted (p = 0; any number of frames and taps)
+    const bool inverse = eps_mode != 1 && p == 0.0 && !G_out && !lmax_out;
 #define CASE(MM)                                                                               \
     case MM:                                                                                   \
-        voxel_weight_kernel<MM><<<grid, kVoxThreads, 0, st>>>(x, d.T, npix, p, eps_in, mx,      \
-                                                              eps_mode, S, G_out, lmax_out);   \
+        if (inverse)                                                                           \
+            voxel_inverse_kernel<MM><<<grid, kVoxThreads, 0, st>>>(x, d.T, npix, eps_in,        \
+                                                                   eps_mode == 0, S);          \
+        else if (eps_mode == 1)                                                                \
+            voxel_weight_kernel<MM, false><<<grid, kVoxThreads, 0, st>>>(                      \
+                x, d.T, npix, p, eps_in, mx, eps_mode, S, G_out, nullptr);                   \
+        else                                                                                   \
+            voxel_weight_kernel<MM, true><<<grid, kVoxThreads, 0, st>>>(                       \
+                x, d.T, npix, p, eps_in, mx, eps_mode, S, G_out, lmax_out);                    \
         break;
     switch (d.M) {
         CASE(1) CASE(2) CASE(3) CASE(4) CASE(5) CASE(6)

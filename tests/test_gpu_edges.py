@@ -4,7 +4,7 @@ and largest of a range), against plain FP64 references."""
 import numpy as np
 import pytest
 
-from tests.gpu_util import to_dev
+from tests.gpu_util import assert_close, pairs_from_full, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -49,3 +49,84 @@ def test_lambda_max(R, filt, kind):
     assert abs(first - lam) <= (4 * s * 2.0 ** -53 + 1e-13) * lam
     for _ in range(3):  # the scratch is left ready for the next launch, and the value is the same
         assert recon.recon_weight(ctx.h, (8, 32, 32), filt, Gd, -1.0, 0.0, S) == first
+
+
+@pytest.mark.parametrize("M", [1, 2, 3, 4, 5, 6])
+def test_voxel_inverse(R, M):
+    """The p = 0 weight alone (the inverse without an eigendecomposition), from T = M (one window)
+    over T = 2 M - 1 (no frame that all pairs share) to many frames. FP64 inside at condition numbers
+    of about 20, so the result is the rounding of S to FP32: 2 x 2^-24."""
+    import torch
+    from oracle import variants as V
+    recon, ctx = R
+    rng = np.random.default_rng(M)
+    for T in sorted({M, 2 * M - 1, 2 * M, 13}):
+        x = (rng.standard_normal((T, 16, 32)) + 1j * rng.standard_normal((T, 16, 32))).astype(np.complex64)
+        x[:, 3, 5] = 0
+        G = V.voxel_grams(x.astype(np.complex128), M)
+        lmax = np.linalg.eigvalsh(G)[..., -1]
+        eps = 0.05 * lmax + 1e-6 * lmax.max()
+        ref = pairs_from_full(V.voxel_S(V.voxel_weights(G, eps, 0.0)))
+        S = torch.empty(ref.shape, dtype=torch.complex64, device="cuda")
+        recon.recon_voxel_weight(ctx.h, to_dev(x), M, to_dev(eps), 0.0, S)
+        got = S.cpu().numpy()
+        assert np.all(np.abs(got - ref) <= 2.0 ** -23 * np.abs(ref).max(axis=0))
+
+
+@pytest.mark.parametrize("first", [False, True])
+@pytest.mark.parametrize("T,P,Q,M", [(1, 16, 16, 1), (2, 16, 16, 2), (7, 32, 16, 3), (21, 64, 64, 2),
+                                     (6, 32, 32, 6), (13, 128, 64, 4), (16, 256, 256, 3),
+                                     (24, 192, 192, 1), (24, 16, 256, 5), (11, 512, 512, 2)])
+def test_residual_carry(R, T, P, Q, M, first):
+    """r + lam W_{S_old - S_new} x (no CG step), runs of 2, 4, 8 and 16 frames with remainders. Each
+    element is a sum of M^2 complex products and r: (4 M^2 + 4) roundings of 2^-24."""
+    import torch
+    recon, ctx = R
+    rng = np.random.default_rng(T * P + M)
+
+    def c(*shape):
+        return (rng.standard_normal(shape) + 1j * rng.standard_normal(shape)).astype(np.complex64)
+
+    npair, k, lam = M * (M + 1) // 2, T - M + 1, 0.37
+    x, r, So, Sn = c(T, P, Q), c(T, P, Q), c(npair, P, Q), c(npair, P, Q)
+    e = 0
+    full = np.zeros((M, M, P, Q), dtype=np.complex128)
+    for a in range(M):
+        for b in range(a, M):
+            for S in (So, Sn):
+                if a == b:
+                    S[e].imag = 0
+            d = -Sn[e].astype(np.complex128) + (0 if first else So[e])
+            full[a, b], full[b, a] = d, d.conj()
+            e += 1
+    ref = np.zeros((T, P, Q), dtype=np.complex128) if first else r.astype(np.complex128)
+    for a in range(M):
+        for b in range(M):
+            ref[M - 1 - a:M - 1 - a + k] += lam * full[a, b] * x[M - 1 - b:M - 1 - b + k]
+    rd = to_dev(r)
+    hist = recon.recon_cg(ctx.h, to_dev(np.ones((T, P, Q), np.uint8)), (3, 3, M),
+                          None if first else to_dev(So), to_dev(Sn), lam, to_dev(x), rd, 0)
+    got = rd.cpu().numpy()
+    assert_close(got, ref, (4 * M * M + 4) * 2.0 ** -24)
+    rr = float(np.sum(np.abs(got.astype(np.complex128)) ** 2))
+    assert abs(hist[0] - rr) <= 1e-6 * rr
+
+
+@pytest.mark.parametrize("T", [2, 8, 9, 16, 17, 31, 33, 64])
+def test_t2fit_frame_counts(R, T):
+    """Frame counts at the edges of the register variants, FP32 against the FP64 fit: the gate of the
+    other fit tests."""
+    import torch
+    from oracle import t2fit
+    recon, ctx = R
+    rng = np.random.default_rng(T)
+    times = [1.0 + 59.0 * n / max(T - 1, 1) for n in range(T)]
+    t2 = 20 + 100 * rng.random((32, 32))
+    x = np.exp(-np.array(times)[:, None, None] / t2) * (0.2 + rng.random((32, 32)))
+    x = (x + 0.005 * (rng.standard_normal(x.shape) + 1j * rng.standard_normal(x.shape))).astype(np.complex64)
+    out = torch.empty((32, 32), dtype=torch.float32, device="cuda")
+    recon.recon_t2fit(ctx.h, to_dev(x), times, out)
+    ref = t2fit.fit_t2(x.astype(np.complex128), times)
+    got = out.cpu().numpy().astype(np.float64)
+    assert np.array_equal(np.isnan(got), np.isnan(ref))
+    assert t2fit.t2_rel_l2(ref, got) < 1e-4
