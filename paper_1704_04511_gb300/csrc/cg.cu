@@ -464,22 +464,53 @@ __global__ void sum_partials_kernel(const double* __restrict__ parts, int n, dou
 }
 
 // Residual carry between IRLS iterations: r = (first ? r0 : r) + lam W_{dS} x with
-// dS = S_old - S_new (or -S_new when first); partial |r|^2. One thread per pixel, all frames.
+// dS = S_old - S_new (or -S_new when first); partial |r|^2.
 // r0 = A^H b - A^H A x0 = x0 - A^H A x0 for x0 = A^H b: zero for one coil and 0/1 masks (A A^H
 // is then a projection), x0 - aha_x when A^H A x0 is supplied (coils).
-template <int M>
-__global__ void __launch_bounds__(kThreads)
+// A work unit is one pixel a thread and a run of up to FC frames, whose x values and the M - 1 on
+// either side are held in registers (one read of each instead of M^2; the order of the sums is the
+// window sum's whatever FC). The kernel runs once per IRLS iteration and is bound by latency for
+// small series, by memory for large ones: FC trades the units in flight against the re-reading of
+// S and of the frames at a run's ends (resid_run below). 64x64x21, M = 2: 14.0 -> 7.9 us;
+// 256x256x16, M = 3: 15.4 -> 11.8; 128x128x64x12, M = 2: 82 -> 60 (one thread a pixel with all frames before).
+constexpr int kResThreads = 128;
+template <int M, int FC>
+__global__ void __launch_bounds__(kResThreads)
 resid_carry_kernel(float2* __restrict__ r, const float2* __restrict__ x,
                    const float2* __restrict__ aha_x, const float2* __restrict__ S_old,
                    const float2* __restrict__ S_new, float lam, int first, int T, int circ,
-                   size_t npix,
-                   double* __restrict__ parts, unsigned int* counter,
+                   size_t npix, int nrun, int run, double* __restrict__ parts, unsigned int* counter,
                    double* __restrict__ rr_out) {
-    __shared__ double red[kThreads / 32];
+    __shared__ double red[kResThreads / 32];
+    pdl_wait();
     const int k = circ ? T : T - M + 1;
+    const long long nunit = (long long)((npix + kResThreads - 1) / kResThreads) * nrun;
     float acc = 0.f, comp = 0.f;
-    for (size_t px = (size_t)blockIdx.x * blockDim.x + threadIdx.x; px < npix;
-         px += (size_t)gridDim.x * blockDim.x) {
+    // the runs of a pixel block are neighbouring units: its S and shared frames meet in L2
+    for (long long u = blockIdx.x; u < nunit; u += gridDim.x) {
+        const size_t px = (size_t)(u / nrun) * kResThreads + threadIdx.x;
+        const int f0 = (int)(u % nrun) * run, f1 = min(T, f0 + run);
+        if (px >= npix) continue;
+        float2 xw[FC + 2 * (M - 1)], rv[FC];  // x_{f0 - (M - 1) + i}, r_{f0 + i}
+#pragma unroll
+        for (int i = 0; i < FC + 2 * (M - 1); ++i) {
+            const int f = f0 - (M - 1) + i;
+            xw[i] = make_float2(0.f, 0.f);
+            if (f < f1 + M - 1 && (circ || (f >= 0 && f < T)))
+                xw[i] = x[(size_t)wrap_frame(f, T) * npix + px];
+        }
+#pragma unroll
+        for (int i = 0; i < FC; ++i) {
+            rv[i] = make_float2(0.f, 0.f);
+            if (f0 + i >= f1) continue;
+            const size_t g = (size_t)(f0 + i) * npix + px;
+            if (!first) {
+                rv[i] = r[g];
+            } else if (aha_x) {  // x0 - A^H A x0 (coils: A A^H is no projection)
+                const float2 av = aha_x[g];
+                rv[i] = make_float2(xw[i + M - 1].x - av.x, xw[i + M - 1].y - av.y);
+            }
+        }
         float2 s[M][M];
         load_S<M>(S_new, npix, px, s);
         if (first) {
@@ -495,32 +526,28 @@ resid_carry_kernel(float2* __restrict__ r, const float2* __restrict__ x,
 #pragma unroll
                 for (int b = 0; b < M; ++b) s[a][b] = csub(so[a][b], s[a][b]);
         }
-        for (int n = 0; n < T; ++n) {
+#pragma unroll
+        for (int i = 0; i < FC; ++i) {
+            const int n = f0 + i;
+            if (n >= f1) break;
             float2 w = make_float2(0.f, 0.f);
 #pragma unroll
             for (int a = 0; a < M; ++a) {
                 const int j = n - M + 1 + a;
                 if (!circ && (j < 0 || j >= k)) continue;  // circ: every window
 #pragma unroll
-                for (int b = 0; b < M; ++b)
-                    w = cfma(s[a][b], x[(size_t)wrap_frame(n + a - b, T) * npix + px], w);
+                for (int b = 0; b < M; ++b) w = cfma(s[a][b], xw[i + M - 1 + a - b], w);
             }
-            float2 rv = make_float2(0.f, 0.f);
-            if (!first) {
-                rv = r[(size_t)n * npix + px];
-            } else if (aha_x) {  // x0 - A^H A x0 (coils: A A^H is no projection)
-                const float2 xv = x[(size_t)n * npix + px], av = aha_x[(size_t)n * npix + px];
-                rv = make_float2(xv.x - av.x, xv.y - av.y);
-            }
-            rv.x = fmaf(lam, w.x, rv.x);
-            rv.y = fmaf(lam, w.y, rv.y);
-            r[(size_t)n * npix + px] = rv;
-            const float term = fmaf(rv.x, rv.x, rv.y * rv.y) - comp;
+            rv[i].x = fmaf(lam, w.x, rv[i].x);
+            rv[i].y = fmaf(lam, w.y, rv[i].y);
+            r[(size_t)n * npix + px] = rv[i];
+            const float term = fmaf(rv[i].x, rv[i].x, rv[i].y * rv[i].y) - comp;
             const float sum = acc + term;
             comp = (sum - acc) - term;
             acc = sum;
         }
     }
+    pdl_trigger();
     const double tot = block_sum_f_t0(acc, red);
     last_block_sum(tot, parts, counter, rr_out);
 }
@@ -771,23 +798,38 @@ cudaError_t launch_sum_partials(const Partials& in, double* out, cudaStream_t st
     return cudaGetLastError();
 }
 
+// Frames of a run of the residual carry: the longest of 16, 8, 4, 2 that leaves kResFill threads in
+// flight (about 20 warps an SM), 2 for the smallest series.
+constexpr long long kResFill = 100000;
+int resid_run(const Dims& d) {
+    int fc = 16;
+    while (fc > 2 && (long long)d.pixels() * ((d.T + fc - 1) / fc) < kResFill) fc /= 2;
+    return fc;
+}
+
 cudaError_t launch_resid_carry(const Dims& d, float2* r, const float2* x, const float2* S_old,
                                const float2* S_new, float lam, int first, const RedSlot& rs,
                                double* rr_out, cudaStream_t st, const float2* aha_x) {
-    const int g = pix_grid(d.pixels());
-#define CASE(MM)                                                                              \
-    case MM:                                                                                  \
-        resid_carry_kernel<MM><<<g, kThreads, 0, st>>>(r, x, aha_x, S_old, S_new, lam, first, \
-                                                       d.T, d.circ, d.pixels(), rs.parts,     \
-                                                       rs.counter,                            \
-                                                       rr_out);                               \
-        break;
+    const size_t npix = d.pixels();
+    const int fc = resid_run(d), nrun = (d.T + fc - 1) / fc, run = (d.T + nrun - 1) / nrun;
+    const long long nunit = (long long)((npix + kResThreads - 1) / kResThreads) * nrun;
+    const dim3 grid((unsigned)(nunit < kMaxParts ? nunit : kMaxParts));
+#define RUN(MM, FF)                                                                             \
+    return launch_pdl(resid_carry_kernel<MM, FF>, grid, dim3(kResThreads), 0, st, r, x, aha_x,  \
+                      S_old, S_new, lam, first, d.T, d.circ, npix, nrun, run, rs.parts,         \
+                      rs.counter, rr_out);
+#define CASE(MM)                       \
+    case MM:                           \
+        if (fc == 16) RUN(MM, 16)      \
+        if (fc == 8) RUN(MM, 8)        \
+        if (fc == 4) RUN(MM, 4)        \
+        RUN(MM, 2)
     switch (d.M) {
         CASE(1) CASE(2) CASE(3) CASE(4) CASE(5) CASE(6)
         default: return cudaErrorInvalidValue;
     }
 #undef CASE
-    return cudaGetLastError();
+#undef RUN
 }
 
 cudaError_t launch_coil_unimodular(const Dims& d, const float2* coils, unsigned int* dev,
