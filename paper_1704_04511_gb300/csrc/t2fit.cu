@@ -18,6 +18,7 @@ namespace recon {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kT2Threads = 128;  // small images spread over more SMs
 
 RECON_DEV float magnitude_rn(float2 v) {
     return __fsqrt_rn(__fadd_rn(__fmul_rn(v.x, v.x), __fmul_rn(v.y, v.y)));
@@ -36,15 +37,29 @@ frame0_max_kernel(const float2* __restrict__ x, size_t npix, unsigned int* __res
     if ((threadIdx.x & 31) == 0) atomicMax(amax, __float_as_uint(m));
 }
 
-__global__ void __launch_bounds__(kThreads)
+// One pixel a thread, its NT >= T samples and the echo times in registers, the loops over frames
+// unrolled without branches (a frame beyond T adds exact zeros): the exponentials of a step are then
+// independent instructions. (A loop over T with an array of the largest T and the times read from the
+// parameters ran one exponential after the other: 20 % issue.) A Gauss-Newton step is a function of
+// (A, R) alone: once a step returns values that it had before, the remaining steps go round the same
+// cycle, and only the steps left over modulo its length are run. The values are bitwise those of
+// running them all; most pixels stand after five steps of 20, a few per cent go round in the last
+// bits. 256x256x16, 20 steps: 31.7 -> 19 us.
+template <int NT>
+__global__ void __launch_bounds__(kT2Threads)
 t2fit_kernel(const float2* __restrict__ x, int T, size_t npix, T2Times tm, float frac,
              const unsigned int* __restrict__ amax, int n_gn, float* __restrict__ t2,
              float* __restrict__ amp) {
     const size_t px = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (px >= npix) return;
     const float thr = __fmul_rn(frac, __uint_as_float(amax[0]));
-    float y[kT2MaxT];
-    for (int n = 0; n < T; ++n) y[n] = magnitude_rn(x[(size_t)n * npix + px]);
+    float y[NT], tt[NT];
+#pragma unroll
+    for (int n = 0; n < NT; ++n) {
+        y[n] = n < T ? magnitude_rn(x[(size_t)n * npix + px]) : 0.f;
+        const float t = n < T ? tm.t[n] : 0.f;
+        asm volatile("mov.f32 %0, %1;" : "=f"(tt[n]) : "f"(t));  // stays in a register
+    }
     if (!(y[0] > thr)) {
         t2[px] = __int_as_float(0x7fc00000);  // NaN: not foreground
         if (amp) amp[px] = __int_as_float(0x7fc00000);
@@ -52,28 +67,36 @@ t2fit_kernel(const float2* __restrict__ x, int T, size_t npix, T2Times tm, float
     }
     constexpr float kRmin = 1e-4f;  // 1 / T2 >= 1e-4 per ms (T2 <= 1e4 ms)
     // log-linear initial guess: log y = log A - R t
-    float tbar = 0.f, lbar = 0.f;
-    for (int n = 0; n < T; ++n) {
-        tbar += tm.t[n];
-        lbar += logf(fmaxf(y[n], 1e-30f));
+    float tbar = 0.f, lbar = 0.f, ly[NT];
+#pragma unroll
+    for (int n = 0; n < NT; ++n) {
+        ly[n] = n < T ? logf(fmaxf(y[n], 1e-30f)) : 0.f;
+        tbar += tt[n];  // 0 beyond T
+        lbar += ly[n];
     }
     tbar /= T;
     lbar /= T;
     float sxy = 0.f, sxx = 0.f;
-    for (int n = 0; n < T; ++n) {
-        const float dt = tm.t[n] - tbar;
-        sxy = fmaf(dt, logf(fmaxf(y[n], 1e-30f)) - lbar, sxy);
+#pragma unroll
+    for (int n = 0; n < NT; ++n) {
+        const float dt = n < T ? tt[n] - tbar : 0.f;
+        sxy = fmaf(dt, ly[n] - lbar, sxy);
         sxx = fmaf(dt, dt, sxx);
     }
     float R = fmaxf(-sxy / sxx, kRmin);
     float A = expf(lbar + R * tbar);
+    // the two states before and one of 1, 2, 4, ... steps ago (cycles of one, two and any length)
+    float A1 = __int_as_float(0x7fc00000), R1 = A1, Ac = A1, Rc = A1;
+    int len = 1, power = 1;
     for (int it = 0; it < n_gn; ++it) {
+        const float A0 = A, R0 = R;
         float a11 = 0.f, a12 = 0.f, a22 = 0.f, g1 = 0.f, g2 = 0.f;
-        for (int n = 0; n < T; ++n) {
-            const float e = expf(-tm.t[n] * R);
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            const float e = n < T ? expf(-tt[n] * R) : 0.f;
             const float model = A * e;
             const float res = model - y[n];
-            const float jr = -tm.t[n] * model;
+            const float jr = -tt[n] * model;
             a11 = fmaf(e, e, a11);
             a12 = fmaf(e, jr, a12);
             a22 = fmaf(jr, jr, a22);
@@ -92,6 +115,24 @@ t2fit_kernel(const float2* __restrict__ x, int T, size_t npix, T2Times tm, float
                 R = fmaxf(R - s2 * (h2 - c * h1) * id, kRmin);
             }
         }
+        if (A == A0 && R == R0) break;
+        int cycle = 0;
+        if (A == A1 && R == R1) cycle = 2;
+        else if (A == Ac && R == Rc) cycle = len;
+        if (cycle) {
+            n_gn = it + 1 + (n_gn - 1 - it) % cycle;
+            A1 = Ac = __int_as_float(0x7fc00000);  // found: only the rest is run
+            continue;
+        }
+        A1 = A0;
+        R1 = R0;
+        if (len == power) {
+            Ac = A;
+            Rc = R;
+            power *= 2;
+            len = 0;
+        }
+        ++len;
     }
     t2[px] = 1.0f / R;
     if (amp) amp[px] = A;
@@ -109,9 +150,16 @@ cudaError_t launch_t2fit(const Dims& d, const float2* x, const T2Times& tm, floa
     frame0_max_kernel<<<g0, kThreads, 0, st>>>(x, npix, amax_scratch);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int g1 = (int)((npix + kThreads - 1) / kThreads);
-    t2fit_kernel<<<g1, kThreads, 0, st>>>(x, d.T, npix, tm, frac, amax_scratch, n_gn, t2, amp);
-    return cudaGetLastError();
+    const int g1 = (int)((npix + kT2Threads - 1) / kT2Threads);
+#define CASE(NT)                                                                                  \
+    if (d.T <= NT) {                                                                              \
+        t2fit_kernel<NT><<<g1, kT2Threads, 0, st>>>(x, d.T, npix, tm, frac, amax_scratch, n_gn,   \
+                                                    t2, amp);                                     \
+        return cudaGetLastError();                                                                \
+    }
+    CASE(4) CASE(8) CASE(12) CASE(16) CASE(20) CASE(24) CASE(32) CASE(64)
+#undef CASE
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace recon
