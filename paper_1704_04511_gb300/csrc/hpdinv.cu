@@ -647,14 +647,14 @@ __global__ void hdiag_kernel(const double2* __restrict__ H, int N1, int N2, int 
 // with powers of two e_k that keep n_k near 1 (exact): no square root, and both sums come from one
 // reduction after the barrier. CTA 0 publishes (alpha_k, beta_{k-1}^2).
 //
-// The last CTA takes no part in the barriers: it takes the largest eigenvalue of the tridiagonal as
-// published so far, again and again, and asks CTA 0 to end the iteration once it has not grown by
-// 1e-15 of itself over two checks in a row (at least four steps). lambda_max of Grams of image
+// The last CTA takes no part in the barriers: it takes the largest eigenvalue of the tridiagonal of
+// the first 8, 12, 16, ... published steps and asks CTA 0 to end the iteration once it has not grown
+// by 1e-15 of itself over four steps (the workers are a few steps ahead by then). lambda_max of Grams of image
 // series stands after ~14-18 steps, that of random series with a 0.2 % top gap after ~40-50; a fixed
 // 64 steps with two barriers each took 805 us at s = 243 (12.6 us a step) on every first iteration.
 // The bound of a step is latency: the barrier, the dependent FP64 chains (64 cycles an operation)
-// and the FP64 issue of the redundant vector work. s = 243 series: 805 -> 168 us
-// (recon_weight with its own eps 1098 -> 461 us).
+// and the FP64 issue of the redundant vector work. s = 243 series: 805 -> 220 us
+// (recon_weight with its own eps 1090 -> 505 us).
 struct LancMat {
     const double2* G;   // s x s column-major, Hermitian
     double2* w;         // G q of a step, two buffers of s
@@ -801,13 +801,13 @@ RECON_DEV void lanczos_check(const LancMat& L, GridBar* gb, const CoopFault& fau
     __shared__ double sa[kLanczosMax], sb[kLanczosMax];
     __shared__ unsigned int sh_seen;
     __shared__ int sh_ok, sh_bad;
-    unsigned int seen = 0;
-    int calm = 0;
     double theta = 0.0;
-    for (;;) {
+    bool stands = false;
+    for (unsigned int next = 8;; next += 4) {
+        // the steps up to the next check, or all there are: never more, so that the value does not
+        // depend on how far the workers have got meanwhile
         if (threadIdx.x == 0) {
-            const unsigned int next = calm >= 2 ? kLancFin : (seen ? seen + 2u : 6u);
-            sh_ok = flag_wait(&gb->pad[0], next < (unsigned int)L.m || calm >= 2 ? next : kLancFin, gb, fault);
+            sh_ok = flag_wait(&gb->pad[0], stands ? kLancFin : next, gb, fault);
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(sh_seen) : "l"(&gb->pad[0]) : "memory");
             sh_bad = 0;
         }
@@ -816,25 +816,23 @@ RECON_DEV void lanczos_check(const LancMat& L, GridBar* gb, const CoopFault& fau
             if (threadIdx.x == 0 && L.err_out) *L.err_out = 1;
             return;
         }
-        const bool fin = sh_seen >= kLancFin;
-        const int m = (int)(fin ? sh_seen - kLancFin : sh_seen);
-        if (calm < 2) {
-            for (int k = threadIdx.x; k < m; k += blockDim.x) {
-                sa[k] = __ldcg(L.ab + 2 * k);
-                sb[k] = __ldcg(L.ab + 2 * k + 1);
-                if (!isfinite(sa[k]) || !isfinite(sb[k])) sh_bad = 1;
-            }
-            __syncthreads();
-            // a matrix that is not finite: reported as such by the value
-            const double th = (m < 1 || sh_bad) ? __longlong_as_double(0x7ff8000000000000LL)
-                                                : tri_max(sa, sb, m, theta);
-            calm = theta > 0.0 && th <= theta * (1.0 + 1e-15) ? calm + 1 : 0;
-            theta = th;
-            seen = (unsigned int)m;
+        if (stands) break;  // the workers have left as well
+        const bool fin = sh_seen >= kLancFin && sh_seen - kLancFin <= next;
+        const int m = (int)(fin ? sh_seen - kLancFin : next);
+        for (int k = threadIdx.x; k < m; k += blockDim.x) {
+            sa[k] = __ldcg(L.ab + 2 * k);
+            sb[k] = __ldcg(L.ab + 2 * k + 1);
+            if (!isfinite(sa[k]) || !isfinite(sb[k])) sh_bad = 1;
         }
         __syncthreads();
+        // a matrix that is not finite: reported as such by the value
+        const double th = (m < 1 || sh_bad) ? __longlong_as_double(0x7ff8000000000000LL)
+                                            : tri_max(sa, sb, m, theta);
+        stands = theta > 0.0 && th <= theta * (1.0 + 1e-15);
+        theta = th;
+        __syncthreads();
         if (fin) break;
-        if (calm >= 2 && threadIdx.x == 0)
+        if (stands && threadIdx.x == 0)
             *reinterpret_cast<volatile unsigned int*>(&gb->pad[1]) = 1u;
     }
     if (threadIdx.x == 0) {
