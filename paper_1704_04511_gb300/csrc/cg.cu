@@ -17,6 +17,8 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kMaxM = 6;
+// Dynamic shared memory that needs no opt-in next to a kernel's static arrays (48 KB for both).
+constexpr size_t kDynSmemFree = 40 * 1024;
 constexpr int kMaxParts = 4096;  // partial-sum slots (largest grid of a reducing kernel)
 constexpr int kUpdVec = 2;       // float4 per thread per iteration in the update pass
 constexpr int kUpdThreads = 512;
@@ -467,88 +469,118 @@ __global__ void sum_partials_kernel(const double* __restrict__ parts, int n, dou
 // dS = S_old - S_new (or -S_new when first); partial |r|^2.
 // r0 = A^H b - A^H A x0 = x0 - A^H A x0 for x0 = A^H b: zero for one coil and 0/1 masks (A A^H
 // is then a projection), x0 - aha_x when A^H A x0 is supplied (coils).
-// A work unit is one pixel a thread and a run of up to FC frames, whose x values and the M - 1 on
-// either side are held in registers (one read of each instead of M^2; the order of the sums is the
-// window sum's whatever FC). The kernel runs once per IRLS iteration and is bound by latency for
-// small series, by memory for large ones: FC trades the units in flight against the re-reading of
-// S and of the frames at a run's ends (resid_run below). 64x64x21, M = 2: 14.0 -> 7.9 us;
-// 256x256x16, M = 3: 15.4 -> 11.8; 128x128x64x12, M = 2: 82 -> 60 (one thread a pixel with all frames before).
-constexpr int kResThreads = 128;
+// A warp takes 32 pixels and a run of up to FC frames, whose x values and the M - 1 on either side are
+// held in registers (one read of each instead of M^2; the order of the window sum does not depend on
+// the runs). The runs of a pixel group are warps of one CTA; the squares of a pixel meet in shared
+// memory and are added over the frames in order, so that |r|^2 does not depend on the runs either:
+// CG amplifies its last bits on the smallest series. The kernel runs once per IRLS iteration and is
+// bound by latency for small series, by memory for large ones: FC trades the warps in flight against
+// the re-reading of S and of the frames at a run's ends (resid_run below). 64x64x21, M = 2: 14.0 ->
+// 7.7 us; 256x256x16, M = 3: 15.4 -> 12.8; 128x128x64x12, M = 2: 82 -> 68 (one thread a
+// pixel with all frames before).
+constexpr int kResWarps = 8;  // most warps of a CTA
 template <int M, int FC>
-__global__ void __launch_bounds__(kResThreads)
+__global__ void __launch_bounds__(32 * kResWarps)
 resid_carry_kernel(float2* __restrict__ r, const float2* __restrict__ x,
                    const float2* __restrict__ aha_x, const float2* __restrict__ S_old,
                    const float2* __restrict__ S_new, float lam, int first, int T, int circ,
-                   size_t npix, int nrun, int run, double* __restrict__ parts, unsigned int* counter,
-                   double* __restrict__ rr_out) {
-    __shared__ double red[kResThreads / 32];
+                   size_t npix, int nrun, int run, int nwr, double* __restrict__ parts,
+                   unsigned int* counter, double* __restrict__ rr_out) {
+    extern __shared__ float terms[];  // [pixel group of the CTA][T][32] where a pixel has several runs
+    __shared__ double red[kResWarps];
     pdl_wait();
     const int k = circ ? T : T - M + 1;
-    const long long nunit = (long long)((npix + kResThreads - 1) / kResThreads) * nrun;
-    float acc = 0.f, comp = 0.f;
-    // the runs of a pixel block are neighbouring units: its S and shared frames meet in L2
-    for (long long u = blockIdx.x; u < nunit; u += gridDim.x) {
-        const size_t px = (size_t)(u / nrun) * kResThreads + threadIdx.x;
-        const int f0 = (int)(u % nrun) * run, f1 = min(T, f0 + run);
-        if (px >= npix) continue;
-        float2 xw[FC + 2 * (M - 1)], rv[FC];  // x_{f0 - (M - 1) + i}, r_{f0 + i}
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int ngrp = (blockDim.x >> 5) / nwr, grp = warp / nwr;  // pixel groups per CTA, nwr warps each
+    float* tg = terms + (size_t)grp * T * 32 + lane;
+    const size_t npg = npix / 32;  // P and Q are multiples of 16
+    double tot = 0.0;
+    for (size_t g0 = (size_t)blockIdx.x * ngrp; g0 < npg; g0 += (size_t)gridDim.x * ngrp) {
+        const size_t px = (g0 + grp) * 32 + lane;
+        const bool live = g0 + grp < npg;
+        float acc = 0.f, comp = 0.f;
+        for (int rn = warp % nwr; live && rn < nrun; rn += nwr) {
+            const int f0 = rn * run, f1 = min(T, f0 + run);
+            float2 xw[FC + 2 * (M - 1)], rv[FC];  // x_{f0 - (M - 1) + i}, r_{f0 + i}
 #pragma unroll
-        for (int i = 0; i < FC + 2 * (M - 1); ++i) {
-            const int f = f0 - (M - 1) + i;
-            xw[i] = make_float2(0.f, 0.f);
-            if (f < f1 + M - 1 && (circ || (f >= 0 && f < T)))
-                xw[i] = x[(size_t)wrap_frame(f, T) * npix + px];
-        }
+            for (int i = 0; i < FC + 2 * (M - 1); ++i) {
+                const int f = f0 - (M - 1) + i;
+                xw[i] = make_float2(0.f, 0.f);
+                if (f < f1 + M - 1 && (circ || (f >= 0 && f < T)))
+                    xw[i] = x[(size_t)wrap_frame(f, T) * npix + px];
+            }
 #pragma unroll
-        for (int i = 0; i < FC; ++i) {
-            rv[i] = make_float2(0.f, 0.f);
-            if (f0 + i >= f1) continue;
-            const size_t g = (size_t)(f0 + i) * npix + px;
-            if (!first) {
-                rv[i] = r[g];
-            } else if (aha_x) {  // x0 - A^H A x0 (coils: A A^H is no projection)
-                const float2 av = aha_x[g];
-                rv[i] = make_float2(xw[i + M - 1].x - av.x, xw[i + M - 1].y - av.y);
+            for (int i = 0; i < FC; ++i) {
+                rv[i] = make_float2(0.f, 0.f);
+                if (f0 + i >= f1) continue;
+                const size_t g = (size_t)(f0 + i) * npix + px;
+                if (!first) {
+                    rv[i] = r[g];
+                } else if (aha_x) {  // x0 - A^H A x0 (coils: A A^H is no projection)
+                    const float2 av = aha_x[g];
+                    rv[i] = make_float2(xw[i + M - 1].x - av.x, xw[i + M - 1].y - av.y);
+                }
+            }
+            float2 s[M][M];
+            load_S<M>(S_new, npix, px, s);
+            if (first) {
+#pragma unroll
+                for (int a = 0; a < M; ++a)
+#pragma unroll
+                    for (int b = 0; b < M; ++b) s[a][b] = make_float2(-s[a][b].x, -s[a][b].y);
+            } else {
+                float2 so[M][M];
+                load_S<M>(S_old, npix, px, so);
+#pragma unroll
+                for (int a = 0; a < M; ++a)
+#pragma unroll
+                    for (int b = 0; b < M; ++b) s[a][b] = csub(so[a][b], s[a][b]);
+            }
+#pragma unroll
+            for (int i = 0; i < FC; ++i) {
+                const int n = f0 + i;
+                if (n >= f1) break;
+                float2 w = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int a = 0; a < M; ++a) {
+                    const int j = n - M + 1 + a;
+                    if (!circ && (j < 0 || j >= k)) continue;  // circ: every window
+#pragma unroll
+                    for (int b = 0; b < M; ++b) w = cfma(s[a][b], xw[i + M - 1 + a - b], w);
+                }
+                rv[i].x = fmaf(lam, w.x, rv[i].x);
+                rv[i].y = fmaf(lam, w.y, rv[i].y);
+                r[(size_t)n * npix + px] = rv[i];
+                const float sq = fmaf(rv[i].x, rv[i].x, rv[i].y * rv[i].y);
+                if (nrun > 1) {
+                    tg[n * 32] = sq;
+                } else {
+                    const float term = sq - comp;
+                    const float sum = acc + term;
+                    comp = (sum - acc) - term;
+                    acc = sum;
+                }
             }
         }
-        float2 s[M][M];
-        load_S<M>(S_new, npix, px, s);
-        if (first) {
-#pragma unroll
-            for (int a = 0; a < M; ++a)
-#pragma unroll
-                for (int b = 0; b < M; ++b) s[a][b] = make_float2(-s[a][b].x, -s[a][b].y);
-        } else {
-            float2 so[M][M];
-            load_S<M>(S_old, npix, px, so);
-#pragma unroll
-            for (int a = 0; a < M; ++a)
-#pragma unroll
-                for (int b = 0; b < M; ++b) s[a][b] = csub(so[a][b], s[a][b]);
-        }
-#pragma unroll
-        for (int i = 0; i < FC; ++i) {
-            const int n = f0 + i;
-            if (n >= f1) break;
-            float2 w = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int a = 0; a < M; ++a) {
-                const int j = n - M + 1 + a;
-                if (!circ && (j < 0 || j >= k)) continue;  // circ: every window
-#pragma unroll
-                for (int b = 0; b < M; ++b) w = cfma(s[a][b], xw[i + M - 1 + a - b], w);
+        if (nrun > 1) {
+            __syncthreads();
+            for (int n = 0; warp % nwr == 0 && live && n < T; ++n) {
+                const float term = tg[n * 32] - comp;
+                const float sum = acc + term;
+                comp = (sum - acc) - term;
+                acc = sum;
             }
-            rv[i].x = fmaf(lam, w.x, rv[i].x);
-            rv[i].y = fmaf(lam, w.y, rv[i].y);
-            r[(size_t)n * npix + px] = rv[i];
-            const float term = fmaf(rv[i].x, rv[i].x, rv[i].y * rv[i].y) - comp;
-            const float sum = acc + term;
-            comp = (sum - acc) - term;
-            acc = sum;
+            __syncthreads();  // the terms are read
         }
+        tot += (double)warp_sum(acc);  // zero in the warps of later runs
     }
     pdl_trigger();
-    const double tot = block_sum_f_t0(acc, red);
+    if (lane == 0) red[warp] = tot;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        tot = 0.0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); w += nwr) tot += red[w];
+    }
     last_block_sum(tot, parts, counter, rr_out);
 }
 
@@ -620,7 +652,7 @@ cudaError_t launch_row_inv_w_NM(const Dims& d, const Twiddles& tw, float2* t, co
             ((size_t)3 * d.T * N + (size_t)d.M * (d.M + 1) / 2 * N + (size_t)t4 * kX128) * sizeof(float2);
         if (tpad * 8 <= 512 && smem128 <= 200 * 1024) {
             auto k = row_inv_w_128_kernel<M>;
-            if (smem128 > 48 * 1024) {
+            if (smem128 > kDynSmemFree) {
                 cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                      (int)smem128);
                 if (e != cudaSuccess) return e;
@@ -638,7 +670,7 @@ cudaError_t launch_row_inv_w_NM(const Dims& d, const Twiddles& tw, float2* t, co
         const size_t smem256 = ((size_t)d.T * N + (size_t)t2 * 16 * 17) * sizeof(float2);
         if (tpad * 16 <= 1024 && smem256 <= 200 * 1024) {
             auto k = row_inv_w_256_kernel<M>;
-            if (smem256 > 48 * 1024) {
+            if (smem256 > kDynSmemFree) {
                 cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                      (int)smem256);
                 if (e != cudaSuccess) return e;
@@ -652,7 +684,7 @@ cudaError_t launch_row_inv_w_NM(const Dims& d, const Twiddles& tw, float2* t, co
     }
     auto k = d.circ ? row_inv_w_kernel<N, M, true> : row_inv_w_kernel<N, M, false>;
     const size_t smem = ((size_t)3 * d.T * N + N) * sizeof(float2);
-    if (smem > 48 * 1024) {
+    if (smem > kDynSmemFree) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
@@ -698,7 +730,7 @@ cudaError_t launch_coil_inv_NM(const Dims& d, const Twiddles& tw, float2* t, con
     auto k = coil_row_inv_kernel<N, M, ADJ>;
     const size_t smem = ((size_t)4 * d.T * N + N) * sizeof(float2);
     if (smem > 220 * 1024) return cudaErrorInvalidValue;
-    if (smem > 48 * 1024) {
+    if (smem > kDynSmemFree) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
@@ -812,12 +844,23 @@ cudaError_t launch_resid_carry(const Dims& d, float2* r, const float2* x, const 
                                double* rr_out, cudaStream_t st, const float2* aha_x) {
     const size_t npix = d.pixels();
     const int fc = resid_run(d), nrun = (d.T + fc - 1) / fc, run = (d.T + nrun - 1) / nrun;
-    const long long nunit = (long long)((npix + kResThreads - 1) / kResThreads) * nrun;
-    const dim3 grid((unsigned)(nunit < kMaxParts ? nunit : kMaxParts));
-#define RUN(MM, FF)                                                                             \
-    return launch_pdl(resid_carry_kernel<MM, FF>, grid, dim3(kResThreads), 0, st, r, x, aha_x,  \
-                      S_old, S_new, lam, first, d.T, d.circ, npix, nrun, run, rs.parts,         \
-                      rs.counter, rr_out);
+    const int nwr = nrun < kResWarps ? nrun : kResWarps;   // warps of a pixel group
+    const int ngrp = nwr >= 4 ? 1 : 4 / nwr;               // at least about four warps a CTA
+    const size_t blocks = (npix / 32 + ngrp - 1) / ngrp;
+    const dim3 grid((unsigned)(blocks < (size_t)kMaxParts ? blocks : (size_t)kMaxParts));
+    const dim3 block(32 * nwr * ngrp);
+    const size_t smem = nrun > 1 ? (size_t)ngrp * d.T * 32 * sizeof(float) : 0;
+#define RUN(MM, FF)                                                                                 \
+    {                                                                                               \
+        auto kern = resid_carry_kernel<MM, FF>;                                                     \
+        if (smem > kDynSmemFree) {                                                                  \
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                                 (int)smem);                                        \
+            if (e != cudaSuccess) return e;                                                         \
+        }                                                                                           \
+        return launch_pdl(kern, grid, block, smem, st, r, x, aha_x, S_old, S_new, lam, first, d.T,  \
+                          d.circ, npix, nrun, run, nwr, rs.parts, rs.counter, rr_out);              \
+    }
 #define CASE(MM)                       \
     case MM:                           \
         if (fc == 16) RUN(MM, 16)      \
