@@ -87,7 +87,8 @@ void recon_destroy(recon_ctx* c);
 /* Description of the last error on this context (static storage; never NULL). */
 const char* recon_last_error(const recon_ctx* c);
 
-/* Device bytes of workspace recon_solve needs for this problem (the admission formula). */
+/* Device bytes of workspace recon_solve needs for this problem (the admission formula; what a context
+ * without a budget may keep on top of it is stated at RECON_OPT_GRAPHS). */
 size_t recon_bytes_needed(recon_dims d, recon_filter f, int kspace_bf16);
 
 /* Full reconstruction, Algorithm 1 (Sec. III): x0 = A^H b, then prm->irls iterations of
@@ -152,8 +153,11 @@ int recon_poll(recon_ctx* c, int ticket, int* done);
 
 /* Context options (value 0 = off, 1 = on unless stated):
  * RECON_OPT_GRAPHS: recon_solve and recon_solve_batch capture a whole solve (every launch of
- *   Algorithm 1) into a CUDA graph on first use and replay it while the shapes, parameters,
- *   buffer pointers and workspace stay the same (one graph per slot). Not used for the
+ *   Algorithm 1) into a CUDA graph on first use and replay it while the shapes, parameters and
+ *   workspace stay the same (one graph per slot). A context without a memory budget copies the masks
+ *   (and coil maps) into its workspace and the image out of it, 9 T P Q (+ 8 n_coils P Q) bytes a slot
+ *   where the device has them, so that the graph serves any buffers; with a budget the graph points
+ *   into the caller's buffers and is captured anew when these change. Not used for the
  *   eigensolver-library path or while launch classes are timed.
  * RECON_OPT_AUTOTUNE: on the first solve of each shape (P, Q, T, R, coils) the context times the
  *   column passes of the CG operator with tiles of 8, 16 and 32 columns (CUDA events on its own

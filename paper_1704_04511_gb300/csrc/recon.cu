@@ -238,8 +238,28 @@ void prof_collect(recon_ctx* c) {
     c->ev_used = 0;
 }
 
-// Device buffer `name` of at least `bytes` (contents undefined on growth).
-int ensure(recon_ctx* c, const char* name, size_t bytes, void** out) {
+// Free the staging copies of every slot (stage_solve), as when other buffers find no memory: the
+// graphs that point into them are stale then. Work queued on another slot may still use them.
+void release_staging(recon_ctx* c) {
+    cudaDeviceSynchronize();
+    auto drop = [c](std::map<std::string, Buf>& bufs, unsigned long& gen) {
+        for (const char* name : {"gx", "gm", "gc"}) {
+            auto it = bufs.find(name);
+            if (it == bufs.end()) continue;
+            if (it->second.ptr) cudaFree(it->second.ptr);
+            c->allocated -= it->second.bytes;
+            bufs.erase(it);
+            ++gen;
+        }
+    };
+    drop(c->bufs, c->ws_gen);
+    for (size_t i = 0; i < c->slots.size(); ++i)
+        if ((int)i != c->active) drop(c->slots[i].bufs, c->slots[i].ws_gen);
+}
+
+// Device buffer `name` of at least `bytes` (contents undefined on growth). staging: one that the
+// solve can do without.
+int ensure(recon_ctx* c, const char* name, size_t bytes, void** out, bool staging = false) {
     Buf& b = c->bufs[name];
     if (b.bytes >= bytes && b.ptr) {
         *out = b.ptr;
@@ -255,6 +275,11 @@ int ensure(recon_ctx* c, const char* name, size_t bytes, void** out) {
     if (c->budget && c->allocated + want > c->budget)
         return fail(c, RECON_ENOMEM, std::string("workspace budget exceeded allocating ") + name);
     cudaError_t e = cudaMalloc(&b.ptr, want);
+    if (e != cudaSuccess && !staging) {  // the staging copies make room for the rest
+        cudaGetLastError();
+        release_staging(c);
+        e = cudaMalloc(&b.ptr, want);
+    }
     if (e != cudaSuccess) {
         b = Buf{};
         cudaGetLastError();
@@ -805,10 +830,8 @@ int prepare_voxel(recon_ctx* c, Solve* sv) {
     return RECON_OK;
 }
 
-// Status reset and x0 = A^H b (Algorithm 1 initialisation). Enqueues only.
-int solve_begin(recon_ctx* c, Solve* sv) {
-    int rc = reset_status(c, sv->w);
-    if (rc) return rc;
+// x0 = A^H b (Algorithm 1 initialisation). Enqueues only.
+int solve_adjoint(recon_ctx* c, Solve* sv) {
     ProfScope ps(c, RECON_PROF_ADJOINT);
     if (sv->coils) {
         RC_CUDA(recon::launch_adjoint_coils_cols(sv->d, sv->tw, sv->kspace, sv->masks, sv->w.t,
@@ -819,6 +842,12 @@ int solve_begin(recon_ctx* c, Solve* sv) {
     RC_CUDA(recon::launch_adjoint(sv->d, sv->tw, sv->kspace, sv->prm->kspace_bf16, sv->masks,
                                   sv->w.t, sv->x, c->stream));
     return RECON_OK;
+}
+
+// Status reset and x0. Enqueues only.
+int solve_begin(recon_ctx* c, Solve* sv) {
+    int rc = reset_status(c, sv->w);
+    return rc ? rc : solve_adjoint(c, sv);
 }
 
 // IRLS iteration n of Algorithm 1: Gram, weight, residual carry, CG. Enqueues only.
@@ -872,11 +901,48 @@ recon_ctx::GraphKey graph_key(recon_ctx* c, const Solve& sv) {
     return k;
 }
 
+// Copies of the masks (and coil maps) and an iterate in the slot's workspace, for a graph that does
+// not depend on the caller's buffers: a program that reconstructs one scan after the other passes
+// other buffers each time, and capturing and instantiating a solve costs 2 to 3.5 ms of host time
+// (solves on changing buffers: 32x32x8, 20 x 10: 6.7 -> 4.1 ms; 256x256x16, 30 x 15: 24.8 ->
+// 19.8; four of these at 10 x 15: 22.2 -> 18.3), against three copies of 8 E + E bytes in
+// and out. Contexts with a budget keep to recon_bytes_needed and to the caller's buffers, and so
+// does a solve that finds no memory for the copies. False: not staged.
+bool stage_solve(recon_ctx* c, Solve* sv) {
+    if (c->budget) return false;
+    void *x = nullptr, *m = nullptr, *co = nullptr;
+    const size_t ne = sv->d.elems();
+    const std::string err = c->err;
+    int rc = ensure(c, "gx", ne * sizeof(float2), &x, true);
+    if (!rc) rc = ensure(c, "gm", ne, &m, true);
+    const size_t cb = sv->coils ? (size_t)sv->d.nc * sv->d.pixels() * sizeof(float2) : 0;
+    if (!rc && cb) rc = ensure(c, "gc", cb, &co, true);
+    if (rc) {
+        c->err = err;
+        release_staging(c);
+        return false;
+    }
+    Solve a = *sv;  // x0 straight from the caller's buffers
+    a.x = reinterpret_cast<float2*>(x);
+    rc = solve_adjoint(c, &a);
+    cudaError_t e = rc ? cudaErrorUnknown
+                       : cudaMemcpyAsync(m, sv->masks, ne, cudaMemcpyDeviceToDevice, c->stream);
+    if (e == cudaSuccess && cb)
+        e = cudaMemcpyAsync(co, sv->coils, cb, cudaMemcpyDeviceToDevice, c->stream);
+    if (e != cudaSuccess) return false;  // the unstaged solve meets the error again and reports it
+    sv->x = a.x;
+    sv->masks = reinterpret_cast<const uint8_t*>(m);
+    sv->coils = reinterpret_cast<const float2*>(co);
+    sv->kspace = nullptr;
+    return true;
+}
+
 // Enqueue a whole solve on the active slot's stream: as one replay of a captured CUDA graph
-// (captured on first use, cached per slot and keyed by shapes, parameters, buffers and the
-// workspace generation), or as direct launches when graphs are off, when the eigensolver
-// library path is used, or while launch classes are being timed.
-int solve_enqueue_all(recon_ctx* c, Solve& sv) {
+// (captured on first use, cached per slot and keyed by shapes, parameters, the workspace generation
+// and, where the solve is not staged, the caller's buffers), or as direct launches when graphs are
+// off, when the eigensolver library path is used, or while launch classes are being timed.
+int solve_enqueue_all(recon_ctx* c, const Solve& solve) {
+    Solve sv = solve;
     const recon_params* prm = sv.prm;
     const bool direct = !c->graphs || wants_eig(prm->p, prm->weight_method) || sv.w.fault.withhold;
     if (direct) {
@@ -884,6 +950,7 @@ int solve_enqueue_all(recon_ctx* c, Solve& sv) {
         for (int n = 0; n < prm->irls && !rc; ++n) rc = solve_iter(c, sv, n);
         return rc;
     }
+    const bool staged = stage_solve(c, &sv);
     const recon_ctx::GraphKey k = graph_key(c, sv);
     if (!c->gexec || std::memcmp(&k, &c->gkey, sizeof(k)) != 0) {
         if (c->gexec) {
@@ -894,7 +961,7 @@ int solve_enqueue_all(recon_ctx* c, Solve& sv) {
         c->gprof = c->prof ? new GraphProf() : nullptr;
         c->capturing = c->gprof;
         RC_CUDA(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeRelaxed));
-        int rc = solve_begin(c, &sv);
+        int rc = staged ? reset_status(c, sv.w) : solve_begin(c, &sv);
         for (int n = 0; n < prm->irls && !rc; ++n) rc = solve_iter(c, sv, n);
         cudaGraph_t g = nullptr;
         const cudaError_t ec = cudaStreamEndCapture(c->stream, &g);
@@ -914,6 +981,9 @@ int solve_enqueue_all(recon_ctx* c, Solve& sv) {
     }
     RC_CUDA(cudaGraphLaunch(c->gexec, c->stream));
     if (c->gprof) ++c->gprof->replays;
+    if (staged)
+        RC_CUDA(cudaMemcpyAsync(solve.x, sv.x, sv.d.elems() * sizeof(float2), cudaMemcpyDeviceToDevice,
+                                c->stream));
     return RECON_OK;
 }
 

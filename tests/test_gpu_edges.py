@@ -130,3 +130,72 @@ def test_t2fit_frame_counts(R, T):
     got = out.cpu().numpy().astype(np.float64)
     assert np.array_equal(np.isnan(got), np.isnan(ref))
     assert t2fit.t2_rel_l2(ref, got) < 1e-4
+
+
+@pytest.mark.parametrize("kind", ["solve", "bf16", "coils", "voxel", "volume"])
+def test_graph_serves_other_buffers(R, kind):
+    """One context over several scans in buffers of their own, with the masks of one changed in place
+    between calls and another shape in between: bitwise the results of a fresh context without
+    graphs and of one with a budget (whose graphs point into the caller's buffers)."""
+    import torch
+    recon, _ = R
+    rng = np.random.default_rng(7)
+
+    def scan(T, R_, P, Q):
+        shape = (T, R_, P, Q) if R_ else (T, P, Q)
+        n = 3 if kind == "coils" else 0
+        b = rng.standard_normal(((n,) if n else ()) + shape + (2,)).astype(np.float32)
+        b = torch.from_numpy(b).cuda()
+        b = b.to(torch.bfloat16) if kind == "bf16" else torch.view_as_complex(b).contiguous()
+        m = torch.from_numpy((rng.random(shape) < 0.4).astype(np.uint8)).cuda()
+        C = torch.from_numpy((rng.standard_normal((3, P, Q)) + 1j).astype(np.complex64)).cuda() if n else None
+        return b, m, C
+
+    def call(ctx, b, m, C):
+        out = torch.empty(tuple(m.shape), dtype=torch.complex64, device="cuda")
+        if kind == "coils":
+            recon.recon_solve_coils(ctx.h, b, m, C, (3, 3, 2), 0.1, 0.0, 2, 4, out)
+        elif kind == "voxel":
+            recon.recon_solve_variant(ctx.h, b, m, (1, 1, 3), 1e-2, 0.0, 2, 4, out, recon.RECON_VARIANT_HLR_VOXEL)
+        elif kind == "volume":
+            recon.recon_solve3(ctx.h, b, m, (3, 2, 2, 2), 1e-2, 0.0, 2, 4, out)
+        else:
+            recon.recon_solve(ctx.h, b, m, (3, 3, 2), 1e-2, 0.0, 3, 4, out)
+        return out
+
+    dims = [(5, 16, 32, 16)] * 3 if kind == "volume" else [(6, 0, 32, 64)] * 3
+    scans = [scan(*d) for d in dims] + [scan(4, 16 if kind == "volume" else 0, 16, 32)]
+    order = [0, 1, 2, 0, 3, 1, 0, 0]
+    with recon.Context(0) as kept, recon.Context(0) as plain, recon.Context(0, mem_budget_bytes=1 << 30) as tight:
+        recon.recon_set_option(plain.h, recon.RECON_OPT_GRAPHS, 0)
+        for step, i in enumerate(order):
+            b, m, C = scans[i]
+            if step == 6:
+                m.copy_(torch.flip(m, dims=(-1,)))
+                torch.cuda.synchronize()
+            got = call(kept, b, m, C)
+            ref = call(plain, b, m, C)
+            assert torch.equal(torch.view_as_real(got), torch.view_as_real(ref))
+            assert torch.equal(torch.view_as_real(call(tight, b, m, C)), torch.view_as_real(ref))
+
+
+@pytest.mark.parametrize("T", [10, 11, 12])
+@pytest.mark.parametrize("Q", [128, 256])
+def test_shared_memory_next_to_the_default_limit(Q, T):
+    """Frame counts whose dynamic shared memory alone is just under the 48 KB of a launch without
+    opt-in, and over it with the kernel's static arrays (256-point rows, T = 11), in a process state
+    where no larger series came before."""
+    import subprocess
+    import sys
+    code = ("import torch\n"
+            "from paper_1704_04511_gb300 import recon\n"
+            f"T, P, Q = {T}, 16, {Q}\n"
+            "c = recon.Context(0)\n"
+            "x = torch.randn((T, P, Q), dtype=torch.complex64, device='cuda')\n"
+            "m = torch.ones((T, P, Q), dtype=torch.uint8, device='cuda')\n"
+            "S = torch.zeros((1, P, Q), dtype=torch.complex64, device='cuda')\n"
+            "y = torch.empty_like(x)\n"
+            "torch.cuda.synchronize()\n"
+            "recon.recon_apply_normal(c.h, m, (3, 3, 1), S, 0.5, x, y)\n"
+            "assert (y - x).abs().max() < 1e-5 * x.abs().max()\n")
+    subprocess.run([sys.executable, "-c", code], check=True, timeout=120)
