@@ -23,7 +23,7 @@ LIB = os.path.join(LIBDIR, "librecon.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["fft.cu", "cg.cu", "gram.cu", "weight.cu", "hpdinv.cu", "t2fit.cu", "recon.cu",
            "gram_static.cu", "variants.cu"]
-HEADERS = ["common.cuh", "kernels.h", "regfft.cuh"]
+HEADERS = ["common.cuh", "kernels.h", "regfft.cuh", "stockham.cuh"]
 
 
 def _nvcc() -> str:

@@ -7,9 +7,14 @@
 //     (W x)_n(r) = sum_{a : 0 <= n-M+1+a < k} sum_b S_ab(r) x_{n+a-b}(r),
 // which is sum_j E_j^T S(r) E_j x(r) with (E_j x)(r)[m] = x_{j+M-1-m}(r). S is stored as its
 // upper triangle, pair (a <= b) at index a(2M-a+1)/2 + (b-a), layout [pair][P][Q] complex64.
+#include <map>
+#include <mutex>
+#include <tuple>
+
 #include "common.cuh"
 #include "kernels.h"
 #include "regfft.cuh"
+#include "stockham.cuh"
 
 namespace recon {
 
@@ -79,61 +84,216 @@ RECON_DEV float2 w_frame(const float2 (&s)[M][M], const float2 (&c)[2 * M - 1],
     return w;
 }
 
-// Pass C of a CG step. One CTA per image row r1 holds that row of every frame: it inverse-
-// transforms the k-space rows of t (giving A^H A p; the 1/(PQ) scale was applied with the mask),
-// adds lam W p from the p rows, writes q over t and emits the partial Re <p, q> of its row.
+// The W phase of pass C for frames [n0, n1) of one image row, by the whole CTA: res[n - n0][at(c)]
+// holds the transformed rows; q = res + lam W p goes to t, and Re (conj p) q of every element takes the
+// place of res.
+// A thread takes a column and a run of FC frames, whose p values and the M - 1 on either side it reads
+// straight from global memory into registers (each once per run; no copy of the p rows in shared
+// memory). kDiag: the diagonal form of w_frame where it applies.
+// The loads of a thread's first task (WLoads) are issued before the transform of the rows.
+template <int M>
+struct WLoads {
+    static constexpr int FC = M <= 4 ? 4 : 2;
+    float2 pw[FC + 2 * (M - 1)];    // p_{f0 - (M - 1) + i}
+    float2 s[M * (M + 1) / 2];      // upper triangle of S(r)
+};
 template <int N, int M, bool CIRC>
-__global__ void __launch_bounds__(kThreads)
-row_inv_w_kernel(float2* t, const float2* __restrict__ p, const float2* __restrict__ S,
-                 float lam, int T, int P, double* __restrict__ pq_parts,
-                 const float2* __restrict__ tw_g) {
-    extern __shared__ float2 sm[];
-    __shared__ double red[kThreads / 32];
-    float2* a = sm;
-    float2* b = a + (size_t)T * N;
-    float2* pt = b + (size_t)T * N;
-    float2* tw = pt + (size_t)T * N;
-    const size_t npix = (size_t)P * N;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = tw_g[i];
-    pdl_wait();
-    const int k = CIRC ? T : T - M + 1;
-    float acc = 0.f, comp = 0.f;  // Kahan-compensated per-thread partial of Re <p, q>
-    for (int r1 = blockIdx.x; r1 < P; r1 += gridDim.x) {
-    __syncthreads();  // the previous row's results are stored
-    for (int e = threadIdx.x; e < T * N; e += blockDim.x) {
-        const int n = e / N, c = e % N;
-        const size_t g = (size_t)n * npix + (size_t)r1 * N + c;
-        a[e] = t[g];
-        pt[e] = p[g];
+RECON_DEV void w_load(WLoads<M>& v, const float2* __restrict__ prow, const float2* __restrict__ Srow,
+                      int e, int T, int n0, int n1, size_t npix) {
+    constexpr int FC = WLoads<M>::FC;
+    const int c = e % N, f0 = n0 + (e / N) * FC, f1 = min(n1, f0 + FC);
+#pragma unroll
+    for (int i = 0; i < FC + 2 * (M - 1); ++i) {
+        const int f = f0 - (M - 1) + i;
+        v.pw[i] = make_float2(0.f, 0.f);
+        if (f0 < n1 && f < f1 + M - 1 && (CIRC || (f >= 0 && f < T)))
+            v.pw[i] = prow[(size_t)(CIRC ? wrap_frame(f, T) : f) * npix + c];
     }
-    __syncthreads();
-    float2* res = fft_smem<N, true, false>(a, b, T, N, 1, tw);
-    for (int c = threadIdx.x; c < N; c += blockDim.x) {
+#pragma unroll
+    for (int i = 0; i < M * (M + 1) / 2; ++i) v.s[i] = Srow[(size_t)i * npix + c];
+}
+
+template <int N, int M, bool CIRC, bool kDiag>
+RECON_DEV void w_phase(WLoads<M>& v, float2* __restrict__ trow, const float2* __restrict__ prow,
+                       const float2* __restrict__ Srow, float2* res, float lam, int T, int n0, int n1,
+                       size_t npix) {
+    using F = RegFft<N>;
+    constexpr int FC = WLoads<M>::FC;
+    const int k = CIRC ? T : T - M + 1;
+    const int nrun = (n1 - n0 + FC - 1) / FC;
+    for (int e = threadIdx.x; e < N * nrun; e += blockDim.x) {
+        if (e != (int)threadIdx.x) w_load<N, M, CIRC>(v, prow, Srow, e, T, n0, n1, npix);
+        const int c = e % N, f0 = n0 + (e / N) * FC, f1 = min(n1, f0 + FC);
         float2 s[M][M];
-        load_S<M>(S, npix, (size_t)r1 * N + c, s);
+#pragma unroll
+        for (int a = 0; a < M; ++a)
+#pragma unroll
+            for (int b = a; b < M; ++b) {
+                s[a][b] = v.s[a * (2 * M - a + 1) / 2 + (b - a)];
+                s[b][a] = cconj(s[a][b]);
+            }
         float2 cs[2 * M - 1];
-        s_diagonals<M>(s, cs);
-        for (int n = 0; n < T; ++n) {
-            const float2 w = w_frame<M, CIRC>(s, cs, pt + c, N, n, T, k);
-            float2 q = res[n * N + c];
+        if constexpr (kDiag) s_diagonals<M>(s, cs);
+#pragma unroll
+        for (int i = 0; i < FC; ++i) {
+            const int n = f0 + i;
+            if (n >= f1) break;
+            float2 w = make_float2(0.f, 0.f);
+            if (kDiag && (CIRC || (M >= 3 && M <= 5 && n >= M - 1 && n < k))) {
+#pragma unroll
+                for (int d = 0; d < 2 * M - 1; ++d) w = cfma(cs[d], v.pw[i + d], w);
+            } else {
+#pragma unroll
+                for (int a = 0; a < M; ++a) {
+                    const int j = n - M + 1 + a;
+                    if (j < 0 || j >= k) continue;
+#pragma unroll
+                    for (int b = 0; b < M; ++b) w = cfma(s[a][b], v.pw[i + M - 1 + a - b], w);
+                }
+            }
+            float2* rp = res + (size_t)(n - n0) * F::kBuf + F::at(c);
+            float2 q = *rp;
             q.x = fmaf(lam, w.x, q.x);
             q.y = fmaf(lam, w.y, q.y);
-            res[n * N + c] = q;
-            const float2 pv = pt[n * N + c];
-            const float term = fmaf(pv.x, q.x, pv.y * q.y) - comp;
-            const float sum = acc + term;
-            comp = (sum - acc) - term;
-            acc = sum;
+            trow[(size_t)n * npix + c] = q;
+            const float2 pv = v.pw[i + M - 1];
+            rp->x = fmaf(pv.x, q.x, pv.y * q.y);
         }
     }
-    __syncthreads();  // every column of q written
-    if (r1 + (int)gridDim.x >= P) pdl_trigger();
-    for (int e = threadIdx.x; e < T * N; e += blockDim.x) {
-        const int n = e / N, c = e % N;
-        t[(size_t)n * npix + (size_t)r1 * N + c] = res[e];
+}
+
+// The terms that w_phase left, added per column over the frames in order (Kahan), and over the columns
+// by FP32 warp trees: a warp's sum in its lane 0, FP64, zero elsewhere. Columns c and c + kThreads share
+// an accumulator, so that the sum is that of a CTA of kThreads threads, one column each, whatever the
+// launch shape (CG amplifies the last bits of Re <p, q> on the smallest series).
+template <int N>
+RECON_DEV double w_terms(const float2* res, int T) {
+    using F = RegFft<N>;
+    const int nc = N < kThreads ? N : kThreads;
+    double tot = 0.0;
+    for (int c0 = 0; c0 < nc; c0 += blockDim.x) {
+        float acc = 0.f, comp = 0.f;
+        if (c0 + (int)threadIdx.x < nc) {
+            for (int c = c0 + threadIdx.x; c < N; c += kThreads)
+                for (int n = 0; n < T; ++n) {
+                    const float term = res[(size_t)n * F::kBuf + F::at(c)].x - comp;
+                    const float sum = acc + term;
+                    comp = (sum - acc) - term;
+                    acc = sum;
+                }
+        }
+        tot += (double)warp_sum(acc);
     }
+    return tot;
+}
+
+// Sum over the CTA's warps of a value held by every lane 0 (thread 0 gets it).
+RECON_DEV double warps_sum_t0(double v, double* red) {
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double t = 0.0;
+    if (threadIdx.x < 32) {
+        t = threadIdx.x < blockDim.x / 32 ? red[threadIdx.x] : 0.0;
+        t = warp_sum(t);
     }
-    const double tot = block_sum_f_t0(acc, red);
+    return t;
+}
+
+// Launch shape of the row passes that hold every frame of an image row: the frames in `passes` equal
+// parts of at most inv_threads / (N / 8) sequences, whole warps; `bufs` exchange buffers.
+template <int N>
+__host__ __device__ constexpr int inv_threads() { return N == 192 ? 384 : 512; }
+struct InvShape {
+    int passes, per, threads, bufs;
+};
+template <int N>
+InvShape inv_shape(int T) {
+    constexpr int L = RegFft<N>::kLanes;
+    InvShape v;
+    v.passes = (T * L + inv_threads<N>() - 1) / inv_threads<N>();
+    v.per = (T + v.passes - 1) / v.passes;
+    v.threads = (v.per * L + 31) / 32 * 32;
+    if (v.threads < 64) v.threads = 64;
+    v.bufs = (v.passes - 1) * v.per + (v.threads + L - 1) / L;
+    return v;
+}
+
+// Pass C of a CG step. A CTA takes a run of `per` frames of an image row r1 (W reads the neighbouring
+// frames' p from global memory, so the runs are independent), N / 8 threads per frame: it
+// inverse-transforms the k-space rows of t (giving A^H A p; the 1/(PQ) scale was applied with the mask;
+// elements in registers, exchange buffers that then hold the transformed rows), adds lam W p, writes q
+// over t and emits a partial of Re <p, q>. Rows of up to 32 elements keep all their frames in one CTA
+// and with it the order of that sum (see w_terms). 64x64x21 7.8 -> 4.4 us per launch, 192x192x24
+// 17.4 -> 9.6, 512x512x16 66.6 -> 32.3, against one CTA per row with passes over shared memory and
+// three copies of the row's frames there.
+constexpr int kRunThreads = 256;   // most threads of a CTA (512 for rows of up to 32 elements)
+constexpr int kRunUnits = 608;     // units wanted: four CTAs an SM
+template <int N>
+__host__ __device__ constexpr int run_threads() { return N <= 32 ? 512 : kRunThreads; }
+struct RunShape {
+    int nrun, per, threads, bufs;
+};
+template <int N>
+RunShape run_shape(int T, int rows) {
+    constexpr int L = RegFft<N>::kLanes;
+    RunShape v;
+    int n = (T * L + run_threads<N>() - 1) / run_threads<N>();
+    if (N > 32) {  // more, shorter runs (of four frames at least) until the units fill the chip
+        // (rounded down: a few units more than fit at once would take a second round of their own)
+        const int fill = kRunUnits / rows, most = (T + 3) / 4;
+        if (n < fill) n = fill < most ? fill : (n > most ? n : most);
+    }
+    v.per = (T + n - 1) / n;
+    v.nrun = (T + v.per - 1) / v.per;
+    v.threads = (v.per * L + 31) / 32 * 32;
+    if (v.threads < 64) v.threads = 64;
+    v.bufs = (v.threads + L - 1) / L;
+    return v;
+}
+
+template <int N, int M, bool CIRC>
+__global__ void __launch_bounds__(run_threads<N>(), N <= 32 || M > 4 ? 1 : 3)
+row_inv_w_kernel(float2* t, const float2* __restrict__ p, const float2* __restrict__ S,
+                 float lam, int T, int P, int nrun, int per, double* __restrict__ pq_parts,
+                 const float2* __restrict__ tw_g) {
+    using F = RegFft<N>;
+    extern __shared__ float2 sm[];
+    __shared__ double red[16];
+    float2* tw = sm;
+    float2* res = sm + N;
+    const size_t npix = (size_t)P * N;
+    for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = tw_g[i];
+    const int fl = threadIdx.x / F::kLanes, i = threadIdx.x % F::kLanes;
+    float2* sx = res + fl * F::kBuf;
+    pdl_wait();
+    double tot = 0.0;
+    __syncthreads();  // tw
+    const int nunit = P * nrun;
+    for (int un = blockIdx.x; un < nunit; un += gridDim.x) {
+        const int r1 = un / nrun, n0 = (un % nrun) * per, n1 = min(T, n0 + per);
+        float2* trow = t + (size_t)r1 * N;
+        const bool ok = n0 + fl < n1;
+        float2 u[F::kOut];
+#pragma unroll
+        for (int m = 0; m < 8; ++m)
+            u[m] = ok ? trow[(size_t)(n0 + fl) * npix + i + m * F::kLanes] : make_float2(0.f, 0.f);
+        WLoads<M> wl;
+        w_load<N, M, CIRC>(wl, p + (size_t)r1 * N, S + (size_t)r1 * N, threadIdx.x, T, n0, n1, npix);
+        F::template run<true, false>(u, sx, 1, tw, i);
+        F::sync();  // the last exchange is read
+#pragma unroll
+        for (int m = 0; m < F::kOut; ++m) {
+            const int e = F::out_at(i, m);
+            if (e >= 0) sx[F::at(e)] = u[m];
+        }
+        __syncthreads();
+        w_phase<N, M, CIRC, true>(wl, trow, p + (size_t)r1 * N, S + (size_t)r1 * N, res, lam, T, n0, n1, npix);
+        __syncthreads();  // the terms
+        if (un + (int)gridDim.x >= nunit) pdl_trigger();
+        tot += w_terms<N>(res, n1 - n0);
+        __syncthreads();  // the terms are read
+    }
+    tot = warps_sum_t0(tot, red);
     if (threadIdx.x == 0) pq_parts[blockIdx.x] = tot;
 }
 
@@ -324,81 +484,91 @@ row_inv_w_128_kernel(float2* t, const float2* __restrict__ p, const float2* __re
 }
 
 // Pass C of a CG step with coils (ADJ = false), or the coil combination of the adjoint
-// (ADJ = true). One CTA per image row r1 holds that row of every frame: for each coil c it
-// inverse-transforms the rows t[c][n][r1] and accumulates conj(C_c) * (...) (Eq.
-// measurement-ij: A^H = sum_c conj(C_c) F^H mask). ADJ: the sum is x[n][r1]. Otherwise lam W p is
-// added from the p rows, q goes over coil 0's plane of t (rows r1, read by this CTA only) and the
-// row's partial Re <p, q> to pq_parts.
+// (ADJ = true). One CTA per image row r1, N / 8 threads per frame: for each coil c they
+// inverse-transform the row t[c][n][r1] and accumulate conj(C_c) * (...) in registers, the next coil's
+// row in flight meanwhile (Eq. measurement-ij: A^H = sum_c conj(C_c) F^H mask). ADJ: the sum is
+// x[n][r1]. Otherwise lam W p is added as in row_inv_w_kernel, q goes over coil 0's plane of t (rows r1,
+// read by this CTA only) and the row's partial Re <p, q> to pq_parts. 12 coils at 128x128x12: 42.3 ->
+// 12.5 us per launch, against a block barrier after every pass of every coil.
 template <int N, int M, bool ADJ>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(inv_threads<N>())
 coil_row_inv_kernel(float2* t, const float2* __restrict__ p, const float2* __restrict__ coils,
-                    const float2* __restrict__ S, float lam, int T, int P, int nc,
+                    const float2* __restrict__ S, float lam, int T, int P, int nc, int passes, int per,
                     double* __restrict__ pq_parts, float2* __restrict__ x_out,
                     const float2* __restrict__ tw_g) {
+    using F = RegFft<N>;
     extern __shared__ float2 sm[];
-    __shared__ double red[kThreads / 32];
-    float2* a = sm;
-    float2* b = a + (size_t)T * N;
-    float2* acc = b + (size_t)T * N;
-    float2* pt = acc + (size_t)T * N;
-    float2* tw = pt + (size_t)T * N;
+    __shared__ double red[16];
+    float2* tw = sm;
+    float2* res = sm + N;
     const int r1 = blockIdx.x;
     const size_t npix = (size_t)P * N;
     const size_t series = (size_t)T * npix;
     for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = tw_g[i];
+    const int fl = threadIdx.x / F::kLanes, i = threadIdx.x % F::kLanes;
     pdl_wait();
-    for (int e = threadIdx.x; e < T * N; e += blockDim.x) {
-        acc[e] = make_float2(0.f, 0.f);
-        if (!ADJ) pt[e] = p[(size_t)(e / N) * npix + (size_t)r1 * N + e % N];
-    }
-    for (int c = 0; c < nc; ++c) {
-        __syncthreads();  // a, b free again
-        for (int e = threadIdx.x; e < T * N; e += blockDim.x)
-            a[e] = t[c * series + (size_t)(e / N) * npix + (size_t)r1 * N + e % N];
-        __syncthreads();
-        float2* res = fft_smem<N, true, false>(a, b, T, N, 1, tw);
-        for (int e = threadIdx.x; e < T * N; e += blockDim.x) {
-            const float2 cv = coils[((size_t)c * P + r1) * N + e % N];
-            acc[e] = cfmacj(cv, res[e], acc[e]);
+    __syncthreads();  // tw
+    float2* trow = t + (size_t)r1 * N;
+    const float2* crow = coils + (size_t)r1 * N;
+    for (int ps = 0; ps < passes; ++ps) {
+        const int n = ps * per + fl;
+        const bool ok = fl < per && n < T;
+        float2* sx = res + (size_t)n * F::kBuf;
+        float2 acc[F::kOut], nx[8];
+#pragma unroll
+        for (int m = 0; m < F::kOut; ++m) acc[m] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int m = 0; m < 8; ++m)
+            nx[m] = ok ? trow[(size_t)n * npix + i + m * F::kLanes] : make_float2(0.f, 0.f);
+        for (int c = 0; c < nc; ++c) {
+            float2 u[F::kOut], cv[F::kOut];
+#pragma unroll
+            for (int m = 0; m < 8; ++m) u[m] = nx[m];
+            if (c + 1 < nc && ok) {
+#pragma unroll
+                for (int m = 0; m < 8; ++m)
+                    nx[m] = trow[(size_t)(c + 1) * series + (size_t)n * npix + i + m * F::kLanes];
+            }
+#pragma unroll
+            for (int m = 0; m < F::kOut; ++m) {
+                const int e = F::out_at(i, m);
+                cv[m] = e >= 0 ? crow[(size_t)c * npix + e] : make_float2(0.f, 0.f);
+            }
+            F::sync();  // the previous coil's last exchange is read
+            F::template run<true, false>(u, sx, 1, tw, i);
+#pragma unroll
+            for (int m = 0; m < F::kOut; ++m) acc[m] = cfmacj(cv[m], u[m], acc[m]);
         }
-    }
-    __syncthreads();
-    if constexpr (ADJ) {
-        pdl_trigger();
-        for (int e = threadIdx.x; e < T * N; e += blockDim.x)
-            x_out[(size_t)(e / N) * npix + (size_t)r1 * N + e % N] = acc[e];
-        return;
-    } else {
-        const int k = T - M + 1;
-        float accd = 0.f, comp = 0.f;  // Kahan-compensated per-thread partial of Re <p, q>
-        for (int c = threadIdx.x; c < N; c += blockDim.x) {
-            float2 s[M][M];
-            load_S<M>(S, npix, (size_t)r1 * N + c, s);
-            for (int n = 0; n < T; ++n) {
-                float2 w = make_float2(0.f, 0.f);
+        if constexpr (ADJ) {
+            if (ok) {
 #pragma unroll
-                for (int aa = 0; aa < M; ++aa) {
-                    const int j = n - M + 1 + aa;
-                    if (j < 0 || j >= k) continue;
-#pragma unroll
-                    for (int bb = 0; bb < M; ++bb)
-                    w = cfma(s[aa][bb], pt[wrap_frame(n + aa - bb, T) * N + c], w);
+                for (int m = 0; m < F::kOut; ++m) {
+                    const int e = F::out_at(i, m);
+                    if (e >= 0) x_out[(size_t)n * npix + (size_t)r1 * N + e] = acc[m];
                 }
-                float2 q = acc[n * N + c];
-                q.x = fmaf(lam, w.x, q.x);
-                q.y = fmaf(lam, w.y, q.y);
-                acc[n * N + c] = q;
-                const float2 pv = pt[n * N + c];
-                const float term = fmaf(pv.x, q.x, pv.y * q.y) - comp;
-                const float sum = accd + term;
-                comp = (sum - accd) - term;
-                accd = sum;
+            }
+        } else {
+            F::sync();
+#pragma unroll
+            for (int m = 0; m < F::kOut; ++m) {
+                const int e = F::out_at(i, m);
+                if (e >= 0) sx[F::at(e)] = acc[m];
             }
         }
-        const double tot = block_sum_f_t0(accd, red);
+        // spare threads of a pass share the next pass's first buffers
+        if (ps + 1 < passes) __syncthreads();
+    }
+    if constexpr (ADJ) {
         pdl_trigger();
-        for (int e = threadIdx.x; e < T * N; e += blockDim.x)
-            t[(size_t)(e / N) * npix + (size_t)r1 * N + e % N] = acc[e];
+        return;
+    } else {
+        __syncthreads();
+        WLoads<M> wl;
+        w_load<N, M, false>(wl, p + (size_t)r1 * N, S + (size_t)r1 * N, threadIdx.x, T, 0, T, npix);
+        w_phase<N, M, false, false>(wl, trow, p + (size_t)r1 * N, S + (size_t)r1 * N, res, lam, T, 0, T, npix);
+        __syncthreads();  // the terms
+        pdl_trigger();
+        const double tot = warps_sum_t0(w_terms<N>(res, T), red);
         if (threadIdx.x == 0) pq_parts[blockIdx.x] = tot;
     }
 }
@@ -628,14 +798,31 @@ apply_w_kernel(const float2* __restrict__ x, const float2* __restrict__ S, float
 
 // Grid of a row kernel: one CTA per row while the rows fit one resident wave, else one wave
 // (the CTAs then loop over rows), so that the pass leaves at most a wave of partials.
+// The occupancy query costs more host time than a launch: its answers are kept (a few shapes per
+// kernel; the table is shared by all threads).
 template <typename K>
-cudaError_t row_grid(K kern, int threads, size_t smem, int rows, int* grid) {
-    int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+cudaError_t row_grid(K kern, int threads, size_t smem, long long rows, int* grid) {
+    static std::mutex mu;
+    static std::map<std::tuple<int, const void*, int, size_t>, int> known;
+    int dev = 0, per_sm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    long long wave = (long long)(per_sm < 1 ? 1 : per_sm) * num_sms();
+    const auto key = std::make_tuple(dev, reinterpret_cast<const void*>(kern), threads, smem);
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        auto it = known.find(key);
+        if (it != known.end()) per_sm = it->second;
+    }
+    if (!per_sm) {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+        if (e != cudaSuccess) return e;
+        if (per_sm < 1) per_sm = 1;
+        std::lock_guard<std::mutex> lock(mu);
+        if (known.size() < 4096) known[key] = per_sm;
+    }
+    long long wave = (long long)per_sm * num_sms();
     if (wave > kMaxParts) wave = kMaxParts;
-    *grid = rows < wave ? rows : (int)wave;
+    *grid = (int)(rows < wave ? rows : wave);
     return cudaSuccess;
 }
 
@@ -683,15 +870,16 @@ cudaError_t launch_row_inv_w_NM(const Dims& d, const Twiddles& tw, float2* t, co
         }
     }
     auto k = d.circ ? row_inv_w_kernel<N, M, true> : row_inv_w_kernel<N, M, false>;
-    const size_t smem = ((size_t)3 * d.T * N + N) * sizeof(float2);
+    const RunShape v = run_shape<N>(d.T, rows);
+    const size_t smem = ((size_t)v.bufs * RegFft<N>::kBuf + N) * sizeof(float2);
     if (smem > kDynSmemFree) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    cudaError_t e = row_grid(k, kThreads, smem, rows, &grid);
+    cudaError_t e = row_grid(k, v.threads, smem, (long long)rows * v.nrun, &grid);
     if (e != cudaSuccess) return e;
     pq->n = grid;
-    return launch_pdl(k, dim3(grid), dim3(kThreads), smem, st, t, p, S, lam, d.T, rows,
+    return launch_pdl(k, dim3(grid), dim3(v.threads), smem, st, t, p, S, lam, d.T, rows, v.nrun, v.per,
                       pq->parts, tw.twQ);
 }
 
@@ -728,14 +916,16 @@ cudaError_t launch_coil_inv_NM(const Dims& d, const Twiddles& tw, float2* t, con
                                const float2* coils, const float2* S, float lam, double* pq_parts,
                                float2* x_out, cudaStream_t st) {
     auto k = coil_row_inv_kernel<N, M, ADJ>;
-    const size_t smem = ((size_t)4 * d.T * N + N) * sizeof(float2);
-    if (smem > 220 * 1024) return cudaErrorInvalidValue;
+    // (the series that the coil passes take: four copies of the rows within the shared memory)
+    if (((size_t)4 * d.T * N + N) * sizeof(float2) > 220 * 1024) return cudaErrorInvalidValue;
+    const InvShape v = inv_shape<N>(d.T);
+    const size_t smem = ((size_t)v.bufs * RegFft<N>::kBuf + N) * sizeof(float2);
     if (smem > kDynSmemFree) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    return launch_pdl(k, dim3(d.P), dim3(kThreads), smem, st, t, p, coils, S, lam, d.T, d.P, d.nc,
-                      pq_parts, x_out, tw.twQ);
+    return launch_pdl(k, dim3(d.P), dim3(v.threads), smem, st, t, p, coils, S, lam, d.T, d.P, d.nc,
+                      v.passes, v.per, pq_parts, x_out, tw.twQ);
 }
 
 template <int N, bool ADJ>

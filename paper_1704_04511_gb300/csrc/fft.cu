@@ -2,14 +2,15 @@
 // (Sec. II-A, Eq. measurement-ij with one coil) and by the CG operator (Sec. III-A, Eq. grad-ls).
 //
 // Layout: frames [T][P][Q] complex64, Q contiguous. A row pass transforms length-Q rows
-// (ROWS rows per CTA, staged in shared memory); a column pass transforms a P x 8 tile of
-// 8 adjacent columns of one frame (64-byte row segments), optionally applying the
+// (elements in registers, a few rows per CTA); a column pass transforms a tile of 8, 16 or 32
+// adjacent columns of one frame (64- to 256-byte row segments), optionally applying the
 // sampling mask between a forward and an inverse transform so that A^H A needs one column pass.
 #include <cuda_bf16.h>
 
 #include "common.cuh"
 #include "kernels.h"
 #include "regfft.cuh"
+#include "stockham.cuh"
 
 namespace recon {
 
@@ -17,9 +18,6 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kColTile = 8;
-
-template <int N>
-__host__ __device__ constexpr int rows_per_cta() { return N >= 1024 ? 1 : 1024 / N; }
 
 // Columns per CTA of the column passes: 8, 16 or 32 (64- to 256-byte row segments). The default
 // for the volume passes is about 2048 elements per CTA (8 per thread, 33 KB of shared memory,
@@ -31,90 +29,120 @@ constexpr bool col_tile_ok() { return (size_t)(2 * N * C + N) * sizeof(float2) <
 
 enum ColMode { COL_FWD = 0, COL_INV = 1, COL_MASK_OP = 2, COL_ADJ_C64 = 3, COL_ADJ_BF16 = 4 };
 
+// Threads of a row pass: whole warps and whole sequences, 64 where these fit (small CTAs: the
+// passes are latency-bound and an SM holds many).
+template <int N>
+__host__ __device__ constexpr int row_threads() { return N == 192 ? 96 : (N == 512 ? 128 : 64); }
+template <int N>
+__host__ __device__ constexpr int row_seqs() { return row_threads<N>() / RegFft<N>::kLanes; }
+
 template <int N, bool INV>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(row_threads<N>())
 row_fft_kernel(const float2* in, float2* out, int nrows, float scale,
                const float2* __restrict__ tw_g) {
-    constexpr int ROWS = rows_per_cta<N>();
-    extern __shared__ float2 sm[];
-    float2* a = sm;
-    float2* b = a + ROWS * N;
-    float2* tw = b + ROWS * N;
+    using F = RegFft<N>;
+    __shared__ float2 tw[N];
+    __shared__ float2 sx[row_seqs<N>()][F::kBuf];
     for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = tw_g[i];
-    const int row0 = blockIdx.x * ROWS;
-    const int nr = min(ROWS, nrows - row0);
-    const size_t base = (size_t)row0 * N;
-    for (int e = threadIdx.x; e < nr * N; e += blockDim.x) a[e] = in[base + e];
-    __syncthreads();
-    float2* res = fft_smem<N, INV, false>(a, b, nr, N, 1, tw);
-    for (int e = threadIdx.x; e < nr * N; e += blockDim.x) out[base + e] = cscale(res[e], scale);
+    const int lr = threadIdx.x / F::kLanes, i = threadIdx.x % F::kLanes;
+    const int row = blockIdx.x * row_seqs<N>() + lr;
+    const bool ok = row < nrows;
+    const size_t base = (size_t)row * N;
+    float2 u[F::kOut];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) u[m] = ok ? in[base + i + m * F::kLanes] : make_float2(0.f, 0.f);
+    __syncthreads();  // tw
+    F::template run<INV, false>(u, sx[lr], 1, tw, i);
+    if (!ok) return;
+#pragma unroll
+    for (int m = 0; m < F::kOut; ++m) {
+        const int e = F::out_at(i, m);
+        if (e >= 0) out[base + e] = cscale(u[m], scale);
+    }
 }
 
 // Pass A of a CG step: p = r (first) or r + beta p with beta = |r_c|^2 / |r_{c-1}|^2, |r_c|^2
 // summed here from the update pass's per-CTA partials (CTA 0 also stores it); p is written back
-// and its row FFT goes to t.
+// and its row FFT goes to t. The elements stay in registers (RegFft): 192x192x24 9.0 -> 7.5 us per
+// launch, 512x512x16 35.9 -> 24.0, against passes over shared memory with a block barrier each.
 template <int N>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(row_threads<N>())
 row_fwd_pupdate_kernel(const float2* __restrict__ r, float2* __restrict__ p,
                        float2* __restrict__ t, int nrows, const double* __restrict__ rr_parts,
                        int n_rr, const double* __restrict__ rr_prev, double* __restrict__ rr_out,
                        int first, const float2* __restrict__ tw_g) {
-    constexpr int ROWS = rows_per_cta<N>();
-    extern __shared__ float2 sm[];
+    using F = RegFft<N>;
+    __shared__ float2 tw[N];
+    __shared__ float2 sx[row_seqs<N>()][F::kBuf];
     __shared__ float beta_s;
-    __shared__ double s_rr;
-    float2* a = sm;
-    float2* b = a + ROWS * N;
-    float2* tw = b + ROWS * N;
     for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = tw_g[i];
     pdl_wait();
-    float beta = 0.f;
+    const int lr = threadIdx.x / F::kLanes, i = threadIdx.x % F::kLanes;
+    const int row = blockIdx.x * row_seqs<N>() + lr;
+    const bool ok = row < nrows;
+    const size_t base = (size_t)row * N + i;
+    float2 u[F::kOut], pv[8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) u[m] = ok ? r[base + m * F::kLanes] : make_float2(0.f, 0.f);
     if (!first) {
-        const double rr_new = sum_partials(rr_parts, n_rr, &s_rr);
-        if (threadIdx.x == 0) {
-            beta_s = (float)(rr_new * rcp_nr(rr_prev[0]));
-            if (blockIdx.x == 0) rr_out[0] = rr_new;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) pv[m] = ok ? p[base + m * F::kLanes] : make_float2(0.f, 0.f);
+        if (threadIdx.x < 32) {  // |r|^2 from the update pass's partials, loads in flight
+            const double rr_new = warp0_sum_array(rr_parts, n_rr);
+            if (threadIdx.x == 0) {
+                beta_s = (float)(rr_new * rcp_nr(rr_prev[0]));
+                if (blockIdx.x == 0) rr_out[0] = rr_new;
+            }
         }
-        __syncthreads();
-        beta = beta_s;
     }
-    const int row0 = blockIdx.x * ROWS;
-    const int nr = min(ROWS, nrows - row0);
-    const size_t base = (size_t)row0 * N;
-    for (int e = threadIdx.x; e < nr * N; e += blockDim.x) {
-        float2 v = r[base + e];
-        if (!first) {
-            const float2 pv = p[base + e];
-            v.x = fmaf(beta, pv.x, v.x);
-            v.y = fmaf(beta, pv.y, v.y);
+    __syncthreads();  // tw, beta
+    if (!first) {
+        const float beta = beta_s;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            u[m].x = fmaf(beta, pv[m].x, u[m].x);
+            u[m].y = fmaf(beta, pv[m].y, u[m].y);
         }
-        p[base + e] = v;
-        a[e] = v;
     }
-    __syncthreads();
-    float2* res = fft_smem<N, false, false>(a, b, nr, N, 1, tw);
+    if (ok) {
+#pragma unroll
+        for (int m = 0; m < 8; ++m) p[base + m * F::kLanes] = u[m];
+    }
+    F::template run<false, false>(u, sx[lr], 1, tw, i);
     pdl_trigger();
-    for (int e = threadIdx.x; e < nr * N; e += blockDim.x) t[base + e] = res[e];
+    if (!ok) return;
+#pragma unroll
+    for (int m = 0; m < F::kOut; ++m) {
+        const int e = F::out_at(i, m);
+        if (e >= 0) t[(size_t)row * N + e] = u[m];
+    }
 }
 
 // Pass A of a CG step with coils (Eq. measurement-ij): p = r (first) or r + beta p as in
 // row_fwd_pupdate_kernel, then for every coil c the row FFT of C_c * p goes to the coil-major
-// transform buffer t[c][n] (rows of the T x P row space; coil maps [nc][P][Q]).
+// transform buffer t[c][n] (rows of the T x P row space; coil maps [nc][P][Q]). A CTA updates
+// coil_rows rows of p, keeps them in shared memory, and deals the (coil, row) transforms to its
+// thread groups: 12 coils at 128x128x12 23.5 -> 11.4 us per launch, against one coil after the other
+// on 192 CTAs.
 template <int N>
-__global__ void __launch_bounds__(kThreads)
+__host__ __device__ constexpr int coil_threads() { return N == 192 ? 192 : 256; }
+template <int N>
+__host__ __device__ constexpr int coil_rows() { return N >= 512 ? 1 : 512 / N; }
+
+template <int N>
+__global__ void __launch_bounds__(coil_threads<N>())
 coil_row_fwd_kernel(const float2* __restrict__ r, float2* __restrict__ p, float2* __restrict__ t,
                     const float2* __restrict__ coils, int nrows, int P, int nc,
                     const double* __restrict__ rr_parts, int n_rr,
                     const double* __restrict__ rr_prev, double* __restrict__ rr_out, int first,
                     const float2* __restrict__ tw_g) {
-    constexpr int ROWS = rows_per_cta<N>();
-    extern __shared__ float2 sm[];
+    using F = RegFft<N>;
+    constexpr int ROWS = coil_rows<N>(), GROUPS = coil_threads<N>() / F::kLanes;
+    __shared__ float2 tw[N];
+    __shared__ float2 pk[ROWS * N];
+    __shared__ float2 sx[GROUPS][F::kBuf];
     __shared__ float beta_s;
     __shared__ double s_rr;
-    float2* a = sm;
-    float2* b = a + ROWS * N;
-    float2* pk = b + ROWS * N;
-    float2* tw = pk + ROWS * N;
     for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = tw_g[i];
     pdl_wait();
     float beta = 0.f;
@@ -141,26 +169,119 @@ coil_row_fwd_kernel(const float2* __restrict__ r, float2* __restrict__ p, float2
         p[base + e] = v;
         pk[e] = v;
     }
-    for (int c = 0; c < nc; ++c) {
-        __syncthreads();  // pk written / a, b free again
-        for (int e = threadIdx.x; e < nr * N; e += blockDim.x) {
-            const int row = row0 + e / N;
-            const float2 cv = coils[((size_t)c * P + row % P) * N + e % N];
-            a[e] = cmul(cv, pk[e]);
+    __syncthreads();  // pk, tw
+    const int g = threadIdx.x / F::kLanes, i = threadIdx.x % F::kLanes;
+    const int tasks = nc * nr;
+    float2 cv[8];  // the coil map row of the next task, in flight during the transform
+    auto load_map = [&](int k) {
+        const int c = k / nr, lr = k % nr;
+        const float2* m0 = coils + ((size_t)c * P + (row0 + lr) % P) * N + i;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) cv[m] = k < tasks ? m0[m * F::kLanes] : make_float2(0.f, 0.f);
+    };
+    load_map(g);
+    for (int k0 = 0; k0 < tasks; k0 += GROUPS) {  // uniform: the groups may meet in __syncthreads
+        const int k = k0 + g, c = k / nr, lr = k % nr;
+        const bool ok = k < tasks;
+        float2 u[F::kOut];
+#pragma unroll
+        for (int m = 0; m < 8; ++m) u[m] = cmul(cv[m], pk[(ok ? lr * N : 0) + i + m * F::kLanes]);
+        load_map(k + GROUPS);
+        F::sync();  // the buffer's last reads are done
+        F::template run<false, false>(u, sx[g], 1, tw, i);
+        if (k0 + GROUPS >= tasks) pdl_trigger();
+        if (!ok) continue;
+#pragma unroll
+        for (int m = 0; m < F::kOut; ++m) {
+            const int e = F::out_at(i, m);
+            if (e >= 0) t[c * series + base + (size_t)lr * N + e] = u[m];
         }
-        __syncthreads();
-        float2* res = fft_smem<N, false, false>(a, b, nr, N, 1, tw);
-        if (c == nc - 1) pdl_trigger();
-        for (int e = threadIdx.x; e < nr * N; e += blockDim.x) t[c * series + base + e] = res[e];
     }
 }
 
-// Column pass over an N x C tile (frame blockIdx.y, columns C*blockIdx.x ..), Stockham passes
-// in radix schedule S (fft_radix_at).
-template <int N, int MODE, int C, int S>
+// Column pass over an N x C tile (frame blockIdx.y, columns C*blockIdx.x ..), thread (column c,
+// lane i) holding eight elements of column c in registers (RegFft; C N / 8 threads). Between the
+// forward and the inverse transform of the mask operator the elements stay where they are (a result
+// slot of the last pass is an input slot of the first one; lengths with a factor of three exchange
+// once more). 192x192x24 9.6 -> 7.3 us per launch, 512x512x16 36.1 -> 29.3, against passes over
+// shared memory. (Four columns per CTA at 512: 30.8 us.)
+template <int N, int MODE, int C>
+__global__ void __launch_bounds__(C * RegFft<N>::kLanes, 1024 / (C * RegFft<N>::kLanes))  // 64 registers
+col_reg_kernel(const void* in_, float2* out, const uint8_t* __restrict__ mask,
+               int Q, int mask_frames, float scale, const float2* __restrict__ tw_g) {
+    using F = RegFft<N>;
+    constexpr bool kMasked = MODE == COL_ADJ_C64 || MODE == COL_ADJ_BF16;
+    extern __shared__ float2 sm[];
+    float2* tw = sm;
+    float2* sx = sm + N + threadIdx.x % C;  // element e of column c at at(e) * C + c
+    for (int e = threadIdx.x; e < N; e += blockDim.x) tw[e] = tw_g[e];
+    pdl_wait();
+    const int c = blockIdx.x * C + threadIdx.x % C, i = threadIdx.x / C;
+    const size_t fbase = (size_t)blockIdx.y * N * Q + c;
+    // coil-major series: frame blockIdx.y is coil blockIdx.y / T of frame blockIdx.y % T
+    const size_t mbase = (size_t)(blockIdx.y % mask_frames) * N * Q + c;
+    float2 u[F::kOut];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+        const size_t g = fbase + (size_t)(i + m * F::kLanes) * Q;
+        if constexpr (MODE == COL_ADJ_BF16)
+            u[m] = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(in_)[g]);
+        else
+            u[m] = reinterpret_cast<const float2*>(in_)[g];
+    }
+    // (scaled with __fmul_rn: not contracted into the butterfly's additions)
+    if constexpr (kMasked) {
+#pragma unroll
+        for (int m = 0; m < 8; ++m)
+            u[m] = mask[mbase + (size_t)(i + m * F::kLanes) * Q]
+                       ? make_float2(__fmul_rn(u[m].x, scale), __fmul_rn(u[m].y, scale))
+                       : make_float2(0.f, 0.f);
+    }
+    uint8_t mk[F::kOut];
+    if constexpr (MODE == COL_MASK_OP) {
+#pragma unroll
+        for (int m = 0; m < F::kOut; ++m) {
+            const int e = F::out_at(i, m);
+            mk[m] = e >= 0 ? mask[mbase + (size_t)e * Q] : 0;
+        }
+    }
+    __syncthreads();  // tw
+    F::template run<MODE == COL_INV || kMasked, true>(u, sx, C, tw, i);
+    if constexpr (MODE == COL_MASK_OP) {
+#pragma unroll
+        for (int m = 0; m < F::kOut; ++m)
+            u[m] = mk[m] ? make_float2(__fmul_rn(u[m].x, scale), __fmul_rn(u[m].y, scale))
+                         : make_float2(0.f, 0.f);
+        __syncthreads();  // the last exchange is read
+        if constexpr (F::kOdd) {
+#pragma unroll
+            for (int m = 0; m < F::kOut; ++m) {
+                const int e = F::out_at(i, m);
+                if (e >= 0) sx[F::at(e) * C] = u[m];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int m = 0; m < 8; ++m) u[m] = sx[F::at(i + m * F::kLanes) * C];
+            __syncthreads();
+        }
+        F::template run<true, true>(u, sx, C, tw, i);
+    }
+    pdl_trigger();
+    const float osc = (MODE == COL_FWD || MODE == COL_INV) ? scale : 1.f;
+#pragma unroll
+    for (int m = 0; m < F::kOut; ++m) {
+        const int e = F::out_at(i, m);
+        if (e >= 0) out[fbase + (size_t)e * Q] = cscale(u[m], osc);
+    }
+}
+
+// The same in radix schedule 1 (radix 4 before 8; chosen by the tuner on request only), by passes
+// over shared memory.
+template <int N, int MODE, int C>
 __global__ void __launch_bounds__(kThreads)
-col_kernel(const void* in_, float2* out, const uint8_t* __restrict__ mask,
+col_kernel(const float2* in, float2* out, const uint8_t* __restrict__ mask,
            int Q, int mask_frames, float scale, const float2* __restrict__ tw_g) {
+    constexpr int S = 1;
     extern __shared__ float2 sm[];
     float2* a = sm;
     float2* b = a + N * C;
@@ -171,27 +292,13 @@ col_kernel(const void* in_, float2* out, const uint8_t* __restrict__ mask,
     const size_t fbase = (size_t)blockIdx.y * N * Q;
     // coil-major series: frame blockIdx.y is coil blockIdx.y / T of frame blockIdx.y % T
     const size_t mbase = (size_t)(blockIdx.y % mask_frames) * N * Q;
-    for (int e = threadIdx.x; e < N * C; e += blockDim.x) {
-        const int i = e / C, c = e % C;
-        const size_t g = fbase + (size_t)i * Q + c0 + c;
-        const size_t gm = mbase + (size_t)i * Q + c0 + c;
-        float2 v;
-        if constexpr (MODE == COL_ADJ_BF16) {
-            const __nv_bfloat162 h = reinterpret_cast<const __nv_bfloat162*>(in_)[g];
-            v = __bfloat1622float2(h);
-        } else {
-            v = reinterpret_cast<const float2*>(in_)[g];
-        }
-        if constexpr (MODE == COL_ADJ_C64 || MODE == COL_ADJ_BF16) {
-            v = mask[gm] ? cscale(v, scale) : make_float2(0.f, 0.f);
-        }
-        a[e] = v;
-    }
+    for (int e = threadIdx.x; e < N * C; e += blockDim.x)
+        a[e] = in[fbase + (size_t)(e / C) * Q + c0 + e % C];
     __syncthreads();
     float2* res;
     if constexpr (MODE == COL_FWD) {
         res = fft_smem<N, false, true, 1, S>(a, b, C, 1, C, tw);
-    } else if constexpr (MODE == COL_INV || MODE == COL_ADJ_C64 || MODE == COL_ADJ_BF16) {
+    } else if constexpr (MODE == COL_INV) {
         res = fft_smem<N, true, true, 1, S>(a, b, C, 1, C, tw);
     } else {  // COL_MASK_OP
         float2* f = fft_smem<N, false, true, 1, S>(a, b, C, 1, C, tw);
@@ -787,14 +894,14 @@ col_fold_inv_kernel(float2* t) {
     for (int n = 0; n < 16; ++n) t[base + (size_t)(8 * n) * Q] = u[n];
 }
 
-template <int N>
-size_t row_smem() { return (size_t)(2 * rows_per_cta<N>() * N + N) * sizeof(float2); }
+template <int N, int C>
+size_t col_reg_smem() { return (size_t)(RegFft<N>::kBuf * C + N) * sizeof(float2); }
 template <int N, int C>
 size_t col_smem() { return (size_t)(2 * N * C + N) * sizeof(float2); }
 
 template <typename K>
 cudaError_t set_smem(K kern, size_t bytes) {
-    if (bytes > 48 * 1024)
+    if (bytes > 40 * 1024)  // (next to a kernel's static arrays)
         return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     return cudaSuccess;
 }
@@ -808,11 +915,8 @@ cudaError_t row_fft(int n, const float2* in, float2* out, int nrows, float scale
     switch (n) {
 #define CASE(N)                                                                          \
     case N: {                                                                            \
-        auto k = row_fft_kernel<N, INV>;                                                 \
-        cudaError_t e = set_smem(k, row_smem<N>());                                      \
-        if (e != cudaSuccess) return e;                                                  \
-        const int grid = (nrows + rows_per_cta<N>() - 1) / rows_per_cta<N>();            \
-        k<<<grid, kThreads, row_smem<N>(), st>>>(in, out, nrows, scale, tw);             \
+        const int grid = (nrows + row_seqs<N>() - 1) / row_seqs<N>();                    \
+        row_fft_kernel<N, INV><<<grid, row_threads<N>(), 0, st>>>(in, out, nrows, scale, tw); \
         return cudaGetLastError();                                                       \
     }
         RECON_FFT_SIZES(CASE)
@@ -824,12 +928,20 @@ cudaError_t row_fft(int n, const float2* in, float2* out, int nrows, float scale
 template <int N, int MODE, int C, int S>
 cudaError_t col_launch(int Q, int T, int mask_frames, const void* in, float2* out,
                        const uint8_t* mask, float scale, const float2* tw, cudaStream_t st) {
-    auto k = col_kernel<N, MODE, C, S>;
-    cudaError_t e = set_smem(k, col_smem<N, C>());
-    if (e != cudaSuccess) return e;
-    dim3 grid(Q / C, T);
-    return launch_pdl(k, grid, dim3(kThreads), col_smem<N, C>(), st, in, out, mask, Q, mask_frames,
-                      scale, tw);
+    const dim3 grid(Q / C, T);
+    if constexpr (S == 0) {
+        auto k = col_reg_kernel<N, MODE, C>;
+        cudaError_t e = set_smem(k, col_reg_smem<N, C>());
+        if (e != cudaSuccess) return e;
+        return launch_pdl(k, grid, dim3(C * RegFft<N>::kLanes), col_reg_smem<N, C>(), st, in, out, mask,
+                          Q, mask_frames, scale, tw);
+    } else {
+        auto k = col_kernel<N, MODE, C>;
+        cudaError_t e = set_smem(k, col_smem<N, C>());
+        if (e != cudaSuccess) return e;
+        return launch_pdl(k, grid, dim3(kThreads), col_smem<N, C>(), st, (const float2*)in, out, mask, Q,
+                          mask_frames, scale, tw);
+    }
 }
 
 // Tile width C (rounded down to what Q and the shared memory allow; 8 at least) and radix
@@ -966,14 +1078,11 @@ cudaError_t launch_row_fwd_pupdate(const Dims& d, const Twiddles& tw, const floa
     switch (d.Q) {
 #define CASE(N)                                                                              \
     case N: {                                                                                \
-        auto k = row_fwd_pupdate_kernel<N>;                                                  \
-        cudaError_t e = set_smem(k, row_smem<N>());                                          \
-        if (e != cudaSuccess) return e;                                                      \
-        const int grid = (nrows + rows_per_cta<N>() - 1) / rows_per_cta<N>();                \
-        return launch_pdl(k, dim3(grid), dim3(kThreads), row_smem<N>(), st, r, p, t, nrows,  \
-                          (const double*)rr.parts, rr.n, rr_prev, rr_out, first, tw.twQ);    \
+        const int grid = (nrows + row_seqs<N>() - 1) / row_seqs<N>();                        \
+        return launch_pdl(row_fwd_pupdate_kernel<N>, dim3(grid), dim3(row_threads<N>()), 0, st, r, p, t, \
+                          nrows, (const double*)rr.parts, rr.n, rr_prev, rr_out, first, tw.twQ); \
     }
-        RECON_FFT_SIZES(CASE)
+        CASE(16) CASE(32) CASE(64) CASE(192) CASE(512)
 #undef CASE
         default: return cudaErrorInvalidValue;
     }
@@ -986,14 +1095,10 @@ cudaError_t launch_coil_row_fwd(const Dims& d, const Twiddles& tw, const float2*
     switch (d.Q) {
 #define CASE(N)                                                                              \
     case N: {                                                                                \
-        auto k = coil_row_fwd_kernel<N>;                                                     \
-        const size_t smem = (size_t)(3 * rows_per_cta<N>() * N + N) * sizeof(float2);       \
-        cudaError_t e = set_smem(k, smem);                                                   \
-        if (e != cudaSuccess) return e;                                                      \
-        const int grid = (nrows + rows_per_cta<N>() - 1) / rows_per_cta<N>();                \
-        return launch_pdl(k, dim3(grid), dim3(kThreads), smem, st, r, p, t, coils, nrows,    \
-                          d.P, d.nc, (const double*)rr.parts, rr.n, rr_prev, rr_out, first,  \
-                          tw.twQ);                                                           \
+        const int grid = (nrows + coil_rows<N>() - 1) / coil_rows<N>();                      \
+        return launch_pdl(coil_row_fwd_kernel<N>, dim3(grid), dim3(coil_threads<N>()), 0, st, r, p, t, \
+                          coils, nrows, d.P, d.nc, (const double*)rr.parts, rr.n, rr_prev,    \
+                          rr_out, first, tw.twQ);                                            \
     }
         RECON_FFT_SIZES(CASE)
 #undef CASE

@@ -199,3 +199,68 @@ def test_shared_memory_next_to_the_default_limit(Q, T):
             "recon.recon_apply_normal(c.h, m, (3, 3, 1), S, 0.5, x, y)\n"
             "assert (y - x).abs().max() < 1e-5 * x.abs().max()\n")
     subprocess.run([sys.executable, "-c", code], check=True, timeout=120)
+
+
+def _series(rng, *shape):
+    return (rng.standard_normal(shape) + 1j * rng.standard_normal(shape)).astype(np.complex64)
+
+
+def _hermitian_pairs(rng, M, P, Q):
+    S = _series(rng, M * (M + 1) // 2, P, Q)
+    full = np.zeros((M, M, P, Q), dtype=np.complex128)
+    e = 0
+    for a in range(M):
+        S[e].imag = 0
+        for b in range(a, M):
+            full[a, b], full[b, a] = S[e], S[e].conj()
+            e += 1
+    return S, full
+
+
+def _w(full, x, circ):
+    M, T = full.shape[0], x.shape[0]
+    y = np.zeros(x.shape, dtype=np.complex128)
+    for a in range(M):
+        for b in range(M):
+            if circ:
+                y += full[a, b] * np.roll(x, b - a, 0)
+            else:
+                k = T - M + 1
+                y[M - 1 - a:M - 1 - a + k] += full[a, b] * x[M - 1 - b:M - 1 - b + k]
+    return y
+
+
+@pytest.mark.parametrize("T,P,Q,M", [(1, 16, 16, 1), (300, 16, 16, 2), (8, 32, 32, 2), (150, 16, 32, 3),
+                                     (21, 64, 64, 2), (5, 192, 64, 5), (24, 192, 192, 3), (17, 32, 192, 6),
+                                     (13, 512, 512, 2), (16, 16, 512, 4), (3, 512, 16, 3),
+                                     (13, 256, 128, 3), (12, 128, 256, 2)])
+def test_operators_at_run_edges(R, T, P, Q, M):
+    """A^H A + lam W over row lengths 16 to 512 with frame counts that leave remainders in the runs of
+    frames and in the CTAs' sequences, the time-circular form, three coils and the adjoint, against
+    FP64: the gates of the operator parity tests (1e-5; 2e-6 for the adjoint)."""
+    import torch
+    recon, ctx = R
+    rng = np.random.default_rng(T + P + Q)
+    x = _series(rng, T, P, Q)
+    S, full = _hermitian_pairs(rng, M, P, Q)
+    m = (rng.random((T, P, Q)) < 0.4).astype(np.uint8)
+    lam, xd = 0.7, to_dev(x)
+    y = torch.empty_like(xd)
+
+    def aha(v):
+        return np.fft.ifft2(m * np.fft.fft2(v, norm="ortho"), norm="ortho")
+
+    for circ, variant in ((False, recon.RECON_VARIANT_PROPOSED), (True, recon.RECON_VARIANT_GIRAF)):
+        recon.recon_apply_normal_variant(ctx.h, to_dev(m), (1, 1, M), variant, to_dev(S), lam, xd, y)
+        assert_close(y.cpu().numpy(), aha(x) + lam * _w(full, x, circ), 1e-5)
+    recon.recon_adjoint(ctx.h, xd, to_dev(m), y)
+    assert_close(y.cpu().numpy(), np.fft.ifft2(m * x, norm="ortho"), 2e-6)
+    if 4 * T * Q + Q > 220 * 1024 // 8:
+        return
+    C = _series(rng, 3, P, Q)
+    recon.recon_apply_normal_coils(ctx.h, to_dev(m), to_dev(C), (1, 1, M), to_dev(S), lam, xd, y)
+    ref = sum(c.conj() * aha(c * x) for c in C.astype(np.complex128)) + lam * _w(full, x, False)
+    assert_close(y.cpu().numpy(), ref, 1e-5)
+    b = _series(rng, 3, T, P, Q)
+    recon.recon_adjoint_coils(ctx.h, to_dev(b), to_dev(m), to_dev(C), y)
+    assert_close(y.cpu().numpy(), sum(c.conj() * np.fft.ifft2(m * v, norm="ortho") for c, v in zip(C, b)), 2e-6)
