@@ -648,13 +648,13 @@ __global__ void hdiag_kernel(const double2* __restrict__ H, int N1, int N2, int 
 // reduction after the barrier. CTA 0 publishes (alpha_k, beta_{k-1}^2).
 //
 // The last CTA takes no part in the barriers: it takes the largest eigenvalue of the tridiagonal of
-// the first 8, 12, 16, ... published steps and asks CTA 0 to end the iteration once it has not grown
-// by 1e-15 of itself over four steps (the workers are a few steps ahead by then). lambda_max of Grams of image
-// series stands after ~14-18 steps, that of random series with a 0.2 % top gap after ~40-50; a fixed
-// 64 steps with two barriers each took 805 us at s = 243 (12.6 us a step) on every first iteration.
-// The bound of a step is latency: the barrier, the dependent FP64 chains (64 cycles an operation)
-// and the FP64 issue of the redundant vector work. s = 243 series: 805 -> 220 us
-// (recon_weight with its own eps 1090 -> 505 us).
+// the first 8, 10, 12, ... published steps and asks CTA 0 to end the iteration once it has not grown
+// by 5e-16 of itself over two steps (the workers are a few steps ahead by then; at the last step the
+// value is taken as it is). lambda_max of Grams of image series stands after ~20-26 steps, that of
+// random series with a 0.2 % top gap after ~40-50; a fixed 64 steps with two barriers each took 805 us
+// at s = 243 (12.6 us a step) on every first iteration. The bound of a step is latency: the barrier,
+// the dependent FP64 chains (64 cycles an operation) and the FP64 issue of the redundant vector work.
+// s = 243 series: 137 us (recon_weight with its own eps 1100 -> 424 us).
 struct LancMat {
     const double2* G;   // s x s column-major, Hermitian
     double2* w;         // G q of a step, two buffers of s
@@ -670,6 +670,16 @@ constexpr unsigned int kLancFin = 0x40000000u;  // published step count: the ite
 RECON_DEV int exponent_of(double v) { return (int)((__double_as_longlong(v) >> 52) & 0x7ff) - 1023; }
 RECON_DEV double pow2i(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
+// v 2^e by integer arithmetic (the FP64 pipe is what the Lanczos step waits for); zero below the normal
+// numbers, NaN above them.
+RECON_DEV double scale2(double v, int e) {
+    const int hi = __double2hiint(v), ex = (hi >> 20) & 0x7ff;
+    if (ex == 0x7ff) return v;
+    if (ex == 0 || ex + e <= 0) return 0.0;
+    if (ex + e >= 0x7ff) return __longlong_as_double(0x7ff8000000000000LL);
+    return __hiloint2double(hi + e * (1 << 20), __double2loint(v));
+}
+
 // Two sums over a warp in one tree: lane 0 returns the sum of a, lane 16 that of b (every FP64
 // instruction of a warp costs the SM's FP64 pipe the same, however many lanes it is for).
 RECON_DEV double warp_sum_pair(double a, double b, int lane) {
@@ -681,18 +691,29 @@ RECON_DEV double warp_sum_pair(double a, double b, int lane) {
     return v;
 }
 
-// Barrier of the worker CTAs 0 .. n-1 of a larger grid (as grid_barrier).
+// Barrier of the worker CTAs 0 .. n-1 of a larger grid, as grid_barrier, without fences of its own: the
+// acquire-release arrival orders the CTA's writes (they come before it through the block barrier), and
+// the acquire of the poll, or of the arrival that completes the barrier, orders its reads.
 RECON_DEV bool worker_barrier(GridBar* gb, const CoopFault& fault, unsigned int n) {
     __shared__ int ok_s;
     __syncthreads();
     if (threadIdx.x == 0) {
         int ok = !(fault.withhold > 0 && (int)blockIdx.x == fault.withhold);
         if (ok) {
-            __threadfence();
             const unsigned int inc = blockIdx.x == 0 ? 0x80000000u - (n - 1u) : 1u;
             const unsigned int old = atom_add_acq_rel(&gb->word, inc);
-            if ((((old + inc) ^ old) & 0x80000000u) == 0u) ok = barrier_wait(gb, old, fault);
-            else __threadfence();
+            const long long limit = fault.polls > 0 ? fault.polls : kSpinLimit;
+            long long it = 0;
+            while ((((old + inc) ^ old) & 0x80000000u) == 0u) {  // unless it completed the barrier
+                const unsigned long long we = ld_acquire_pair(gb);
+                if ((unsigned int)(we >> 32) != 0u) ok = 0;  // gb->err
+                if (!ok || (((unsigned int)we ^ old) & 0x80000000u) != 0u) break;
+                if (++it > limit) {
+                    atomicExch(&gb->err, 1);
+                    ok = 0;
+                    break;
+                }
+            }
         }
         ok_s = ok;
     }
@@ -702,19 +723,17 @@ RECON_DEV bool worker_barrier(GridBar* gb, const CoopFault& fault, unsigned int 
 
 // Number of eigenvalues of the tridiagonal (a_k, b_k = beta_{k-1}^2) below x: the sign changes of its
 // characteristic polynomials p_k = (a_k - x) p_{k-1} - b_k p_{k-2}, rescaled by exact powers of two
-// when the exponent drifts (two dependent FP64 operations per step instead of a reciprocal).
+// when the exponent drifts. Three FP64 operations per step; signs and exponents are read as integers
+// (a zero may count with either sign: the polynomials around it have opposite signs).
 RECON_DEV int sturm_count(const double* a, const double* b, int m, double x) {
     double p0 = 1.0, p1 = a[0] - x;
-    if (p1 == 0.0) p1 = -1e-300;
-    int cnt = p1 < 0.0;
+    int cnt = (unsigned int)__double2hiint(p1) >> 31;
     for (int k = 1; k < m; ++k) {
-        double p2 = fma(-b[k], p0, (a[k] - x) * p1);
-        if (p2 == 0.0) p2 = p1 < 0.0 ? 1e-300 : -1e-300;  // a zero counts as a change
-        cnt += (p2 < 0.0) != (p1 < 0.0);
+        const double p2 = fma(-b[k], p0, (a[k] - x) * p1);
+        cnt += (unsigned int)(__double2hiint(p2) ^ __double2hiint(p1)) >> 31;
         p0 = p1;
         p1 = p2;
-        const int ex = max((int)((__double_as_longlong(p0) >> 52) & 0x7ff),
-                           (int)((__double_as_longlong(p1) >> 52) & 0x7ff));
+        const int ex = max((__double2hiint(p0) >> 20) & 0x7ff, (__double2hiint(p1) >> 20) & 0x7ff);
         if (ex > 1023 + 480 || ex < 1023 - 480) {  // keep the larger one near 1
             const double sc = __longlong_as_double((long long)(2046 - ex) << 52);
             p0 *= sc;
@@ -725,46 +744,59 @@ RECON_DEV int sturm_count(const double* a, const double* b, int m, double x) {
 }
 
 // Largest eigenvalue of the m x m tridiagonal in shared memory, by the whole CTA (uniform control
-// flow): multisection with one sample per thread. Without an earlier value (prev <= 0) from the
-// Gershgorin bounds, in FP32 down to 1e-4 relative (FP32 counts are exact for x farther than
-// ~m eps32 |T| from an eigenvalue) and FP64 from there; with one, which the eigenvalue cannot lie
-// below, from samples prev (1 + 2^-51 .. 2^-1.5) spread over the exponents.
-RECON_DEV double tri_max(const double* a, const double* b, int m, double prev) {
+// flow): multisection with one sample per thread (kLancThreads of them), a bounded number of rounds.
+// Without an earlier value (prev <= 0) from the Gershgorin bounds, in FP32 down to 1e-4 relative (FP32
+// counts are exact for x farther than ~m eps32 |T| from an eigenvalue) and fine_max rounds of FP64; with
+// one, which the eigenvalue cannot lie below, a round of samples prev (1 + 2^-51 .. 2^-1.5) spread over
+// the exponents and two more, which leaves 2e-5 of the growth over prev: all of it once that is below
+// 1e-11 of the value, as it is before the end (fine_max = 2 rounds; more of them for a value that no
+// check comes after). Returns the middle of the bracket, *lower: its lower end.
+RECON_DEV double tri_max(const double* a, const double* b, int m, double prev, int fine_max,
+                         double* lower) {
     __shared__ double sh_lo, sh_hi;
     __shared__ int best;
-    const int t = threadIdx.x, nthr = blockDim.x;
+    const int t = threadIdx.x;
+    const double frac = (t + 1) * (1.0 / (kLancThreads + 1));
     __syncthreads();  // a, b; the results of an earlier call are read
-    if (t == 0) {
-        double lo = 1e300, hi = -1e300;
-        for (int k = 0; k < m; ++k) {
-            // FP32 square roots, rounded up: only the bounds of the search
-            const double r = 1.000001 * ((k > 0 ? (double)sqrtf((float)b[k]) : 0.0) +
-                                         (k + 1 < m ? (double)sqrtf((float)b[k + 1]) : 0.0));
-            lo = fmin(lo, a[k] - r);
-            hi = fmax(hi, a[k] + r);
+    if (t < 32) {
+        float lo = 3e38f, hi = -3e38f;  // FP32 bounds, widened beyond its rounding
+        for (int k = t; k < m; k += 32) {
+            const float r = (k > 0 ? sqrtf((float)b[k]) : 0.f) + (k + 1 < m ? sqrtf((float)b[k + 1]) : 0.f);
+            lo = fminf(lo, (float)a[k] - r);
+            hi = fmaxf(hi, (float)a[k] + r);
         }
-        const double pad = 1e-6 * fmax(fabs(lo), fabs(hi));
-        sh_lo = prev > 0.0 ? prev : lo - pad;
-        sh_hi = hi + pad;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+            hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        }
+        if (t == 0) {
+            const double pad = 1e-5 * (double)fmaxf(fabsf(lo), fabsf(hi));
+            sh_lo = prev > 0.0 ? prev : lo - pad;
+            sh_hi = hi + pad;
+            best = -1;
+        }
     }
-    if (t == 0) best = -1;
     __syncthreads();
     if (prev > 0.0) {
         const double x = fma(prev, (double)exp2f(-51.f + 0.39f * (float)t), prev);
         if (sturm_count(a, b, m, x) < m) atomicMax(&best, t);
         __syncthreads();
         const int bt = best;
-        if (bt < 0) return prev;  // within 2^-51 of it
+        if (bt < 0) {  // within 2^-51 of it
+            *lower = prev;
+            return prev;
+        }
         __syncthreads();
         if (t == bt) sh_lo = x;
         if (t == bt + 1) sh_hi = fmin(sh_hi, x);
     }
-    for (int round = 0; round < 24; ++round) {
+    for (int round = 0, fine = 0; round < 16 && fine < fine_max; ++round) {
         __syncthreads();
-        const double lo = sh_lo, hi = sh_hi;
-        if (hi - lo <= 2e-16 * fabs(hi)) break;
-        const bool fp32 = (hi - lo) > 1e-4 * fabs(hi);
-        const double x = lo + (hi - lo) * (t + 1) / (double)(nthr + 1);
+        const double lo = sh_lo, hi = sh_hi, w = hi - lo;
+        if (w <= 2e-16 * fabs(hi)) break;
+        const bool fp32 = w > 1e-4 * fabs(hi) && prev <= 0.0;
+        const double x = fma(w, frac, lo);
         int cnt = 0;
         if (fp32) {
             const float xf = (float)x;
@@ -776,6 +808,7 @@ RECON_DEV double tri_max(const double* a, const double* b, int m, double prev) {
             }
         } else {
             cnt = sturm_count(a, b, m, x);
+            ++fine;
         }
         // the largest eigenvalue lies above the largest sample x with cnt < m
         if (t == 0) best = -1;
@@ -783,14 +816,15 @@ RECON_DEV double tri_max(const double* a, const double* b, int m, double prev) {
         if (cnt < m) atomicMax(&best, t);
         __syncthreads();
         if (t == 0) {
-            const double step = (hi - lo) / (double)(nthr + 1);
-            const double nlo = lo + step * (best + 1);
+            const double step = w * (1.0 / (kLancThreads + 1));
+            const double nlo = fma(step, (double)(best + 1), lo);
             // FP32 counts near the root may be off by rounding: keep one step of margin
             sh_lo = fp32 ? fmax(lo, nlo - step) : nlo;
-            sh_hi = fp32 ? fmin(hi, nlo + 2 * step) : nlo + step;
+            sh_hi = fp32 ? fmin(hi, nlo + 2 * step) : fmin(hi, nlo + step);
         }
     }
     __syncthreads();
+    *lower = sh_lo;
     return 0.5 * (sh_lo + sh_hi);
 }
 
@@ -801,9 +835,10 @@ RECON_DEV void lanczos_check(const LancMat& L, GridBar* gb, const CoopFault& fau
     __shared__ double sa[kLanczosMax], sb[kLanczosMax];
     __shared__ unsigned int sh_seen;
     __shared__ int sh_ok, sh_bad;
-    double theta = 0.0;
+    double theta = 0.0, lower = 0.0;
     bool stands = false;
-    for (unsigned int next = 8;; next += 4) {
+    int scale = 0;
+    for (unsigned int next = 8;; next += 2) {
         // the steps up to the next check, or all there are: never more, so that the value does not
         // depend on how far the workers have got meanwhile
         if (threadIdx.x == 0) {
@@ -819,17 +854,23 @@ RECON_DEV void lanczos_check(const LancMat& L, GridBar* gb, const CoopFault& fau
         if (stands) break;  // the workers have left as well
         const bool fin = sh_seen >= kLancFin && sh_seen - kLancFin <= next;
         const int m = (int)(fin ? sh_seen - kLancFin : next);
+        // in units of 2^scale ~ alpha_0 (exact), so that FP32 holds any matrix
+        const double a0 = m > 0 ? __ldcg(L.ab) : 0.0;
+        scale = a0 != 0.0 && isfinite(a0) ? exponent_of(fabs(a0)) : 0;
         for (int k = threadIdx.x; k < m; k += blockDim.x) {
-            sa[k] = __ldcg(L.ab + 2 * k);
-            sb[k] = __ldcg(L.ab + 2 * k + 1);
-            if (!isfinite(sa[k]) || !isfinite(sb[k])) sh_bad = 1;
+            const double av = __ldcg(L.ab + 2 * k), bv = __ldcg(L.ab + 2 * k + 1);
+            if (!isfinite(av) || !isfinite(bv)) sh_bad = 1;
+            sa[k] = scale2(av, -scale);
+            sb[k] = scale2(bv, -2 * scale);
         }
         __syncthreads();
         // a matrix that is not finite: reported as such by the value
+        double lo = 0.0;
         const double th = (m < 1 || sh_bad) ? __longlong_as_double(0x7ff8000000000000LL)
-                                            : tri_max(sa, sb, m, theta);
-        stands = theta > 0.0 && th <= theta * (1.0 + 1e-15);
+                                            : tri_max(sa, sb, m, lower, fin ? 10 : 2, &lo);
+        stands = lower > 0.0 && th <= lower * (1.0 + 5e-16);
         theta = th;
+        lower = lo;
         __syncthreads();
         if (fin) break;
         if (stands && threadIdx.x == 0)
@@ -838,7 +879,7 @@ RECON_DEV void lanczos_check(const LancMat& L, GridBar* gb, const CoopFault& fau
     if (threadIdx.x == 0) {
         gb->pad[0] = 0u;
         gb->pad[1] = 0u;
-        L.lmax_out[0] = theta;
+        L.lmax_out[0] = scale2(theta, scale);
         if (L.err_out) *L.err_out = 0;
     }
 }
@@ -928,12 +969,11 @@ lanczos_kernel(LancMat L, GridBar* gb, CoopFault fault) {
         a = __shfl_sync(0xffffffffu, t, 0);
         n = __shfl_sync(0xffffffffu, t, 4);
         if (!(n > 0.0)) break;  // an exhausted Krylov space, or a value that is not finite
-        const double rn = rcp_nr(n);
+        const double rn = rcp_pivot(n);
         const double alpha = a * rn, ratio = n * rn_prev;
-        const double b2 = ratio * pow2i(2 * e_prev), gamma = ratio * pow2i(e_prev);
         if (blockIdx.x == 0 && tid == 0) {
             L.ab[2 * k] = alpha;
-            L.ab[2 * k + 1] = b2;
+            L.ab[2 * k + 1] = ratio * pow2i(2 * e_prev);
             asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&gb->pad[0]),
                          "r"((unsigned int)(k + 1)) : "memory");
         }
@@ -941,14 +981,16 @@ lanczos_kernel(LancMat L, GridBar* gb, CoopFault fault) {
             ++k;
             break;
         }
-        // the next vector's norm near 1: beta changes little from step to step
-        int e = exponent_of(n) / 2 + (b2 > 0.0 ? exponent_of(b2) / 2 : alpha != 0.0 ? exponent_of(fabs(alpha)) : 0);
+        // the next vector's norm near 1: beta changes little from step to step (exponents of n_k and of
+        // beta_{k-1}^2 = ratio 4^e_prev, halved); the scale goes into the exponents of w and of the factors
+        int e = exponent_of(n) / 2 +
+                (k > 0 ? exponent_of(ratio) / 2 + e_prev : alpha != 0.0 ? exponent_of(fabs(alpha)) : 0);
         e = min(max(e, -400), 400);
-        const double sc = pow2i(-e);
+        const double ca = -scale2(alpha, -e), cg = -scale2(ratio, e_prev - e);
         for (int i = tid; i < s; i += kLancThreads) {
             const double2 wi = __ldcg(w + i), qi = q[i], pi = p[i];
-            p[i] = make_double2(sc * fma(-gamma, pi.x, fma(-alpha, qi.x, wi.x)),
-                                sc * fma(-gamma, pi.y, fma(-alpha, qi.y, wi.y)));
+            p[i] = make_double2(fma(cg, pi.x, fma(ca, qi.x, scale2(wi.x, -e))),
+                                fma(cg, pi.y, fma(ca, qi.y, scale2(wi.y, -e))));
         }
         double2* sw = q;
         q = p;
