@@ -12,9 +12,10 @@
 //                     accumulation carries the rounding errors of its additions in a second
 //                     float, through the window sums, the DFT terms and the warp tree, and the
 //                     pair becomes one FP64 value);
-//   gram_fill_kernel: one warp per lag: the length-P direction sum_r1 Y[pair][d2][r1] w_P^(d1 r1)
-//                     in FP64 (fixed order, deterministic), then the lag scattered over the
-//                     (l, l') pairs it fills in G (column-major s x s complex128, both triangles).
+//   gram_fill_kernel: one warp per lag pair (d1, -d1): the length-P direction
+//                     sum_r1 Y[pair][d2][r1] w_P^(d1 r1) in FP64 (fixed order, deterministic), then
+//                     the lags scattered over the (l, l') pairs they fill in G (column-major s x s
+//                     complex128, both triangles).
 // Volumes (depth R, N3 depth taps; lag_ab[d] also carries w_R^(d3 r3)): the row kernel runs over
 // the R * P rows unchanged, then the length-P and length-R directions are separated:
 //   gram_depth_kernel: Z[pair][d2][d1][r3] = sum_r1 Y[pair][d2][r3 P + r1] w_P^(d1 r1)  (FP64);
@@ -33,13 +34,16 @@ __host__ __device__ constexpr int row_threads(int M) { return M >= 5 ? 256 : 512
 
 // kLo = false (only where the low parts do not fit in shared memory: M = 6 with 512-point rows
 // and more than 12 frames): each window sum is rounded once to FP32 (hi + lo) before the DFT,
-// whose terms and tree stay compensated. tab: the twiddles of every output lag d2 are laid out
+// whose terms and tree stay compensated. kTab: the twiddles of every output lag d2 are laid out
 // contiguously in c ([L2][Q], built once per CTA), so that the lanes of a warp read consecutive
 // entries; otherwise lane c reads w^(d2 c mod Q) from the length-Q table (bank conflicts for
-// even d2). The same values either way.
-template <int M, bool kLo>
+// even d2). The same values either way. kReal: a frame's product with itself is |x|^2, taken as real (the
+// general product leaves the rounding of re im - im re in its imaginary part), and its Y(-d2) is the
+// conjugate of Y(d2): a quarter of the products and of the DFT outputs less at M = 3, and these bound
+// the kernel (29.7 -> 21.4 us at 256x256x16, 9x9x3, with the staging and the table free of divisions).
+template <int M, bool kLo, bool kReal, bool kTab>
 __global__ void __launch_bounds__(row_threads(M))
-gram_rows_kernel(const float2* __restrict__ x, int T, int P, int Q, int N2, int circ, int tab,
+gram_rows_kernel(const float2* __restrict__ x, int T, int P, int Q, int N2, int circ,
                  const float2* __restrict__ twQ, double2* __restrict__ Y) {
     constexpr int NP = M * (M + 1) / 2;
     extern __shared__ float2 sm[];
@@ -49,19 +53,22 @@ gram_rows_kernel(const float2* __restrict__ x, int T, int P, int Q, int N2, int 
     float2* qp = xs + (size_t)T * Q;         // [NP][Q] pair products (compensated sum, high part)
     float2* ql = qp + (size_t)NP * Q;        // [NP][Q] their low parts (kLo)
     float2* tw = ql + (kLo ? (size_t)NP * Q : 0);  // [Q]
-    float2* dtab = tw + Q;                   // [L2][Q] (tab)
+    float2* dtab = tw + Q;                   // [L2][Q] (kTab)
     const int r1 = blockIdx.x;
     for (int i = threadIdx.x; i < Q; i += blockDim.x) tw[i] = twQ[i];
-    for (int e = threadIdx.x; e < T * Q; e += blockDim.x) {
-        const int n = e / Q, c = e % Q;
-        xs[e] = x[((size_t)n * P + r1) * Q + c];
-    }
+    // (no divisions: they took as long as the products)
+    for (int n = threadIdx.x >> 5; n < T; n += row_threads(M) / 32)
+        for (int c = threadIdx.x & 31; c < Q; c += 32) xs[n * Q + c] = x[((size_t)n * P + r1) * Q + c];
     __syncthreads();
-    if (tab) {  // from the shared copy of the table (no further global loads)
-        for (int e = threadIdx.x; e < L2 * Q; e += blockDim.x) {
-            const int i2 = e / Q, c = e % Q;
-            const int d2m = (i2 - (N2 - 1) + Q) % Q;
-            dtab[e] = tw[(d2m * c) % Q];  // d2m, c < Q <= 512: no overflow in 32 bits
+    if constexpr (kTab) {  // from the shared copy of the table (no further global loads)
+        const int d2m0 = (Q - (N2 - 1) % Q) % Q;  // (-(N2 - 1)) mod Q; d2m0, c < Q <= 512
+        for (int c = threadIdx.x; c < Q; c += blockDim.x) {
+            int ti = (d2m0 * c) % Q;
+            for (int i2 = 0; i2 < L2; ++i2) {
+                dtab[i2 * Q + c] = tw[ti];
+                ti += c;
+                if (ti >= Q) ti -= Q;
+            }
         }
     }
     // q_ab(c) = sum_j conj(x_{j+M-1-a}(c)) x_{j+M-1-b}(c): window w[m] = x_{j+M-1-m}(c)
@@ -80,7 +87,7 @@ gram_rows_kernel(const float2* __restrict__ x, int T, int P, int Q, int N2, int 
                 for (int b = a; b < M; ++b, ++e) {
                     const float2 t = cmulcj(w[a], w[b]);
                     comp_add(acc[e].x, lo[e].x, t.x);
-                    comp_add(acc[e].y, lo[e].y, t.y);
+                    if (!kReal || a != b) comp_add(acc[e].y, lo[e].y, t.y);
                 }
 #pragma unroll
             for (int m = M - 1; m > 0; --m) w[m] = w[m - 1];
@@ -99,9 +106,25 @@ gram_rows_kernel(const float2* __restrict__ x, int T, int P, int Q, int N2, int 
     // Y[pair][d2] = sum_c q[pair][c] w_Q^(d2 c); one warp per output, lanes stride c, each term
     // (hi + lo) w added to a compensated (hi, lo) pair, then a TwoSum shuffle tree
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nout = NP * L2;
+    // kReal: the pairs a < b with every d2 first, then the frames with themselves, d2 >= 0
+    constexpr int NC = NP - M;
+    const int nout = kReal ? NC * L2 + M * N2 : NP * L2;
     for (int o = warp; o < nout; o += row_threads(M) / 32) {
-        const int pr = o / L2, i2 = o % L2;
+        int pr = o / L2, i2 = o % L2;
+        bool self = false;
+        if (kReal) {
+            int a = 0;
+            if (o < NC * L2) {  // the pr-th pair a < b
+                int k = pr;
+                while (k >= M - 1 - a) { k -= M - 1 - a; ++a; }
+                pr = a * (2 * M - a + 1) / 2 + 1 + k;
+            } else {
+                self = true;
+                a = (o - NC * L2) / N2;
+                i2 = N2 - 1 + (o - NC * L2) % N2;
+                pr = a * (2 * M - a + 1) / 2;
+            }
+        }
         const int d2m = (i2 - (N2 - 1) + Q) % Q;
         const float2* qrow = qp + (size_t)pr * Q;
         const float2* qlow = ql + (size_t)pr * Q;
@@ -109,8 +132,25 @@ gram_rows_kernel(const float2* __restrict__ x, int T, int P, int Q, int N2, int 
         int idx = (d2m * lane) % Q;
         const int step = (d2m * 32) % Q;
         float2 y = make_float2(0.f, 0.f), yl = make_float2(0.f, 0.f);
-        for (int c = lane; c < Q; c += 32) {
-            const float2 wt = tab ? trow[c] : tw[idx];
+        if (kReal && self) {
+#pragma unroll 4
+            for (int c = lane; c < Q; c += 32) {
+                const float2 wt = kTab ? trow[c] : tw[idx];
+                const float q = qrow[c].x;
+                comp_add(y.x, yl.x, __fmul_rn(q, wt.x));
+                comp_add(y.y, yl.y, __fmul_rn(q, wt.y));
+                if (kLo) {
+                    const float l = qlow[c].x;
+                    yl.x = __fadd_rn(yl.x, __fmul_rn(l, wt.x));
+                    yl.y = __fadd_rn(yl.y, __fmul_rn(l, wt.y));
+                }
+                idx += step;
+                if (idx >= Q) idx -= Q;
+            }
+        }
+#pragma unroll 4
+        for (int c = kReal && self ? Q : lane; c < Q; c += 32) {
+            const float2 wt = kTab ? trow[c] : tw[idx];
             const float2 t = cmul(qrow[c], wt);
             comp_add(y.x, yl.x, t.x);
             comp_add(y.y, yl.y, t.y);
@@ -122,21 +162,28 @@ gram_rows_kernel(const float2* __restrict__ x, int T, int P, int Q, int N2, int 
             idx += step;
             if (idx >= Q) idx -= Q;
         }
+        // both components in one tree: lanes 0-15 take the real part, 16-31 the imaginary one
+        const bool up = lane & 16;
+        float h = up ? y.y : y.x, l = up ? yl.y : yl.x;
+        float oh = __shfl_xor_sync(0xffffffffu, up ? y.x : y.y, 16);
+        float ol = __shfl_xor_sync(0xffffffffu, up ? yl.x : yl.y, 16);
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const float hx = __shfl_xor_sync(0xffffffffu, y.x, off);
-            const float lx = __shfl_xor_sync(0xffffffffu, yl.x, off);
-            const float hy = __shfl_xor_sync(0xffffffffu, y.y, off);
-            const float ly = __shfl_xor_sync(0xffffffffu, yl.y, off);
-            float sx, ex, sy, ey;
-            two_sum(y.x, hx, sx, ex);
-            two_sum(y.y, hy, sy, ey);
-            y = make_float2(sx, sy);
-            yl.x = __fadd_rn(__fadd_rn(yl.x, lx), ex);
-            yl.y = __fadd_rn(__fadd_rn(yl.y, ly), ey);
+        for (int off = 8;; off >>= 1) {
+            float sm_, er;
+            two_sum(h, oh, sm_, er);
+            h = sm_;
+            l = __fadd_rn(__fadd_rn(l, ol), er);
+            if (off == 0) break;
+            oh = __shfl_xor_sync(0xffffffffu, h, off);
+            ol = __shfl_xor_sync(0xffffffffu, l, off);
         }
-        if (lane == 0)
-            Y[(size_t)o * P + r1] = make_double2((double)y.x + (double)yl.x, (double)y.y + (double)yl.y);
+        oh = __shfl_sync(0xffffffffu, h, 16);
+        ol = __shfl_sync(0xffffffffu, l, 16);
+        if (lane == 0) {
+            const double2 z = make_double2((double)h + (double)l, (double)oh + (double)ol);
+            Y[((size_t)pr * L2 + i2) * P + r1] = z;
+            if (kReal && self) Y[((size_t)pr * L2 + (L2 - 1 - i2)) * P + r1] = zconj(z);
+        }
     }
 }
 
@@ -177,6 +224,83 @@ __global__ void gram_fill_kernel(const double2* __restrict__ Y, int P, int N1, i
     for (int t = lane; t < cnt; t += 32) {
         const int lp1 = lo1 + t / n2, lp2 = lo2 + t % n2;
         const int l1 = lp1 + d1, l2 = lp2 + d2;
+        const size_t i = ((size_t)a * N1 + l1) * N2 + l2;
+        const size_t j = ((size_t)b * N1 + lp1) * N2 + lp2;
+        G[i + j * s] = v;
+        if (i != j) G[j + i * s] = zconj(v);
+    }
+}
+
+// The same with one warp per (pair, d1 >= 0, d2) for d1 and -d1 together (kReal series), rows r1 and
+// P - r1 folded: with U = Y_r1 + Y_{P-r1} and V = Y_r1 - Y_{P-r1}, lag(+-d1) = sum U cos -+ i sum V sin (about
+// a third of the FP64 operations of one warp per lag, on
+// a pipe that issues one per 64 cycles and scheduler: 9.2 -> 7.1 us at 256x256x16, 9x9x3), lanes over
+// r1 in a fixed order, then a fixed shuffle tree; then both lags scattered over the (l, l') pairs of G.
+__global__ void gram_fill_pair_kernel(const double2* __restrict__ Y, int P, int N1, int N2, int M,
+                                 const double2* __restrict__ twPd, double2* __restrict__ lags,
+                                 double2* __restrict__ G) {
+    const int L1 = 2 * N1 - 1, L2 = 2 * N2 - 1, npair = M * (M + 1) / 2;
+    const int s = N1 * N2 * M;
+    const int o = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (o >= npair * N1 * L2) return;
+    const int pr = o / (N1 * L2), rem = o % (N1 * L2);
+    const int d1 = rem / L2, i2 = rem % L2, d2 = i2 - (N2 - 1);
+    int a = 0, e = pr;
+    while (e >= M - a) { e -= M - a; ++a; }
+    const int b = a + e;
+    // a frame with itself: lag_aa[-d] = conj(lag_aa[d]) exactly, so the lag in the non-negative half
+    // (d1 > 0, or d1 = 0 and d2 >= 0) gives both and G is exactly Hermitian
+    const bool self = a == b;
+    if (self && d1 == 0 && d2 < 0) return;
+    const double2* yrow = Y + ((size_t)pr * L2 + i2) * P;
+    const int H = P / 2;
+    double2 E = make_double2(0.0, 0.0), O = E;
+#pragma unroll 4
+    for (int r1 = lane; r1 < H; r1 += 32) {
+        const double2 w = twPd[(d1 * r1) % P];  // cos, -sin
+        double2 u = yrow[r1];
+        if (r1) {
+            const double2 v = yrow[P - r1];
+            O.x = fma(u.x - v.x, -w.y, O.x);
+            O.y = fma(u.y - v.y, -w.y, O.y);
+            u = zadd(u, v);
+        }
+        E.x = fma(u.x, w.x, E.x);
+        E.y = fma(u.y, w.x, E.y);
+    }
+    if (lane == 0) {  // row P / 2
+        const double2 u = yrow[H];
+        E = (d1 & 1) ? make_double2(E.x - u.x, E.y - u.y) : zadd(E, u);
+    }
+    // the four sums in one tree: lane 8 k returns sum k of (E.x, E.y, O.x, O.y)
+    const bool up = lane & 16, up8 = lane & 8;
+    double p0 = up ? O.x : E.x, p1 = up ? O.y : E.y;
+    p0 += __shfl_xor_sync(0xffffffffu, up ? E.x : O.x, 16);
+    p1 += __shfl_xor_sync(0xffffffffu, up ? E.y : O.y, 16);
+    double z = up8 ? p1 : p0;
+    z += __shfl_xor_sync(0xffffffffu, up8 ? p0 : p1, 8);
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) z += __shfl_xor_sync(0xffffffffu, z, off);
+    E = make_double2(__shfl_sync(0xffffffffu, z, 0), __shfl_sync(0xffffffffu, z, 8));
+    O = make_double2(__shfl_sync(0xffffffffu, z, 16), __shfl_sync(0xffffffffu, z, 24));
+    // lag(+-d1) = E -+ i O; lanes 0-15 scatter d1, lanes 16-31 -d1 (a frame with itself: d1 alone)
+    const bool neg = up && !self;
+    double2 v = neg ? make_double2(E.x - O.y, E.y + O.x) : make_double2(E.x + O.y, E.y - O.x);
+    if (d1 == 0) v = E;
+    if (self && d1 == 0 && d2 == 0) v.y = 0.0;  // sum of |x|^2
+    const int e1 = neg ? -d1 : d1;
+    if (lags && (lane == 0 || (lane == 16 && neg && d1))) {
+        double2* lp = lags + (size_t)pr * L1 * L2;
+        lp[(size_t)(e1 + N1 - 1) * L2 + i2] = v;
+        if (self) lp[(size_t)(N1 - 1 - d1) * L2 + (L2 - 1 - i2)] = zconj(v);
+    }
+    const int lo1 = max(0, -e1), hi1 = min(N1, N1 - e1);
+    const int lo2 = max(0, -d2), hi2 = min(N2, N2 - d2);
+    const int n2 = hi2 - lo2, cnt = (hi1 - lo1) * n2;
+    const bool halves = !self && d1 != 0;  // 16 lanes per lag, else all 32
+    for (int t = halves ? (lane & 15) : lane; t < cnt; t += halves ? 16 : 32) {
+        const int lp1 = lo1 + t / n2, lp2 = lo2 + t % n2;
+        const int l1 = lp1 + e1, l2 = lp2 + d2;
         const size_t i = ((size_t)a * N1 + l1) * N2 + l2;
         const size_t j = ((size_t)b * N1 + lp1) * N2 + lp2;
         G[i + j * s] = v;
@@ -265,6 +389,10 @@ void gram_cfg(const Dims& d, bool* lo, bool* tab) {
     *tab = gram_smem_cfg(d, *lo, true) <= kGramSmemMax;
 }
 
+// Image series with rows of 64 and more elements: kReal (see gram_rows_kernel). Shorter rows are
+// latency-bound either way, and volumes keep the last bits (their solves amplify those of S).
+bool gram_real(const Dims& d) { return d.R == 1 && d.Q >= 64; }
+
 }  // namespace
 
 size_t gram_smem(const Dims& d) {
@@ -292,11 +420,16 @@ cudaError_t launch_gram(const Dims& d, const Twiddles& tw, const float2* x, doub
     gram_cfg(d, &lo, &tab);
 #define CASE(MM)                                                                                 \
     case MM: {                                                                                   \
-        auto k = lo ? gram_rows_kernel<MM, true> : gram_rows_kernel<MM, false>;                  \
+        auto k = !lo ? (tab ? gram_rows_kernel<MM, false, false, true>                           \
+                            : gram_rows_kernel<MM, false, false, false>)                         \
+                 : gram_real(d) ? (tab ? gram_rows_kernel<MM, true, true, true>                  \
+                                       : gram_rows_kernel<MM, true, true, false>)                \
+                                : (tab ? gram_rows_kernel<MM, true, false, true>                 \
+                                       : gram_rows_kernel<MM, true, false, false>);              \
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
                                              (int)smem);                                         \
         if (e != cudaSuccess) return e;                                                          \
-        k<<<d.rows(), row_threads(MM), smem, st>>>(x, d.T, d.rows(), d.Q, d.N2, d.circ, (int)tab,\
+        k<<<d.rows(), row_threads(MM), smem, st>>>(x, d.T, d.rows(), d.Q, d.N2, d.circ,           \
                                                tw.twQ, lag_part);                                \
         break;                                                                                   \
     }
@@ -317,6 +450,11 @@ cudaError_t launch_gram(const Dims& d, const Twiddles& tw, const float2* x, doub
         const int nlag3 = (int)d.nlag();
         gram_fill3_kernel<<<(nlag3 + 7) / 8, 256, 0, st>>>(Z, d.R, d.N1, d.N2, d.N3, d.M, tw.twRd,
                                                            lags, G);
+        return cudaGetLastError();
+    }
+    if (gram_real(d)) {
+        const int n = d.npair() * d.N1 * d.L2();
+        gram_fill_pair_kernel<<<(n + 7) / 8, 256, 0, st>>>(lag_part, d.P, d.N1, d.N2, d.M, tw.twPd, lags, G);
         return cudaGetLastError();
     }
     const int nlag = d.npair() * d.L1() * d.L2();

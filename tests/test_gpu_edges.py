@@ -25,11 +25,11 @@ def _spectrum(kind, s, rng):
         X = rng.standard_normal((20 * s, s)) + 1j * rng.standard_normal((20 * s, s))
         return X.conj().T @ X
     U = np.linalg.qr(rng.standard_normal((s, s)) + 1j * rng.standard_normal((s, s)))[0]
-    lam = np.logspace(0, -8, s) if kind == "decades" else np.where(np.arange(s) < 1, 1.0, 1e-3)
-    return 1e6 * (U * lam) @ U.conj().T
+    lam = np.where(np.arange(s) < 1, 1.0, 1e-3) if kind == "one" else np.logspace(0, -8, s)
+    return {"large": 1e60, "small": 1e-60}.get(kind, 1e6) * (U * lam) @ U.conj().T
 
 
-@pytest.mark.parametrize("kind", ["random", "decades", "one"])
+@pytest.mark.parametrize("kind", ["random", "decades", "one", "large", "small"])
 @pytest.mark.parametrize("filt", [(1, 1, 1), (2, 1, 1), (5, 1, 1), (7, 3, 1), (4, 8, 2), (5, 5, 3),
                                   (9, 9, 3), (7, 15, 3), (9, 9, 6)])
 def test_lambda_max(R, filt, kind):
@@ -264,3 +264,29 @@ def test_operators_at_run_edges(R, T, P, Q, M):
     b = _series(rng, 3, T, P, Q)
     recon.recon_adjoint_coils(ctx.h, to_dev(b), to_dev(m), to_dev(C), y)
     assert_close(y.cpu().numpy(), sum(c.conj() * np.fft.ifft2(m * v, norm="ortho") for c, v in zip(C, b)), 2e-6)
+
+
+@pytest.mark.parametrize("T,P,Q,N1,N2,M", [(2, 16, 64, 1, 1, 2), (3, 64, 192, 4, 9, 3), (16, 32, 256, 9, 2, 1),
+                                           (5, 512, 64, 3, 40, 2), (13, 16, 512, 2, 5, 5), (16, 16, 512, 3, 3, 6),
+                                           (9, 192, 32, 16, 3, 3), (4, 16, 128, 16, 1, 4)])
+def test_gram_row_lengths(R, T, P, Q, N1, N2, M):
+    """G and its lags over row lengths on both sides of the real-product variant, one to many lags on
+    either axis, no shared twiddle rows (40 taps of 64) and the two largest filters: FP32 products of the
+    FP32 series with compensated sums, so at most the rounding of a product (2 x 2^-24); G exactly
+    Hermitian."""
+    import torch
+    from oracle import slr
+    recon, ctx = R
+    rng = np.random.default_rng(T * P + Q)
+    x = _series(rng, T, P, Q)
+    s, npair = N1 * N2 * M, M * (M + 1) // 2
+    G = torch.empty((s, s), dtype=torch.complex128, device="cuda")
+    lags = torch.empty((npair, 2 * N1 - 1, 2 * N2 - 1), dtype=torch.complex128, device="cuda")
+    recon.recon_gram(ctx.h, to_dev(x), (N1, N2, M), G, lags)
+    Gn = G.cpu().numpy().T
+    assert_close(Gn, slr.gram_fft(x.astype(np.complex128), N1, N2, M), 2.0 ** -23)
+    assert np.array_equal(Gn, Gn.conj().T)
+    ln = lags.cpu().numpy()
+    for a in range(M):
+        e = a * (2 * M - a + 1) // 2
+        assert np.array_equal(ln[e], ln[e, ::-1, ::-1].conj())
