@@ -58,49 +58,71 @@ RECON_DEV void s_diagonals(const float2 (&s)[M][M], float2 (&c)[2 * M - 1]) {
     }
 }
 
-// (W x)_n at one pixel, from the frame values xs[f * stride] (0 <= f < T), the block s and its
-// diagonal sums c: the diagonal form where all M windows of frame n exist (for 3 <= M <= 5,
-// where it saves products and the block and its sums fit the registers; the circular lifting
-// always), else the window sum.
-template <int M, bool CIRC>
-RECON_DEV float2 w_frame(const float2 (&s)[M][M], const float2 (&c)[2 * M - 1],
-                         const float2* xs, int stride, int n, int T, int k) {
-    float2 w = make_float2(0.f, 0.f);
-    if (CIRC || (M >= 3 && M <= 5 && n >= M - 1 && n < k)) {
+// Row transforms of pass C: kIn elements i + m kLanes of a row in u[m] on entry, element out_at(i, m) of
+// the result in u[m] on return; rows of 128 and 256 elements by the two-stage transforms of regfft.cuh
+// (16 elements a thread, one exchange), the others by the Stockham passes.
+template <int N>
+struct RowFft : RegFft<N> {
+    static constexpr int kIn = 8;
+    static constexpr bool kByWarp = false;
+    RECON_DEV static void fill(float2* tw, const float2* __restrict__ tw_g) {
+        for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = tw_g[i];
+    }
+    RECON_DEV static void inverse(float2 (&u)[RegFft<N>::kOut], float2* sx, const float2* tw, int i) {
+        RegFft<N>::template run<true, false>(u, sx, 1, tw, i);
+    }
+};
+template <int N>
+struct RowFft16 {
+    static constexpr int kLanes = N / 16, kIn = 16, kOut = 16;
+    static constexpr bool kByWarp = true;  // warps without a frame leave the transform out
+    RECON_DEV static void sync() { __syncwarp(); }
+};
+template <>
+struct RowFft<256> : RowFft16<256> {
+    static constexpr int kBuf = 16 * 17;
+    RECON_DEV static int out_at(int i, int m) { return i + 16 * m; }
+    RECON_DEV static int at(int e) { return e + (e >> 4); }
+    RECON_DEV static void fill(float2* tw, const float2* __restrict__ tw_g) { fill_tw256(tw, tw_g); }
+    RECON_DEV static void inverse(float2 (&u)[16], float2* sx, const float2* tw, int i) {
+        row_dft256<true>(u, sx, tw, i);
+    }
+};
+template <>
+struct RowFft<128> : RowFft16<128> {
+    static constexpr int kBuf = kX128;
+    RECON_DEV static int out_at(int i, int m) { return 2 * i + (m & 1) + 16 * (m >> 1); }
+    RECON_DEV static int at(int e) { return e + (e >> 3); }
+    RECON_DEV static void fill(float2* tw, const float2* __restrict__ tw_g) { fill_tw128(tw, tw_g); }
+    RECON_DEV static void inverse(float2 (&u)[16], float2* sx, const float2* tw, int i) {
+        float2 a[8], b[8];
+        row_dft128<true>(u, a, b, sx, tw, i);
 #pragma unroll
-        for (int d = 0; d < 2 * M - 1; ++d) {
-            const int f = n + d - (M - 1);
-            w = cfma(c[d], xs[(CIRC ? wrap_frame(f, T) : f) * stride], w);
+        for (int k = 0; k < 8; ++k) {
+            u[2 * k] = a[k];
+            u[2 * k + 1] = b[k];
         }
-        return w;
     }
-#pragma unroll
-    for (int a = 0; a < M; ++a) {
-        const int j = n - M + 1 + a;
-        if (j < 0 || j >= k) continue;
-#pragma unroll
-        for (int b = 0; b < M; ++b) w = cfma(s[a][b], xs[(n + a - b) * stride], w);
-    }
-    return w;
-}
+};
 
 // The W phase of pass C for frames [n0, n1) of one image row, by the whole CTA: res[n - n0][at(c)]
 // holds the transformed rows; q = res + lam W p goes to t, and Re (conj p) q of every element takes the
 // place of res.
 // A thread takes a column and a run of FC frames, whose p values and the M - 1 on either side it reads
 // straight from global memory into registers (each once per run; no copy of the p rows in shared
-// memory). kDiag: the diagonal form of w_frame where it applies.
+// memory). kDiag: the diagonal form where all M windows of a frame exist (for 3 <= M <= 5, where it saves
+// products and the block and its sums fit the registers; the circular lifting always).
 // The loads of a thread's first task (WLoads) are issued before the transform of the rows.
-template <int M>
+template <class F, int M>
+constexpr int kWRun = M > 4 ? 2 : (F::kIn > 8 ? 8 : 4);
+template <int M, int FC>
 struct WLoads {
-    static constexpr int FC = M <= 4 ? 4 : 2;
     float2 pw[FC + 2 * (M - 1)];    // p_{f0 - (M - 1) + i}
     float2 s[M * (M + 1) / 2];      // upper triangle of S(r)
 };
-template <int N, int M, bool CIRC>
-RECON_DEV void w_load(WLoads<M>& v, const float2* __restrict__ prow, const float2* __restrict__ Srow,
+template <int N, int M, int FC, bool CIRC>
+RECON_DEV void w_load(WLoads<M, FC>& v, const float2* __restrict__ prow, const float2* __restrict__ Srow,
                       int e, int T, int n0, int n1, size_t npix) {
-    constexpr int FC = WLoads<M>::FC;
     const int c = e % N, f0 = n0 + (e / N) * FC, f1 = min(n1, f0 + FC);
 #pragma unroll
     for (int i = 0; i < FC + 2 * (M - 1); ++i) {
@@ -113,16 +135,14 @@ RECON_DEV void w_load(WLoads<M>& v, const float2* __restrict__ prow, const float
     for (int i = 0; i < M * (M + 1) / 2; ++i) v.s[i] = Srow[(size_t)i * npix + c];
 }
 
-template <int N, int M, bool CIRC, bool kDiag>
-RECON_DEV void w_phase(WLoads<M>& v, float2* __restrict__ trow, const float2* __restrict__ prow,
+template <class F, int N, int M, int FC, bool CIRC, bool kDiag>
+RECON_DEV void w_phase(WLoads<M, FC>& v, float2* __restrict__ trow, const float2* __restrict__ prow,
                        const float2* __restrict__ Srow, float2* res, float lam, int T, int n0, int n1,
                        size_t npix) {
-    using F = RegFft<N>;
-    constexpr int FC = WLoads<M>::FC;
     const int k = CIRC ? T : T - M + 1;
     const int nrun = (n1 - n0 + FC - 1) / FC;
     for (int e = threadIdx.x; e < N * nrun; e += blockDim.x) {
-        if (e != (int)threadIdx.x) w_load<N, M, CIRC>(v, prow, Srow, e, T, n0, n1, npix);
+        if (e != (int)threadIdx.x) w_load<N, M, FC, CIRC>(v, prow, Srow, e, T, n0, n1, npix);
         const int c = e % N, f0 = n0 + (e / N) * FC, f1 = min(n1, f0 + FC);
         float2 s[M][M];
 #pragma unroll
@@ -166,9 +186,8 @@ RECON_DEV void w_phase(WLoads<M>& v, float2* __restrict__ trow, const float2* __
 // by FP32 warp trees: a warp's sum in its lane 0, FP64, zero elsewhere. Columns c and c + kThreads share
 // an accumulator, so that the sum is that of a CTA of kThreads threads, one column each, whatever the
 // launch shape (CG amplifies the last bits of Re <p, q> on the smallest series).
-template <int N>
+template <class F, int N>
 RECON_DEV double w_terms(const float2* res, int T) {
-    using F = RegFft<N>;
     const int nc = N < kThreads ? N : kThreads;
     double tot = 0.0;
     for (int c0 = 0; c0 < nc; c0 += blockDim.x) {
@@ -219,28 +238,36 @@ InvShape inv_shape(int T) {
 }
 
 // Pass C of a CG step. A CTA takes a run of `per` frames of an image row r1 (W reads the neighbouring
-// frames' p from global memory, so the runs are independent), N / 8 threads per frame: it
+// frames' p from global memory, so the runs are independent), kLanes threads per frame: it
 // inverse-transforms the k-space rows of t (giving A^H A p; the 1/(PQ) scale was applied with the mask;
 // elements in registers, exchange buffers that then hold the transformed rows), adds lam W p, writes q
 // over t and emits a partial of Re <p, q>. Rows of up to 32 elements keep all their frames in one CTA
-// and with it the order of that sum (see w_terms). 64x64x21 7.8 -> 4.4 us per launch, 192x192x24
-// 17.4 -> 9.6, 512x512x16 66.6 -> 32.3, against one CTA per row with passes over shared memory and
-// three copies of the row's frames there.
-constexpr int kRunThreads = 256;   // most threads of a CTA (512 for rows of up to 32 elements)
-constexpr int kRunUnits = 608;     // units wanted: four CTAs an SM
+// and with it the order of that sum (see w_terms). The pass is bound by latency for image series, by HBM
+// for volumes. 64x64x21 7.8 -> 4.4 us per launch, 192x192x24 17.4 -> 9.6, 512x512x16 66.6 -> 32.3,
+// against one CTA per row with passes over shared memory and three copies of the row's frames there.
+// Rows of 128 and 256 elements took such copies of p (and of t and S) too, with asynchronous staging
+// for volumes: without them and with W in runs of eight frames a volume of 128x128x64x12 (2 x 15 steps)
+// takes 10.5 instead of 11.2 ms, four 256x256x16 solves at once 16.6 instead of 17.9, a single one the
+// same 19.2, 15 steps at 512x128x12 508 instead of 548 us. Registers decide: 80 let two CTAs of 24
+// 256-point frames share an SM (at 128: 671 us for 15 steps at 256x256x24 instead of 633).
+constexpr int kRunThreads = 256;   // most threads of a CTA (512 for rows of up to 32 elements, 384 of 256)
 template <int N>
-__host__ __device__ constexpr int run_threads() { return N <= 32 ? 512 : kRunThreads; }
+__host__ __device__ constexpr int run_threads() { return N <= 32 ? 512 : (N == 256 ? 384 : kRunThreads); }
+// Units wanted: four CTAs an SM, two of the larger ones with 16 elements a thread (15 steps at
+// 256x256x16: 480 us, 515 with four).
+template <class F>
+constexpr int kRunUnits = F::kIn > 8 ? 304 : 608;
 struct RunShape {
     int nrun, per, threads, bufs;
 };
-template <int N>
+template <class F, int N>
 RunShape run_shape(int T, int rows) {
-    constexpr int L = RegFft<N>::kLanes;
+    constexpr int L = F::kLanes;
     RunShape v;
     int n = (T * L + run_threads<N>() - 1) / run_threads<N>();
     if (N > 32) {  // more, shorter runs (of four frames at least) until the units fill the chip
         // (rounded down: a few units more than fit at once would take a second round of their own)
-        const int fill = kRunUnits / rows, most = (T + 3) / 4;
+        const int fill = kRunUnits<F> / rows, most = (T + 3) / 4;
         if (n < fill) n = fill < most ? fill : (n > most ? n : most);
     }
     v.per = (T + n - 1) / n;
@@ -248,21 +275,23 @@ RunShape run_shape(int T, int rows) {
     v.threads = (v.per * L + 31) / 32 * 32;
     if (v.threads < 64) v.threads = 64;
     v.bufs = (v.threads + L - 1) / L;
+    // Rows of 128 and 256 elements: at least a thread per column for W (128x128x12, M = 3: 340 us for 15
+    // steps with 64 threads, 326 with 128); warps without a frame have no part in the transform.
+    if (F::kIn > 8 && v.threads < N) v.threads = N;
     return v;
 }
 
-template <int N, int M, bool CIRC>
-__global__ void __launch_bounds__(run_threads<N>(), N <= 32 || M > 4 ? 1 : 3)
+template <class F, int N, int M, bool CIRC>
+__global__ void __launch_bounds__(run_threads<N>(), N <= 32 || M > 4 ? 1 : (N == 256 ? 2 : 3))
 row_inv_w_kernel(float2* t, const float2* __restrict__ p, const float2* __restrict__ S,
                  float lam, int T, int P, int nrun, int per, double* __restrict__ pq_parts,
                  const float2* __restrict__ tw_g) {
-    using F = RegFft<N>;
     extern __shared__ float2 sm[];
     __shared__ double red[16];
     float2* tw = sm;
     float2* res = sm + N;
     const size_t npix = (size_t)P * N;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = tw_g[i];
+    F::fill(tw, tw_g);
     const int fl = threadIdx.x / F::kLanes, i = threadIdx.x % F::kLanes;
     float2* sx = res + fl * F::kBuf;
     pdl_wait();
@@ -275,211 +304,28 @@ row_inv_w_kernel(float2* t, const float2* __restrict__ p, const float2* __restri
         const bool ok = n0 + fl < n1;
         float2 u[F::kOut];
 #pragma unroll
-        for (int m = 0; m < 8; ++m)
+        for (int m = 0; m < F::kIn; ++m)
             u[m] = ok ? trow[(size_t)(n0 + fl) * npix + i + m * F::kLanes] : make_float2(0.f, 0.f);
-        WLoads<M> wl;
-        w_load<N, M, CIRC>(wl, p + (size_t)r1 * N, S + (size_t)r1 * N, threadIdx.x, T, n0, n1, npix);
-        F::template run<true, false>(u, sx, 1, tw, i);
-        F::sync();  // the last exchange is read
+        constexpr int FC = kWRun<F, M>;
+        WLoads<M, FC> wl;
+        w_load<N, M, FC, CIRC>(wl, p + (size_t)r1 * N, S + (size_t)r1 * N, threadIdx.x, T, n0, n1, npix);
+        if (!F::kByWarp || n0 + (int)(threadIdx.x & ~31u) / F::kLanes < n1) {
+            F::inverse(u, sx, tw, i);
+            F::sync();  // the last exchange is read
 #pragma unroll
-        for (int m = 0; m < F::kOut; ++m) {
-            const int e = F::out_at(i, m);
-            if (e >= 0) sx[F::at(e)] = u[m];
+            for (int m = 0; m < F::kOut; ++m) {
+                const int e = F::out_at(i, m);
+                if (e >= 0) sx[F::at(e)] = u[m];
+            }
         }
         __syncthreads();
-        w_phase<N, M, CIRC, true>(wl, trow, p + (size_t)r1 * N, S + (size_t)r1 * N, res, lam, T, n0, n1, npix);
+        w_phase<F, N, M, FC, CIRC, true>(wl, trow, p + (size_t)r1 * N, S + (size_t)r1 * N, res, lam, T, n0, n1, npix);
         __syncthreads();  // the terms
         if (un + (int)gridDim.x >= nunit) pdl_trigger();
-        tot += w_terms<N>(res, n1 - n0);
+        tot += w_terms<F, N>(res, n1 - n0);
         __syncthreads();  // the terms are read
     }
     tot = warps_sum_t0(tot, red);
-    if (threadIdx.x == 0) pq_parts[blockIdx.x] = tot;
-}
-
-// Pass C for 256-point rows: one CTA per image row r1 with 16 threads per frame; the inverse row
-// transforms run in registers (regfft.cuh), the rest as in row_inv_w_kernel. The block is padded
-// to a multiple of 16 frames (256 threads), at least 32: warps without a frame skip the
-// transform, and the W phase gives each column blockDim / 256 threads, each with a contiguous
-// range of frames. Shared memory: p rows [T][256], then the exchange buffers [T'][16 x 17] (T' = T
-// rounded up to even, the frames of the warps that transform) which afterwards hold the
-// transformed rows [T][256].
-template <int M>
-__global__ void __launch_bounds__(1024)
-row_inv_w_256_kernel(float2* t, const float2* __restrict__ p, const float2* __restrict__ S,
-                     float lam, int T, int P, double* __restrict__ pq_parts,
-                     const float2* __restrict__ tw_g) {
-    constexpr int N = 256;
-    extern __shared__ float2 sm[];
-    __shared__ float2 tw2[256];
-    __shared__ double red[32];
-    float2* pt = sm;
-    float2* res = sm + (size_t)T * N;
-    fill_tw256(tw2, tw_g);
-    pdl_wait();
-    const int n = threadIdx.x / 16, j = threadIdx.x % 16;
-    const bool live = n < T;                            // the block is padded (see the launch)
-    const bool warp_live = (threadIdx.x / 32) * 2 < T;  // a warp holds frames 2w and 2w + 1
-    const size_t npix = (size_t)P * N;
-    const int k = T - M + 1;
-    float acc = 0.f, comp = 0.f;  // Kahan-compensated per-thread partial of Re <p, q>
-    for (int r1 = blockIdx.x; r1 < P; r1 += gridDim.x) {
-    __syncthreads();  // the previous row's results are stored
-    const size_t g0 = (size_t)n * npix + (size_t)r1 * N + j;
-    float2 u[16];
-#pragma unroll
-    for (int n1 = 0; n1 < 16; ++n1) {
-        u[n1] = make_float2(0.f, 0.f);
-        if (live) {
-            u[n1] = t[g0 + 16 * n1];
-            pt[n * N + 16 * n1 + j] = p[g0 + 16 * n1];
-        }
-    }
-    __syncthreads();  // tw2
-    if (warp_live) row_dft256<true>(u, res + n * (16 * 17), tw2, j);  // warp-uniform
-    __syncthreads();  // every exchange buffer read
-    if (live) {
-#pragma unroll
-        for (int k2 = 0; k2 < 16; ++k2) res[n * N + j + 16 * k2] = u[k2];
-    }
-    __syncthreads();
-    {   // W phase: column c, frames [f0, f1) of this thread's group (blockDim.x = ng N)
-        const int c = threadIdx.x % N, ng = blockDim.x / N, g = threadIdx.x / N;
-        const int f0 = g * T / ng, f1 = (g + 1) * T / ng;
-        float2 s[M][M];
-        load_S<M>(S, npix, (size_t)r1 * N + c, s);
-        float2 cs[2 * M - 1];
-        s_diagonals<M>(s, cs);
-        for (int nn = f0; nn < f1; ++nn) {
-            const float2 w = w_frame<M, false>(s, cs, pt + c, N, nn, T, k);
-            float2 q = res[nn * N + c];
-            q.x = fmaf(lam, w.x, q.x);
-            q.y = fmaf(lam, w.y, q.y);
-            res[nn * N + c] = q;
-            const float2 pv = pt[nn * N + c];
-            const float term = fmaf(pv.x, q.x, pv.y * q.y) - comp;
-            const float sum = acc + term;
-            comp = (sum - acc) - term;
-            acc = sum;
-        }
-    }
-    __syncthreads();  // every column of q written
-    if (r1 + (int)gridDim.x >= P) pdl_trigger();
-    for (int e = threadIdx.x; e < T * N; e += blockDim.x) {
-        const int nn = e / N, c = e % N;
-        t[(size_t)nn * npix + (size_t)r1 * N + c] = res[e];
-    }
-    }
-    const double tot = block_sum_f_t0(acc, red);
-    if (threadIdx.x == 0) pq_parts[blockIdx.x] = tot;
-}
-
-// Pass C for 128-point rows: as row_inv_w_256_kernel with 8 threads per frame (row_dft128), the
-// block padded to at least 16 frames (128 threads, one column each in the W phase) and at most
-// 64; warps without a frame skip the transform. A CTA usually owns several rows (volumes have
-// R P rows), so the inputs of its next row are staged into shared memory by asynchronous copies
-// while the current one is processed: the p rows (double-buffered) as the row starts, the t rows
-// once the current ones are in registers, the S row once the current one has been used. Shared
-// memory: p rows [2][T][128], t rows [T][128], S row [npair][128], then the exchange buffers
-// [T4][kX128] (T4 = T rounded up to whole warps) which afterwards hold the transformed rows.
-template <int M>
-__global__ void __launch_bounds__(512)
-row_inv_w_128_kernel(float2* t, const float2* __restrict__ p, const float2* __restrict__ S,
-                     float lam, int T, int P, double* __restrict__ pq_parts,
-                     const float2* __restrict__ tw_g) {
-    constexpr int N = 128;
-    constexpr int NP = M * (M + 1) / 2;
-    extern __shared__ __align__(16) float2 sm[];
-    __shared__ float2 tw8[128];
-    __shared__ double red[32];
-    const int TN = T * N;
-    float2* pst = sm;             // [2][T][N]
-    float2* tst = sm + 2 * TN;    // [T][N]
-    float2* sst = tst + TN;       // [NP][N]
-    float2* res = sst + NP * N;   // [T4][kX128]
-    fill_tw128(tw8, tw_g);
-    pdl_wait();
-    const int n = threadIdx.x / 8, j = threadIdx.x % 8;
-    const bool live = n < T;
-    const bool warp_live = (threadIdx.x / 32) * 4 < T;  // a warp holds frames 4w .. 4w + 3
-    const size_t npix = (size_t)P * N;
-    const int k = T - M + 1;
-    // 16-byte copies of `rows` rows of N values, row f from src + f * stride, to dst + f * N
-    auto stage = [&](float2* dst, const float2* src, size_t stride, int rows) {
-        for (int e = threadIdx.x; e < rows * (N / 2); e += blockDim.x) {
-            const int f = e / (N / 2), c2 = 2 * (e % (N / 2));
-            cp_async16(dst + f * N + c2, src + f * stride + c2);
-        }
-        cp_async_commit();
-    };
-    float acc = 0.f, comp = 0.f;  // Kahan-compensated per-thread partial of Re <p, q>
-    int buf = 0;
-    if ((int)blockIdx.x < P) {
-        const size_t r0 = (size_t)blockIdx.x * N;
-        stage(pst, p + r0, npix, T);
-        stage(tst, t + r0, npix, T);
-        stage(sst, S + r0, npix, NP);
-    }
-    for (int r1 = blockIdx.x; r1 < P; r1 += gridDim.x, buf ^= 1) {
-    const int nxt = r1 + gridDim.x;
-    const size_t rn = (size_t)nxt * N;
-    cp_async_wait<0>();
-    __syncthreads();  // this row's copies landed (every thread's); tw8; the previous row stored
-    // the other p buffer was last read before the previous row's final barrier
-    if (nxt < P) stage(pst + (buf ^ 1) * TN, p + rn, npix, T);
-    float2 a[8], b[8];
-    if (warp_live) {  // warp-uniform
-        float2 u[16];
-#pragma unroll
-        for (int n1 = 0; n1 < 16; ++n1) u[n1] = live ? tst[n * N + 8 * n1 + j] : make_float2(0.f, 0.f);
-        row_dft128<true>(u, a, b, res + n * kX128, tw8, j);
-    }
-    __syncthreads();  // every exchange buffer read; every t row in registers
-    if (nxt < P) stage(tst, t + rn, npix, T);
-    if (live) {
-#pragma unroll
-        for (int k2 = 0; k2 < 8; ++k2) {
-            res[n * N + 2 * j + 16 * k2] = a[k2];
-            res[n * N + 2 * j + 1 + 16 * k2] = b[k2];
-        }
-    }
-    __syncthreads();
-    const float2* pt = pst + buf * TN;
-    for (int c = threadIdx.x; c < N; c += blockDim.x) {
-        float2 s[M][M];  // S(r) from the staged row, pair (a <= b) at a(2M-a+1)/2 + (b-a)
-#pragma unroll
-        for (int aa = 0; aa < M; ++aa)
-#pragma unroll
-            for (int bb = aa; bb < M; ++bb) {
-                const float2 v = sst[(aa * (2 * M - aa + 1) / 2 + (bb - aa)) * N + c];
-                s[aa][bb] = v;
-                s[bb][aa] = cconj(v);
-            }
-        float2 cs[2 * M - 1];
-        s_diagonals<M>(s, cs);
-        for (int nn = 0; nn < T; ++nn) {
-            const float2 w = w_frame<M, false>(s, cs, pt + c, N, nn, T, k);
-            float2 q = res[nn * N + c];
-            q.x = fmaf(lam, w.x, q.x);
-            q.y = fmaf(lam, w.y, q.y);
-            res[nn * N + c] = q;
-            const float2 pv = pt[nn * N + c];
-            const float term = fmaf(pv.x, q.x, pv.y * q.y) - comp;
-            const float sum = acc + term;
-            comp = (sum - acc) - term;
-            acc = sum;
-        }
-    }
-    __syncthreads();  // every column of q written; the S row used
-    if (nxt < P) stage(sst, S + rn, npix, NP);
-    else pdl_trigger();
-    float2* trow = t + (size_t)r1 * N;
-    for (int e = threadIdx.x; e < TN; e += blockDim.x) {
-        const int nn = e / N, c = e % N;
-        trow[nn * npix + c] = res[e];
-    }
-    }
-    const double tot = block_sum_f_t0(acc, red);
     if (threadIdx.x == 0) pq_parts[blockIdx.x] = tot;
 }
 
@@ -563,12 +409,13 @@ coil_row_inv_kernel(float2* t, const float2* __restrict__ p, const float2* __res
         return;
     } else {
         __syncthreads();
-        WLoads<M> wl;
-        w_load<N, M, false>(wl, p + (size_t)r1 * N, S + (size_t)r1 * N, threadIdx.x, T, 0, T, npix);
-        w_phase<N, M, false, false>(wl, trow, p + (size_t)r1 * N, S + (size_t)r1 * N, res, lam, T, 0, T, npix);
+        constexpr int FC = M > 4 ? 2 : 4;
+        WLoads<M, FC> wl;
+        w_load<N, M, FC, false>(wl, p + (size_t)r1 * N, S + (size_t)r1 * N, threadIdx.x, T, 0, T, npix);
+        w_phase<F, N, M, FC, false, false>(wl, trow, p + (size_t)r1 * N, S + (size_t)r1 * N, res, lam, T, 0, T, npix);
         __syncthreads();  // the terms
         pdl_trigger();
-        const double tot = warps_sum_t0(w_terms<N>(res, T), red);
+        const double tot = warps_sum_t0(w_terms<F, N>(res, T), red);
         if (threadIdx.x == 0) pq_parts[blockIdx.x] = tot;
     }
 }
@@ -829,49 +676,12 @@ cudaError_t row_grid(K kern, int threads, size_t smem, long long rows, int* grid
 template <int N, int M>
 cudaError_t launch_row_inv_w_NM(const Dims& d, const Twiddles& tw, float2* t, const float2* p,
                                 const float2* S, float lam, Partials* pq, cudaStream_t st) {
+    using F = RowFft<N>;
     const int rows = d.rows();
     int grid = 0;
-    if (N == 128 && !d.circ) {  // register transforms for the valid (non-circular) lifting
-        // whole warps, and at least 128 threads so that the W phase has one column per thread
-        const int tpad = d.T <= 16 ? 16 : (d.T + 3) / 4 * 4;
-        const int t4 = (d.T + 3) / 4 * 4;  // frames of the warps that transform
-        const size_t smem128 =
-            ((size_t)3 * d.T * N + (size_t)d.M * (d.M + 1) / 2 * N + (size_t)t4 * kX128) * sizeof(float2);
-        if (tpad * 8 <= 512 && smem128 <= 200 * 1024) {
-            auto k = row_inv_w_128_kernel<M>;
-            if (smem128 > kDynSmemFree) {
-                cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)smem128);
-                if (e != cudaSuccess) return e;
-            }
-            cudaError_t e = row_grid(k, tpad * 8, smem128, rows, &grid);
-            if (e != cudaSuccess) return e;
-            pq->n = grid;
-            return launch_pdl(k, dim3(grid), dim3(tpad * 8), smem128, st, t, p, S, lam, d.T, rows,
-                              pq->parts, tw.twQ);
-        }
-    }
-    if (N == 256 && !d.circ) {  // the register kernel serves the valid (non-circular) lifting
-        const int t2 = (d.T + 1) / 2 * 2;                          // frames that transform
-        const int tpad = d.T <= 32 ? 32 : (d.T + 15) / 16 * 16;   // frames of the block
-        const size_t smem256 = ((size_t)d.T * N + (size_t)t2 * 16 * 17) * sizeof(float2);
-        if (tpad * 16 <= 1024 && smem256 <= 200 * 1024) {
-            auto k = row_inv_w_256_kernel<M>;
-            if (smem256 > kDynSmemFree) {
-                cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)smem256);
-                if (e != cudaSuccess) return e;
-            }
-            cudaError_t e = row_grid(k, tpad * 16, smem256, rows, &grid);
-            if (e != cudaSuccess) return e;
-            pq->n = grid;
-            return launch_pdl(k, dim3(grid), dim3(tpad * 16), smem256, st, t, p, S, lam, d.T, rows,
-                              pq->parts, tw.twQ);
-        }
-    }
-    auto k = d.circ ? row_inv_w_kernel<N, M, true> : row_inv_w_kernel<N, M, false>;
-    const RunShape v = run_shape<N>(d.T, rows);
-    const size_t smem = ((size_t)v.bufs * RegFft<N>::kBuf + N) * sizeof(float2);
+    auto k = d.circ ? row_inv_w_kernel<F, N, M, true> : row_inv_w_kernel<F, N, M, false>;
+    const RunShape v = run_shape<F, N>(d.T, rows);
+    const size_t smem = ((size_t)v.bufs * F::kBuf + N) * sizeof(float2);
     if (smem > kDynSmemFree) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;

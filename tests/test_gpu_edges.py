@@ -290,3 +290,24 @@ def test_gram_row_lengths(R, T, P, Q, N1, N2, M):
     for a in range(M):
         e = a * (2 * M - a + 1) // 2
         assert np.array_equal(ln[e], ln[e, ::-1, ::-1].conj())
+
+
+@pytest.mark.parametrize("T,P,Q,M", [(1, 16, 256, 1), (24, 32, 256, 3), (25, 16, 256, 4), (33, 16, 256, 2),
+                                     (9, 256, 256, 5), (31, 16, 256, 6), (3, 16, 128, 2), (33, 16, 128, 3),
+                                     (66, 32, 128, 1), (17, 64, 128, 6), (2, 512, 128, 2)])
+def test_operator_in_frame_runs(R, T, P, Q, M):
+    """A^H A + lam W with rows of 128 and 256 elements: one and several runs of frames, runs that leave
+    threads and warps without a frame, valid and time-circular form, against FP64: the gate of the
+    operator parity tests (1e-5)."""
+    import torch
+    recon, ctx = R
+    rng = np.random.default_rng(T + P + Q + M)
+    x = _series(rng, T, P, Q)
+    S, full = _hermitian_pairs(rng, M, P, Q)
+    m = (rng.random((T, P, Q)) < 0.4).astype(np.uint8)
+    aha = np.fft.ifft2(m * np.fft.fft2(x, norm="ortho"), norm="ortho")
+    xd = to_dev(x)
+    y = torch.empty_like(xd)
+    for circ, variant in ((False, recon.RECON_VARIANT_PROPOSED), (True, recon.RECON_VARIANT_GIRAF)):
+        recon.recon_apply_normal_variant(ctx.h, to_dev(m), (1, 1, M), variant, to_dev(S), 0.7, xd, y)
+        assert_close(y.cpu().numpy(), aha + 0.7 * _w(full, x, circ), 1e-5)
