@@ -47,14 +47,16 @@ def alg_bytes(kind: str, w, n_cg: int) -> float:
     E = w.T * w.P * w.Q * D
     N = w.P * w.Q * D
     npair = w.M * (w.M + 1) // 2
+    # from 2^18 elements on, x += alpha p of every step but the last comes with the next row pass
+    moved = 16.0 * E * (n_cg - 1) / n_cg if E >= 1 << 18 else 0.0  # x read and written there
     if kind == "cg_row_fwd":      # read r (+ p), write p and t
-        return (24.0 * E + 32.0 * E * (n_cg - 1)) / n_cg
+        return (24.0 * E + 32.0 * E * (n_cg - 1)) / n_cg + moved
     if kind == "cg_col_mask":     # read t, mask; write t
         return 17.0 * E
     if kind == "cg_row_inv_w":    # read t, p, S; write q
         return 24.0 * E + 8.0 * npair * N
     if kind == "cg_update":       # read x, r, p, q; write x, r
-        return 48.0 * E
+        return 48.0 * E - 1.5 * moved  # (neither x nor p)
     if kind == "resid_carry":     # read x, r, S_old, S_new; write r (first: no r, S_old)
         return 24.0 * E + 16.0 * npair * N
     if kind == "gram":            # read x

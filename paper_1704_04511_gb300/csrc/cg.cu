@@ -420,44 +420,62 @@ coil_row_inv_kernel(float2* t, const float2* __restrict__ p, const float2* __res
     }
 }
 
-// Pass D: alpha = |r|^2 / Re <p, q> (Re <p, q> summed here from pass C's partials); x += alpha p;
-// r -= alpha q; per-CTA partials of |r_new|^2 for the next pass A.
+// Pass D: alpha = |r|^2 / Re <p, q> (Re <p, q> summed here from pass C's partials), stored for the next
+// pass A; r -= alpha q; per-CTA partials of |r_new|^2 for the next pass A; x += alpha p with kX (else
+// the next pass A does it). Bound by memory (L2 or HBM), 256x256x16 7.5 us with x; the order of the sum
+// is the same with and without x.
+template <bool kX>
 __global__ void __launch_bounds__(kUpdThreads, kUpdPerSM)
 cg_update_kernel(float4* __restrict__ x, float4* __restrict__ r, const float4* __restrict__ p,
                  const float4* __restrict__ q, size_t n4, const double* __restrict__ rr_in,
-                 const double* __restrict__ pq_parts, int n_pq, double* __restrict__ rr_parts) {
+                 const double* __restrict__ pq_parts, int n_pq, double* __restrict__ rr_parts,
+                 double* __restrict__ alpha_out) {
+    constexpr int V = kX ? kUpdVec : 2 * kUpdVec;
     __shared__ double red[kUpdThreads / 32];
     __shared__ double s_pq;
     __shared__ float alpha_s;
     pdl_wait();
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    float4 xv[kUpdVec], rv[kUpdVec], pv[kUpdVec], qv[kUpdVec];
-    // the first loads go out before alpha is known (they do not depend on it)
+    float4 xv[V], rv[V], pv[V], qv[V];
+    auto load = [&](size_t at) {
 #pragma unroll
-    for (int u = 0; u < kUpdVec; ++u) {
-        const size_t i = i0 + (size_t)u * stride;
-        if (i < n4) { xv[u] = x[i]; rv[u] = r[i]; pv[u] = p[i]; qv[u] = q[i]; }
-    }
+        for (int u = 0; u < V; ++u) {
+            const size_t i = at + (size_t)u * stride;
+            if (i >= n4) continue;
+            rv[u] = r[i];
+            qv[u] = q[i];
+            if constexpr (kX) {
+                xv[u] = x[i];
+                pv[u] = p[i];
+            }
+        }
+    };
+    load(i0);  // the first loads go out before alpha is known (they do not depend on it)
     const double pq = sum_partials(pq_parts, n_pq, &s_pq);
-    if (threadIdx.x == 0) alpha_s = (float)(rr_in[0] * rcp_nr(pq));
+    if (threadIdx.x == 0) {
+        alpha_s = (float)(rr_in[0] * rcp_nr(pq));
+        if (blockIdx.x == 0) alpha_out[0] = (double)alpha_s;
+    }
     __syncthreads();
     const float alpha = alpha_s;
     float acc = 0.f, comp = 0.f;
-    for (; i0 < n4; i0 += stride * kUpdVec) {
+    for (; i0 < n4; i0 += stride * V) {
 #pragma unroll
-        for (int u = 0; u < kUpdVec; ++u) {
+        for (int u = 0; u < V; ++u) {
             const size_t i = i0 + (size_t)u * stride;
             if (i >= n4) continue;
-            xv[u].x = fmaf(alpha, pv[u].x, xv[u].x);
-            xv[u].y = fmaf(alpha, pv[u].y, xv[u].y);
-            xv[u].z = fmaf(alpha, pv[u].z, xv[u].z);
-            xv[u].w = fmaf(alpha, pv[u].w, xv[u].w);
+            if constexpr (kX) {
+                xv[u].x = fmaf(alpha, pv[u].x, xv[u].x);
+                xv[u].y = fmaf(alpha, pv[u].y, xv[u].y);
+                xv[u].z = fmaf(alpha, pv[u].z, xv[u].z);
+                xv[u].w = fmaf(alpha, pv[u].w, xv[u].w);
+                x[i] = xv[u];
+            }
             rv[u].x = fmaf(-alpha, qv[u].x, rv[u].x);
             rv[u].y = fmaf(-alpha, qv[u].y, rv[u].y);
             rv[u].z = fmaf(-alpha, qv[u].z, rv[u].z);
             rv[u].w = fmaf(-alpha, qv[u].w, rv[u].w);
-            x[i] = xv[u];
             r[i] = rv[u];
             const float4 w = rv[u];
             const float term = fmaf(w.x, w.x, fmaf(w.y, w.y, fmaf(w.z, w.z, w.w * w.w))) - comp;
@@ -465,12 +483,7 @@ cg_update_kernel(float4* __restrict__ x, float4* __restrict__ r, const float4* _
             comp = (sum - acc) - term;
             acc = sum;
         }
-        const size_t nx = i0 + stride * kUpdVec;
-#pragma unroll
-        for (int u = 0; u < kUpdVec; ++u) {
-            const size_t i = nx + (size_t)u * stride;
-            if (i < n4) { xv[u] = x[i]; rv[u] = r[i]; pv[u] = p[i]; qv[u] = q[i]; }
-        }
+        load(i0 + stride * V);
     }
     pdl_trigger();
     const double tot = block_sum_f_t0(acc, red);
@@ -815,14 +828,15 @@ cudaError_t launch_coil_combine(const Dims& d, const Twiddles& tw, float2* t, co
 
 cudaError_t launch_cg_update(const Dims& d, float2* x, float2* r, const float2* p,
                              const float2* q, const double* rr_in, const Partials& pq,
-                             Partials* rr, cudaStream_t st) {
+                             Partials* rr, double* alpha, bool with_x, cudaStream_t st) {
     const size_t n4 = d.elems() / 2;  // two complex values per float4
     const int grid = upd_grid(n4);
     rr->n = grid;
-    return launch_pdl(cg_update_kernel, dim3(grid), dim3(kUpdThreads), 0, st,
-                      reinterpret_cast<float4*>(x), reinterpret_cast<float4*>(r),
-                      reinterpret_cast<const float4*>(p), reinterpret_cast<const float4*>(q), n4,
-                      rr_in, (const double*)pq.parts, pq.n, rr->parts);
+    return launch_pdl(with_x ? cg_update_kernel<true> : cg_update_kernel<false>, dim3(grid),
+                      dim3(kUpdThreads), 0, st, reinterpret_cast<float4*>(x),
+                      reinterpret_cast<float4*>(r), reinterpret_cast<const float4*>(p),
+                      reinterpret_cast<const float4*>(q), n4, rr_in, (const double*)pq.parts, pq.n,
+                      rr->parts, alpha);
 }
 
 cudaError_t launch_sum_partials(const Partials& in, double* out, cudaStream_t st) {

@@ -36,6 +36,10 @@ __host__ __device__ constexpr int row_threads() { return N == 192 ? 96 : (N == 5
 template <int N>
 __host__ __device__ constexpr int row_seqs() { return row_threads<N>() / RegFft<N>::kLanes; }
 
+RECON_DEV float2 axpy(float a, float2 p, float2 x) {
+    return make_float2(fmaf(a, p.x, x.x), fmaf(a, p.y, x.y));
+}
+
 template <int N, bool INV>
 __global__ void __launch_bounds__(row_threads<N>())
 row_fft_kernel(const float2* in, float2* out, int nrows, float scale,
@@ -63,11 +67,13 @@ row_fft_kernel(const float2* in, float2* out, int nrows, float scale,
 
 // Pass A of a CG step: p = r (first) or r + beta p with beta = |r_c|^2 / |r_{c-1}|^2, |r_c|^2
 // summed here from the update pass's per-CTA partials (CTA 0 also stores it); p is written back
-// and its row FFT goes to t. The elements stay in registers (RegFft): 192x192x24 9.0 -> 7.5 us per
+// and its row FFT goes to t. With alpha (unless first) the previous step's x += *alpha p comes before p
+// is replaced. The elements stay in registers (RegFft): 192x192x24 9.0 -> 7.5 us per
 // launch, 512x512x16 35.9 -> 24.0, against passes over shared memory with a block barrier each.
 template <int N>
 __global__ void __launch_bounds__(row_threads<N>())
 row_fwd_pupdate_kernel(const float2* __restrict__ r, float2* __restrict__ p,
+                       float2* __restrict__ x, const double* __restrict__ alpha,
                        float2* __restrict__ t, int nrows, const double* __restrict__ rr_parts,
                        int n_rr, const double* __restrict__ rr_prev, double* __restrict__ rr_out,
                        int first, const float2* __restrict__ tw_g) {
@@ -81,12 +87,14 @@ row_fwd_pupdate_kernel(const float2* __restrict__ r, float2* __restrict__ p,
     const int row = blockIdx.x * row_seqs<N>() + lr;
     const bool ok = row < nrows;
     const size_t base = (size_t)row * N + i;
-    float2 u[F::kOut], pv[8];
+    float2 u[F::kOut], pv[8], xv[8];
 #pragma unroll
     for (int m = 0; m < 8; ++m) u[m] = ok ? r[base + m * F::kLanes] : make_float2(0.f, 0.f);
     if (!first) {
 #pragma unroll
         for (int m = 0; m < 8; ++m) pv[m] = ok ? p[base + m * F::kLanes] : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int m = 0; m < 8; ++m) xv[m] = ok && alpha ? x[base + m * F::kLanes] : make_float2(0.f, 0.f);
         if (threadIdx.x < 32) {  // |r|^2 from the update pass's partials, loads in flight
             const double rr_new = warp0_sum_array(rr_parts, n_rr);
             if (threadIdx.x == 0) {
@@ -98,6 +106,11 @@ row_fwd_pupdate_kernel(const float2* __restrict__ r, float2* __restrict__ p,
     __syncthreads();  // tw, beta
     if (!first) {
         const float beta = beta_s;
+        if (ok && alpha) {
+            const float al = (float)alpha[0];
+#pragma unroll
+            for (int m = 0; m < 8; ++m) x[base + m * F::kLanes] = axpy(al, pv[m], xv[m]);
+        }
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
             u[m].x = fmaf(beta, pv[m].x, u[m].x);
@@ -131,7 +144,8 @@ __host__ __device__ constexpr int coil_rows() { return N >= 512 ? 1 : 512 / N; }
 
 template <int N>
 __global__ void __launch_bounds__(coil_threads<N>())
-coil_row_fwd_kernel(const float2* __restrict__ r, float2* __restrict__ p, float2* __restrict__ t,
+coil_row_fwd_kernel(const float2* __restrict__ r, float2* __restrict__ p,
+                    float2* __restrict__ x, const double* __restrict__ alpha, float2* __restrict__ t,
                     const float2* __restrict__ coils, int nrows, int P, int nc,
                     const double* __restrict__ rr_parts, int n_rr,
                     const double* __restrict__ rr_prev, double* __restrict__ rr_out, int first,
@@ -145,7 +159,7 @@ coil_row_fwd_kernel(const float2* __restrict__ r, float2* __restrict__ p, float2
     __shared__ double s_rr;
     for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = tw_g[i];
     pdl_wait();
-    float beta = 0.f;
+    float beta = 0.f, al = 0.f;
     if (!first) {
         const double rr_new = sum_partials(rr_parts, n_rr, &s_rr);
         if (threadIdx.x == 0) {
@@ -154,6 +168,7 @@ coil_row_fwd_kernel(const float2* __restrict__ r, float2* __restrict__ p, float2
         }
         __syncthreads();
         beta = beta_s;
+        al = alpha ? (float)alpha[0] : 0.f;
     }
     const int row0 = blockIdx.x * ROWS;
     const int nr = min(ROWS, nrows - row0);
@@ -163,6 +178,7 @@ coil_row_fwd_kernel(const float2* __restrict__ r, float2* __restrict__ p, float2
         float2 v = r[base + e];
         if (!first) {
             const float2 pv = p[base + e];
+            if (alpha) x[base + e] = axpy(al, pv, x[base + e]);
             v.x = fmaf(beta, pv.x, v.x);
             v.y = fmaf(beta, pv.y, v.y);
         }
@@ -324,6 +340,7 @@ constexpr int kR256Rows = 4;  // rows per 64-thread CTA, one half-warp per row
 // Pass A of a CG step for 256-point rows (same contract as row_fwd_pupdate_kernel).
 __global__ void __launch_bounds__(64)
 row_fwd_pupdate_256_kernel(const float2* __restrict__ r, float2* __restrict__ p,
+                           float2* __restrict__ x, const double* __restrict__ alpha,
                            float2* __restrict__ t, int nrows, const double* __restrict__ rr_parts,
                            int n_rr, const double* __restrict__ rr_prev,
                            double* __restrict__ rr_out, int first,
@@ -337,13 +354,17 @@ row_fwd_pupdate_256_kernel(const float2* __restrict__ r, float2* __restrict__ p,
     const int row = blockIdx.x * kR256Rows + lr;
     const bool ok = row < nrows;
     const size_t base = (size_t)row * 256 + j;
-    float2 u[16], pv[16];
+    float2 u[16], pv[16], xv[16];
     if (ok) {
 #pragma unroll
         for (int n1 = 0; n1 < 16; ++n1) u[n1] = r[base + 16 * n1];
         if (!first) {
 #pragma unroll
             for (int n1 = 0; n1 < 16; ++n1) pv[n1] = p[base + 16 * n1];
+            if (alpha) {
+#pragma unroll
+                for (int n1 = 0; n1 < 16; ++n1) xv[n1] = x[base + 16 * n1];
+            }
         }
     } else {
 #pragma unroll
@@ -359,6 +380,11 @@ row_fwd_pupdate_256_kernel(const float2* __restrict__ r, float2* __restrict__ p,
     __syncthreads();  // tw2, beta
     if (!first) {
         const float beta = beta_s;
+        if (ok && alpha) {
+            const float al = (float)alpha[0];
+#pragma unroll
+            for (int n1 = 0; n1 < 16; ++n1) x[base + 16 * n1] = axpy(al, pv[n1], xv[n1]);
+        }
 #pragma unroll
         for (int n1 = 0; n1 < 16; ++n1) {
             u[n1].x = fmaf(beta, pv[n1].x, u[n1].x);
@@ -383,6 +409,7 @@ constexpr int kR128Rows = 8;
 
 __global__ void __launch_bounds__(64)
 row_fwd_pupdate_128_kernel(const float2* __restrict__ r, float2* __restrict__ p,
+                           float2* __restrict__ x, const double* __restrict__ alpha,
                            float2* __restrict__ t, int nrows, const double* __restrict__ rr_parts,
                            int n_rr, const double* __restrict__ rr_prev,
                            double* __restrict__ rr_out, int first,
@@ -396,13 +423,17 @@ row_fwd_pupdate_128_kernel(const float2* __restrict__ r, float2* __restrict__ p,
     const int row = blockIdx.x * kR128Rows + lr;
     const bool ok = row < nrows;
     const size_t base = (size_t)row * 128 + j;
-    float2 u[16], pv[16];
+    float2 u[16], pv[16], xv[16];
     if (ok) {
 #pragma unroll
         for (int n1 = 0; n1 < 16; ++n1) u[n1] = r[base + 8 * n1];
         if (!first) {
 #pragma unroll
             for (int n1 = 0; n1 < 16; ++n1) pv[n1] = p[base + 8 * n1];
+            if (alpha) {
+#pragma unroll
+                for (int n1 = 0; n1 < 16; ++n1) xv[n1] = x[base + 8 * n1];
+            }
         }
     } else {
 #pragma unroll
@@ -418,6 +449,11 @@ row_fwd_pupdate_128_kernel(const float2* __restrict__ r, float2* __restrict__ p,
     __syncthreads();  // tw8, beta
     if (!first) {
         const float beta = beta_s;
+        if (ok && alpha) {
+            const float al = (float)alpha[0];
+#pragma unroll
+            for (int n1 = 0; n1 < 16; ++n1) x[base + 8 * n1] = axpy(al, pv[n1], xv[n1]);
+        }
 #pragma unroll
         for (int n1 = 0; n1 < 16; ++n1) {
             u[n1].x = fmaf(beta, pv[n1].x, u[n1].x);
@@ -677,6 +713,7 @@ col_mask_64_kernel(float2* t, const uint8_t* __restrict__ mask, int Q, float sca
 // one length-128 table serves both directions); Y[k1][p2] goes to row 8 k1 + p2 of t.
 __global__ void __launch_bounds__(128)
 row_fwd_col1_128_kernel(const float2* __restrict__ r, float2* __restrict__ p,
+                        float2* __restrict__ x, const double* __restrict__ alpha,
                         float2* __restrict__ t, const double* __restrict__ rr_parts, int n_rr,
                         const double* __restrict__ rr_prev, double* __restrict__ rr_out,
                         int first, const float2* __restrict__ tw_g) {
@@ -690,12 +727,16 @@ row_fwd_col1_128_kernel(const float2* __restrict__ r, float2* __restrict__ p,
     const int p2 = blockIdx.x % 8;
     const size_t sbase = (size_t)(blockIdx.x / 8) * 128 * 128;
     const size_t base = sbase + (size_t)(8 * p1 + p2) * 128 + j;
-    float2 u[16], pv[16];
+    float2 u[16], pv[16], xv[16];
 #pragma unroll
     for (int n1 = 0; n1 < 16; ++n1) u[n1] = r[base + 8 * n1];
     if (!first) {
 #pragma unroll
         for (int n1 = 0; n1 < 16; ++n1) pv[n1] = p[base + 8 * n1];
+        if (alpha) {
+#pragma unroll
+            for (int n1 = 0; n1 < 16; ++n1) xv[n1] = x[base + 8 * n1];
+        }
     }
     if (!first && threadIdx.x < 32) {  // |r|^2 from the update pass's partials, loads in flight
         const double rr_new = warp0_sum_array(rr_parts, n_rr);
@@ -707,6 +748,11 @@ row_fwd_col1_128_kernel(const float2* __restrict__ r, float2* __restrict__ p,
     __syncthreads();  // tw8, beta
     if (!first) {
         const float beta = beta_s;
+        if (alpha) {
+            const float al = (float)alpha[0];
+#pragma unroll
+            for (int n1 = 0; n1 < 16; ++n1) x[base + 8 * n1] = axpy(al, pv[n1], xv[n1]);
+        }
 #pragma unroll
         for (int n1 = 0; n1 < 16; ++n1) {
             u[n1].x = fmaf(beta, pv[n1].x, u[n1].x);
@@ -1059,27 +1105,31 @@ cudaError_t launch_adjoint(const Dims& d, const Twiddles& tw, const void* b, int
 }
 
 cudaError_t launch_row_fwd_pupdate(const Dims& d, const Twiddles& tw, const float2* r, float2* p,
-                                   float2* t, const Partials& rr, const double* rr_prev,
+                                   float2* x, const double* alpha, float2* t, const Partials& rr,
+                                   const double* rr_prev,
                                    double* rr_out, int first, cudaStream_t st) {
     const int nrows = d.T * d.rows();
     if (vol_fold(d))  // the row DFT and the first half of the length-P DFT (see vol_fold)
-        return launch_pdl(row_fwd_col1_128_kernel, dim3(d.T * d.R * 8), dim3(128), 0, st, r, p, t,
+        return launch_pdl(row_fwd_col1_128_kernel, dim3(d.T * d.R * 8), dim3(128), 0, st, r, p, x, alpha, t,
                           (const double*)rr.parts, rr.n, rr_prev, rr_out, first, tw.twQ);
     if (d.Q == 256) {
         const int grid = (nrows + kR256Rows - 1) / kR256Rows;
-        return launch_pdl(row_fwd_pupdate_256_kernel, dim3(grid), dim3(64), 0, st, r, p, t, nrows,
+        return launch_pdl(row_fwd_pupdate_256_kernel, dim3(grid), dim3(64), 0, st, r, p, x, alpha, t,
+                          nrows,
                           (const double*)rr.parts, rr.n, rr_prev, rr_out, first, tw.twQ);
     }
     if (d.Q == 128) {
         const int grid = (nrows + kR128Rows - 1) / kR128Rows;
-        return launch_pdl(row_fwd_pupdate_128_kernel, dim3(grid), dim3(64), 0, st, r, p, t, nrows,
+        return launch_pdl(row_fwd_pupdate_128_kernel, dim3(grid), dim3(64), 0, st, r, p, x, alpha, t,
+                          nrows,
                           (const double*)rr.parts, rr.n, rr_prev, rr_out, first, tw.twQ);
     }
     switch (d.Q) {
 #define CASE(N)                                                                              \
     case N: {                                                                                \
         const int grid = (nrows + row_seqs<N>() - 1) / row_seqs<N>();                        \
-        return launch_pdl(row_fwd_pupdate_kernel<N>, dim3(grid), dim3(row_threads<N>()), 0, st, r, p, t, \
+        return launch_pdl(row_fwd_pupdate_kernel<N>, dim3(grid), dim3(row_threads<N>()), 0, st, r, p, \
+                          x, alpha, t, \
                           nrows, (const double*)rr.parts, rr.n, rr_prev, rr_out, first, tw.twQ); \
     }
         CASE(16) CASE(32) CASE(64) CASE(192) CASE(512)
@@ -1089,14 +1139,16 @@ cudaError_t launch_row_fwd_pupdate(const Dims& d, const Twiddles& tw, const floa
 }
 
 cudaError_t launch_coil_row_fwd(const Dims& d, const Twiddles& tw, const float2* r, float2* p,
-                                float2* t, const float2* coils, const Partials& rr,
+                                float2* x, const double* alpha, float2* t, const float2* coils,
+                                const Partials& rr,
                                 const double* rr_prev, double* rr_out, int first, cudaStream_t st) {
     const int nrows = d.T * d.P;
     switch (d.Q) {
 #define CASE(N)                                                                              \
     case N: {                                                                                \
         const int grid = (nrows + coil_rows<N>() - 1) / coil_rows<N>();                      \
-        return launch_pdl(coil_row_fwd_kernel<N>, dim3(grid), dim3(coil_threads<N>()), 0, st, r, p, t, \
+        return launch_pdl(coil_row_fwd_kernel<N>, dim3(grid), dim3(coil_threads<N>()), 0, st, r, p, \
+                          x, alpha, t, \
                           coils, nrows, d.P, d.nc, (const double*)rr.parts, rr.n, rr_prev,    \
                           rr_out, first, tw.twQ);                                            \
     }

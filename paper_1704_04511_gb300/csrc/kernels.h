@@ -105,9 +105,11 @@ cudaError_t launch_adjoint(const Dims& d, const Twiddles& tw, const void* b, int
 cudaError_t launch_fft2(const Dims& d, const Twiddles& tw, const float2* x, float2* y, int inv,
                         cudaStream_t st);
 // CG step, pass A: p = r (first) or r + beta p with beta = |r|^2 / *rr_prev, |r|^2 the sum of
-// the update pass's partials `rr` (also stored to *rr_out); t = row-FFT(p).
+// the update pass's partials `rr` (also stored to *rr_out); t = row-FFT(p). Unless first, the
+// previous step's x += *alpha p comes with it when alpha is given (see launch_cg_update).
 cudaError_t launch_row_fwd_pupdate(const Dims& d, const Twiddles& tw, const float2* r, float2* p,
-                                   float2* t, const Partials& rr, const double* rr_prev,
+                                   float2* x, const double* alpha, float2* t, const Partials& rr,
+                                   const double* rr_prev,
                                    double* rr_out, int first, cudaStream_t st);
 // CG step, pass B: t = column-IFFT(mask * column-FFT(t)) / (PQ), in place.
 cudaError_t launch_col_mask(const Dims& d, const Twiddles& tw, float2* t, const uint8_t* mask,
@@ -117,11 +119,12 @@ cudaError_t launch_col_mask(const Dims& d, const Twiddles& tw, float2* t, const 
 // CG step, pass C: q = row-IFFT(t) + lam W p written over t; partials of Re <p, q> to *pq.
 cudaError_t launch_row_inv_w(const Dims& d, const Twiddles& tw, float2* t, const float2* p,
                              const float2* S, float lam, Partials* pq, cudaStream_t st);
-// CG step, pass D: alpha = *rr_in / Re <p, q> (sum of `pq`); x += alpha p; r -= alpha q;
-// partials of |r|^2 to *rr.
+// CG step, pass D: alpha = *rr_in / Re <p, q> (sum of `pq`), stored to *alpha; r -= alpha q; partials
+// of |r|^2 to *rr; x += alpha p too with `with_x` (the last step, and steps whose next pass A is not
+// given alpha).
 cudaError_t launch_cg_update(const Dims& d, float2* x, float2* r, const float2* p,
                              const float2* q, const double* rr_in, const Partials& pq,
-                             Partials* rr, cudaStream_t st);
+                             Partials* rr, double* alpha, bool with_x, cudaStream_t st);
 // *out = the sum of the partials `in` (one warp).
 cudaError_t launch_sum_partials(const Partials& in, double* out, cudaStream_t st);
 // Residual carry: r = (first ? r0 : r) + lam W_{S_old - S_new} x (S_old ignored when first),
@@ -206,7 +209,8 @@ cudaError_t launch_lanczos_lmax(int s, const double2* G, void* scratch, double* 
 // ---- coils (Eq. measurement-ij with receiver sensitivities C_c; d.nc coils, coil-major) ----
 // Pass A: p = r (first) or r + beta p (as launch_row_fwd_pupdate); t[c] = row-FFT(C_c * p).
 cudaError_t launch_coil_row_fwd(const Dims& d, const Twiddles& tw, const float2* r, float2* p,
-                                float2* t, const float2* coils, const Partials& rr,
+                                float2* x, const double* alpha, float2* t, const float2* coils,
+                                const Partials& rr,
                                 const double* rr_prev, double* rr_out, int first, cudaStream_t st);
 // Pass C: q = sum_c conj(C_c) row-IFFT(t[c]) + lam W p over coil 0's plane of t; partials of
 // Re <p, q> to *pq.

@@ -568,7 +568,7 @@ int cg_block(recon_ctx* c, const Dims& d, const Twiddles& tw, Work& w, const uin
             // keeps the projection, and the exact identity avoids the FP32 cancellation.
             const recon::Partials none{nullptr, 0};
             recon::Partials scratch{w.rparts, 0};
-            RC_CUDA(recon::launch_coil_row_fwd(d, tw, x, w.p, w.t, coils, none, nullptr, nullptr, 1,
+            RC_CUDA(recon::launch_coil_row_fwd(d, tw, x, w.p, nullptr, nullptr, w.t, coils, none, nullptr, nullptr, 1,
                                                c->stream));
             RC_CUDA(recon::launch_col_mask(d, tw, w.t, mask, c->stream));
             RC_CUDA(recon::launch_coil_row_inv_w(d, tw, w.t, w.p, coils, S_new, 0.f, &scratch,
@@ -582,15 +582,22 @@ int cg_block(recon_ctx* c, const Dims& d, const Twiddles& tw, Work& w, const uin
     // the update pass; the update pass leaves those of |r|^2 in w.rparts for the next pass A,
     // which also stores the sum in rr[it] (rr[0] comes from the residual carry).
     recon::Partials pq{w.parts, 0}, rr{w.rparts, 0};
+    // x += alpha p of a step comes with the next pass A, which reads p anyway: 9 instead of 10 series of
+    // traffic a step besides the transforms. Series of 2^18 elements or more (15 steps at 192x128x20 436
+    // instead of 455 us, 512x512x16 1185 instead of 1243, 2 x 15 at 128x128x64x12 10.75 instead of
+    // 11.37 ms); the passes of smaller ones are bound by latency, and pass A is the longer chain
+    // (128x128x12, pixel-wise prior: 978 against 972 us).
+    const bool defer = d.elems() >= (size_t)1 << 18;
     for (int it = 0; it < n_cg; ++it) {
         const double* rr_prev = it > 0 ? w.rr + it - 1 : w.rr;
+        const double* alpha = it > 0 && defer ? w.pq + it - 1 : nullptr;  // the previous step's, for x
         {
             ProfScope ps(c, RECON_PROF_CG_ROWFWD);
             if (coils)
-                RC_CUDA(recon::launch_coil_row_fwd(d, tw, w.r, w.p, w.t, coils, rr, rr_prev,
-                                                   w.rr + it, it == 0, c->stream));
+                RC_CUDA(recon::launch_coil_row_fwd(d, tw, w.r, w.p, x, alpha, w.t, coils, rr,
+                                                   rr_prev, w.rr + it, it == 0, c->stream));
             else
-                RC_CUDA(recon::launch_row_fwd_pupdate(d, tw, w.r, w.p, w.t, rr, rr_prev,
+                RC_CUDA(recon::launch_row_fwd_pupdate(d, tw, w.r, w.p, x, alpha, w.t, rr, rr_prev,
                                                       w.rr + it, it == 0, c->stream));
         }
         {
@@ -606,7 +613,8 @@ int cg_block(recon_ctx* c, const Dims& d, const Twiddles& tw, Work& w, const uin
                 RC_CUDA(recon::launch_row_inv_w(d, tw, w.t, w.p, S_new, lam, &pq, c->stream));
         }
         ProfScope ps(c, RECON_PROF_CG_UPDATE);
-        RC_CUDA(recon::launch_cg_update(d, x, w.r, w.p, w.t, w.rr + it, pq, &rr, c->stream));
+        RC_CUDA(recon::launch_cg_update(d, x, w.r, w.p, w.t, w.rr + it, pq, &rr, w.pq + it,
+                                        !defer || it + 1 == n_cg, c->stream));
     }
     if (n_cg > 0) RC_CUDA(recon::launch_sum_partials(rr, w.rr + n_cg, c->stream));
     return RECON_OK;
@@ -1522,7 +1530,7 @@ int apply_normal_impl(recon_ctx* c, const Dims& d0, const uint8_t* masks, const 
     recon::Partials pq{(double*)parts, 0};
     const recon::Partials none{nullptr, 0};
     // the CG operator passes with first = 1 (p = x); y receives (A^H A + lambda W) x
-    RC_CUDA(recon::launch_row_fwd_pupdate(d, tw, (const float2*)x, (float2*)pp, (float2*)y, none,
+    RC_CUDA(recon::launch_row_fwd_pupdate(d, tw, (const float2*)x, (float2*)pp, nullptr, nullptr, (float2*)y, none,
                                           nullptr, nullptr, 1, c->stream));
     RC_CUDA(recon::launch_col_mask(d, tw, (float2*)y, masks, c->stream));
     RC_CUDA(recon::launch_row_inv_w(d, tw, (float2*)y, (const float2*)pp, (const float2*)S,
@@ -1752,8 +1760,8 @@ int recon_apply_normal_coils(recon_ctx* c, recon_dims dd, recon_filter f, const 
     recon::Partials pq{(double*)parts, 0};
     const recon::Partials none{nullptr, 0};
     // the coil passes with first = 1 (p = x); q lands in coil 0's plane of t
-    RC_CUDA(recon::launch_coil_row_fwd(d, tw, (const float2*)x, (float2*)pp, (float2*)t,
-                                       (const float2*)coils, none, nullptr, nullptr, 1, c->stream));
+    RC_CUDA(recon::launch_coil_row_fwd(d, tw, (const float2*)x, (float2*)pp, nullptr, nullptr,
+                                       (float2*)t, (const float2*)coils, none, nullptr, nullptr, 1, c->stream));
     RC_CUDA(recon::launch_col_mask(d, tw, (float2*)t, masks, c->stream));
     RC_CUDA(recon::launch_coil_row_inv_w(d, tw, (float2*)t, (const float2*)pp, (const float2*)coils,
                                          (const float2*)S, (float)lambda, &pq, c->stream));

@@ -311,3 +311,60 @@ def test_operator_in_frame_runs(R, T, P, Q, M):
     for circ, variant in ((False, recon.RECON_VARIANT_PROPOSED), (True, recon.RECON_VARIANT_GIRAF)):
         recon.recon_apply_normal_variant(ctx.h, to_dev(m), (1, 1, M), variant, to_dev(S), 0.7, xd, y)
         assert_close(y.cpu().numpy(), aha + 0.7 * _w(full, x, circ), 1e-5)
+
+
+@pytest.mark.parametrize("T,P,Q", [(7, 64, 64), (16, 128, 128), (15, 128, 128), (64, 64, 64), (7, 256, 192),
+                                   (9, 128, 256), (1, 512, 512), (512, 32, 16)])
+@pytest.mark.parametrize("steps", [1, 2, 5])
+def test_cg_steps_around_the_deferred_update(R, T, P, Q, steps):
+    """x and r after CG steps on both sides of 2^18 elements, where x += alpha p moves to the next step's
+    first pass and stays with the last one, against FP64 CG on a well-conditioned operator (eigenvalues
+    0.5 to about 3): the rounding of the operator, 1e-5."""
+    recon, ctx = R
+    rng = np.random.default_rng(T + P + Q + steps)
+    S = np.abs(rng.standard_normal((1, P, Q))).clip(0.5, 2.0).astype(np.complex64)
+    x = _series(rng, T, P, Q)
+    m = (rng.random((T, P, Q)) < 0.4).astype(np.uint8)
+    xd, rd = to_dev(x), to_dev(np.zeros_like(x))
+    recon.recon_cg(ctx.h, to_dev(m), (1, 1, 1), None, to_dev(S), 1.0, xd, rd, steps)
+
+    def op(v):
+        return np.fft.ifft2(m * np.fft.fft2(v, norm="ortho"), norm="ortho") + S[0].real * v
+
+    ref = x.astype(np.complex128)
+    r = -S[0].real * ref
+    p, rr = r.copy(), np.vdot(r, r).real
+    for _ in range(steps):
+        q = op(p)
+        alpha = rr / np.vdot(p, q).real
+        ref = ref + alpha * p
+        r = r - alpha * q
+        new = np.vdot(r, r).real
+        p, rr = r + new / rr * p, new
+    scale = np.linalg.norm(x)
+    assert np.linalg.norm(xd.cpu().numpy() - ref) < 1e-5 * scale
+    assert np.linalg.norm(rd.cpu().numpy() - r) < 1e-5 * scale
+
+
+@pytest.mark.parametrize("T", [15, 16])
+def test_coil_and_volume_solves_around_the_deferred_update(R, T):
+    """The same for the coil and the volume passes: one IRLS iteration against the oracle, whose
+    parity gate (1e-4) it takes."""
+    import torch
+    from oracle import slr, slr3
+    recon, ctx = R
+    rng = np.random.default_rng(T)
+    m = (rng.random((T, 128, 128)) < 0.4).astype(np.uint8)
+    C = _series(rng, 2, 128, 128)
+    C /= np.sqrt((np.abs(C) ** 2).sum(0))
+    b = _series(rng, 2, T, 128, 128) * m
+    out = torch.empty(m.shape, dtype=torch.complex64, device="cuda")
+    recon.recon_solve_coils(ctx.h, to_dev(b), to_dev(m), to_dev(C), (2, 2, 2), 0.1, 0.0, 1, 3, out)
+    ref = slr.irls(b.astype(np.complex128), m, 2, 2, 2, 0.1, 0.0, 1, 3, coils=C.astype(np.complex128))
+    assert_close(out.cpu().numpy(), ref, 1e-4)
+    m3 = (rng.random((T, 16, 32, 32)) < 0.4).astype(np.uint8)
+    b3 = _series(rng, T, 16, 32, 32) * m3
+    out = torch.empty(m3.shape, dtype=torch.complex64, device="cuda")
+    recon.recon_solve3(ctx.h, to_dev(b3), to_dev(m3), (2, 2, 2, 2), 0.1, 0.0, 1, 3, out)
+    ref = slr3.irls3(b3.astype(np.complex128), m3, 2, 2, 2, 2, 0.1, 0.0, 1, 3)
+    assert_close(out.cpu().numpy(), ref, 1e-4)
