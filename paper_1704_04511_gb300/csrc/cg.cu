@@ -263,8 +263,14 @@ struct RunShape {
 template <class F, int N>
 RunShape run_shape(int T, int rows) {
     constexpr int L = F::kLanes;
+    // Frames of a CTA in whole sequences: 24 threads a frame (192-point rows) do not divide the CTA's
+    // 256, and a share of 256 / 24 frames rounded up would ask for more.
+    constexpr int most_frames = run_threads<N>() / L;
+    static_assert((most_frames * L + 31) / 32 * 32 <= run_threads<N>() && 64 <= run_threads<N>() &&
+                      (F::kIn <= 8 || N <= run_threads<N>()),
+                  "a run's threads exceed the kernel's launch bounds");
     RunShape v;
-    int n = (T * L + run_threads<N>() - 1) / run_threads<N>();
+    int n = (T + most_frames - 1) / most_frames;
     if (N > 32) {  // more, shorter runs (of four frames at least) until the units fill the chip
         // (rounded down: a few units more than fit at once would take a second round of their own)
         const int fill = kRunUnits<F> / rows, most = (T + 3) / 4;
@@ -676,7 +682,7 @@ cudaError_t row_grid(K kern, int threads, size_t smem, long long rows, int* grid
     if (!per_sm) {
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
         if (e != cudaSuccess) return e;
-        if (per_sm < 1) per_sm = 1;
+        if (per_sm < 1) return cudaErrorLaunchOutOfResources;  // no CTA of this shape fits an SM
         std::lock_guard<std::mutex> lock(mu);
         if (known.size() < 4096) known[key] = per_sm;
     }

@@ -368,3 +368,31 @@ def test_coil_and_volume_solves_around_the_deferred_update(R, T):
     recon.recon_solve3(ctx.h, to_dev(b3), to_dev(m3), (2, 2, 2, 2), 0.1, 0.0, 1, 3, out)
     ref = slr3.irls3(b3.astype(np.complex128), m3, 2, 2, 2, 2, 0.1, 0.0, 1, 3)
     assert_close(out.cpu().numpy(), ref, 1e-4)
+
+
+@pytest.mark.parametrize("T,grid", [(10, (256, 192)), (11, (512, 192)), (21, (256, 192)), (21, (512, 192)),
+                                    (21, (16, 16, 192)), (31, (192, 192)), (32, (192, 192)), (32, (16, 32, 192)),
+                                    (42, (128, 192)), (42, (32, 16, 192)), (44, (192, 192))])
+def test_operator_with_192_point_rows(R, T, grid):
+    """A^H A + lam W with rows of 192 elements, whose 24 threads a frame do not divide a CTA, in frame
+    counts on both sides of a run's ten frames and with enough image rows that the runs are as long
+    as they get: valid and time-circular form and volumes, against FP64: the gate of the operator
+    parity tests (1e-5)."""
+    import torch
+    recon, ctx = R
+    rng = np.random.default_rng(T + grid[0])
+    x = _series(rng, T, *grid)
+    S, full = _hermitian_pairs(rng, 2, int(np.prod(grid[:-1])), grid[-1])
+    S, full = S.reshape((3,) + grid), full.reshape((2, 2) + grid)
+    m = (rng.random((T,) + grid) < 0.4).astype(np.uint8)
+    axes = tuple(range(1, x.ndim))
+    aha = np.fft.ifftn(m * np.fft.fftn(x, axes=axes), axes=axes)
+    xd = to_dev(x)
+    y = torch.empty_like(xd)
+    if len(grid) == 3:
+        recon.recon_apply_normal3(ctx.h, to_dev(m), (1, 1, 1, 2), to_dev(S), 0.7, xd, y)
+        assert_close(y.cpu().numpy(), aha + 0.7 * _w(full, x, False), 1e-5)
+        return
+    for circ, variant in ((False, recon.RECON_VARIANT_PROPOSED), (True, recon.RECON_VARIANT_GIRAF)):
+        recon.recon_apply_normal_variant(ctx.h, to_dev(m), (1, 1, 2), variant, to_dev(S), 0.7, xd, y)
+        assert_close(y.cpu().numpy(), aha + 0.7 * _w(full, x, circ), 1e-5)
