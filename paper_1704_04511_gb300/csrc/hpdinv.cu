@@ -828,6 +828,25 @@ RECON_DEV double tri_max(const double* a, const double* b, int m, double prev, i
     return 0.5 * (sh_lo + sh_hi);
 }
 
+// The published word at which a check of `next` steps takes the iteration as ended: strictly fewer steps
+// than that. One that ends with the very step of a check (s or the limit of the steps, or an exhausted
+// space) is checked there as one that goes on, and brought to its last digits in the next turn:
+// whether its end is published yet by then is a matter of time, and the two ways of getting to the
+// value differ in its last bit.
+__host__ __device__ constexpr bool lanc_ended(unsigned int seen, unsigned int next) {
+    return seen >= kLancFin && seen - kLancFin < next;
+}
+// A check of `next` steps, of an iteration that ends after m >= next, does the same with every word that it
+// may find published.
+constexpr bool lanc_timeless() {
+    for (unsigned int next = 8; next <= kLanczosMax; next += 2)
+        for (unsigned int m = next; m <= kLanczosMax; ++m)
+            for (unsigned int k = next; k <= m; ++k)
+                if (lanc_ended(k, next) != lanc_ended(kLancFin + m, next)) return false;
+    return true;
+}
+static_assert(lanc_timeless(), "lambda_max depends on how far the workers are");
+
 // The checking CTA (see above). It alone writes lmax_out and the status word, and hands the two
 // words it shares with CTA 0 (gb->pad: published steps, stop request) back zeroed, as the host
 // leaves them when it zeroes the scratch header.
@@ -852,7 +871,7 @@ RECON_DEV void lanczos_check(const LancMat& L, GridBar* gb, const CoopFault& fau
             return;
         }
         if (stands) break;  // the workers have left as well
-        const bool fin = sh_seen >= kLancFin && sh_seen - kLancFin <= next;
+        const bool fin = lanc_ended(sh_seen, next);
         const int m = (int)(fin ? sh_seen - kLancFin : next);
         // in units of 2^scale ~ alpha_0 (exact), so that FP32 holds any matrix
         const double a0 = m > 0 ? __ldcg(L.ab) : 0.0;

@@ -396,3 +396,29 @@ def test_operator_with_192_point_rows(R, T, grid):
     for circ, variant in ((False, recon.RECON_VARIANT_PROPOSED), (True, recon.RECON_VARIANT_GIRAF)):
         recon.recon_apply_normal_variant(ctx.h, to_dev(m), (1, 1, 2), variant, to_dev(S), 0.7, xd, y)
         assert_close(y.cpu().numpy(), aha + 0.7 * _w(full, x, circ), 1e-5)
+
+
+@pytest.mark.parametrize("filt", [(8, 1, 1), (5, 2, 1), (4, 3, 1), (7, 1, 2), (8, 2, 1), (6, 3, 1), (6, 2, 2),
+                                  (8, 8, 1), (8, 4, 3)])
+@pytest.mark.parametrize("kind", ["random", "decades", "rank"])
+def test_lambda_max_at_the_last_step(R, filt, kind):
+    """The same bits from every launch where the iteration can end with the step of a check: s = 8 to
+    24 (the end of the Krylov space), 64 and 96 (the limit of the steps) and matrices of rank 8 and 12,
+    and the value within 4 s 2^-53 + 1e-13."""
+    import torch
+    recon, ctx = R
+    N1, N2, M = filt
+    s = N1 * N2 * M
+    rng = np.random.default_rng(s)
+    if kind == "rank":
+        X = rng.standard_normal((min(8 + s % 8, s), s)) + 1j * rng.standard_normal((min(8 + s % 8, s), s))
+        G = X.conj().T @ X
+    else:
+        G = _spectrum(kind, s, rng)
+    G = 0.5 * (G + G.conj().T)
+    S = torch.empty((M * (M + 1) // 2, 32, 32), dtype=torch.complex64, device="cuda")
+    Gd = to_dev(np.ascontiguousarray(G.T))
+    lam = np.linalg.eigvalsh(G)[-1]
+    got = {recon.recon_weight(ctx.h, (8, 32, 32), filt, Gd, -1.0, 0.0, S) for _ in range(200)}
+    assert len(got) == 1
+    assert abs(got.pop() - lam) <= (4 * s * 2.0 ** -53 + 1e-13) * lam
