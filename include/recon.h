@@ -157,7 +157,8 @@ int recon_poll(recon_ctx* c, int ticket, int* done);
  *   workspace stay the same (one graph per slot). A context without a memory budget copies the masks
  *   (and coil maps) into its workspace and the image out of it, 9 T P Q (+ 8 n_coils P Q) bytes a slot
  *   where the device has them, so that the graph serves any buffers; with a budget the graph points
- *   into the caller's buffers and is captured anew when these change. Not used for the
+ *   into the caller's buffers and is captured anew when these change, and so does that of a slot that
+ *   found no memory for the copies, until its workspace changes. Not used for the
  *   eigensolver-library path or while launch classes are timed.
  * RECON_OPT_AUTOTUNE: on the first solve of each shape (P, Q, T, R, coils) the context times the
  *   column passes of the CG operator with tiles of 8, 16 and 32 columns (CUDA events on its own

@@ -82,6 +82,7 @@ struct recon_ctx {
     // Batch slots: each has its own stream, workspace and eigensolver handle. The fields
     // stream / bufs / solver above always hold the ACTIVE slot's; the others are parked here.
     unsigned long ws_gen = 0;          // bumped when the active slot's workspace moves
+    unsigned long unstaged = 0;        // the ws_gen at which it found no memory for staging copies
     struct GraphKey {
         int T, P, Q, N1, N2, M, irls, cg, bf16, method, R, N3;
         double lambda, p, gamma, eps0_frac;
@@ -117,7 +118,7 @@ struct recon_ctx {
         bool own_stream = false;
         std::map<std::string, Buf> bufs;
         cusolverDnHandle_t solver = nullptr;
-        unsigned long ws_gen = 0;
+        unsigned long ws_gen = 0, unstaged = 0;
         GraphKey gkey = {};
         cudaGraphExec_t gexec = nullptr;
         GraphProf* gprof = nullptr;
@@ -238,23 +239,41 @@ void prof_collect(recon_ctx* c) {
     c->ev_used = 0;
 }
 
-// Free the staging copies of every slot (stage_solve), as when other buffers find no memory: the
-// graphs that point into them are stale then. Work queued on another slot may still use them.
-void release_staging(recon_ctx* c) {
-    cudaDeviceSynchronize();
-    auto drop = [c](std::map<std::string, Buf>& bufs, unsigned long& gen) {
-        for (const char* name : {"gx", "gm", "gc"}) {
-            auto it = bufs.find(name);
-            if (it == bufs.end()) continue;
-            if (it->second.ptr) cudaFree(it->second.ptr);
-            c->allocated -= it->second.bytes;
-            bufs.erase(it);
+// The staging copies of one slot (stage_solve): whether it has any, and freeing them (the graphs that
+// point into them are stale then).
+constexpr const char* kStaging[] = {"gx", "gm", "gc"};
+bool has_staging(const std::map<std::string, Buf>& bufs) {
+    for (const char* name : kStaging) {
+        auto it = bufs.find(name);
+        if (it != bufs.end() && it->second.ptr) return true;
+    }
+    return false;
+}
+void drop_staging(recon_ctx* c, std::map<std::string, Buf>& bufs, unsigned long& gen) {
+    for (const char* name : kStaging) {
+        auto it = bufs.find(name);
+        if (it == bufs.end()) continue;
+        if (it->second.ptr) {
+            cudaFree(it->second.ptr);
             ++gen;
         }
-    };
-    drop(c->bufs, c->ws_gen);
+        c->allocated -= it->second.bytes;
+        bufs.erase(it);
+    }
+}
+
+// Free the staging copies of every slot, as when other buffers find no memory; false: there are none.
+// Work queued on another slot may still use them.
+bool release_staging(recon_ctx* c) {
+    bool any = has_staging(c->bufs);
+    for (size_t i = 0; i < c->slots.size() && !any; ++i)
+        any = (int)i != c->active && has_staging(c->slots[i].bufs);
+    if (!any) return false;
+    cudaDeviceSynchronize();
+    drop_staging(c, c->bufs, c->ws_gen);
     for (size_t i = 0; i < c->slots.size(); ++i)
-        if ((int)i != c->active) drop(c->slots[i].bufs, c->slots[i].ws_gen);
+        if ((int)i != c->active) drop_staging(c, c->slots[i].bufs, c->slots[i].ws_gen);
+    return true;
 }
 
 // Device buffer `name` of at least `bytes` (contents undefined on growth). staging: one that the
@@ -269,16 +288,15 @@ int ensure(recon_ctx* c, const char* name, size_t bytes, void** out, bool stagin
         cudaFree(b.ptr);
         c->allocated -= b.bytes;
         b = Buf{};
+        ++c->ws_gen;  // captured solves that point into this workspace are stale now
     }
-    ++c->ws_gen;  // captured solves that point into this workspace are stale now
     const size_t want = bytes < 256 ? 256 : bytes;
     if (c->budget && c->allocated + want > c->budget)
         return fail(c, RECON_ENOMEM, std::string("workspace budget exceeded allocating ") + name);
     cudaError_t e = cudaMalloc(&b.ptr, want);
     if (e != cudaSuccess && !staging) {  // the staging copies make room for the rest
         cudaGetLastError();
-        release_staging(c);
-        e = cudaMalloc(&b.ptr, want);
+        if (release_staging(c)) e = cudaMalloc(&b.ptr, want);
     }
     if (e != cudaSuccess) {
         b = Buf{};
@@ -286,6 +304,7 @@ int ensure(recon_ctx* c, const char* name, size_t bytes, void** out, bool stagin
         return fail(c, RECON_ENOMEM, std::string("cudaMalloc failed for ") + name + ": " +
                                          cudaGetErrorString(e));
     }
+    ++c->ws_gen;
     b.bytes = want;
     c->allocated += want;
     *out = b.ptr;
@@ -639,6 +658,7 @@ int select_slot(recon_ctx* c, int i) {
     park.bufs = std::move(c->bufs);
     park.solver = c->solver;
     park.ws_gen = c->ws_gen;
+    park.unstaged = c->unstaged;
     park.gkey = c->gkey;
     park.gexec = c->gexec;
     park.gprof = c->gprof;
@@ -656,6 +676,7 @@ int select_slot(recon_ctx* c, int i) {
     c->bufs = std::move(next.bufs);
     c->solver = next.solver;
     c->ws_gen = next.ws_gen;
+    c->unstaged = next.unstaged;
     c->gkey = next.gkey;
     c->gexec = next.gexec;
     c->gprof = next.gprof;
@@ -915,9 +936,10 @@ recon_ctx::GraphKey graph_key(recon_ctx* c, const Solve& sv) {
 // (solves on changing buffers: 32x32x8, 20 x 10: 6.7 -> 4.1 ms; 256x256x16, 30 x 15: 24.8 ->
 // 19.8; four of these at 10 x 15: 22.2 -> 18.3), against three copies of 8 E + E bytes in
 // and out. Contexts with a budget keep to recon_bytes_needed and to the caller's buffers, and so
-// does a solve that finds no memory for the copies. False: not staged.
+// does a slot that found no memory for the copies, until its workspace changes: asking again on every
+// call would cost a failing allocation each time, and take the slot's graph with it. False: not staged.
 bool stage_solve(recon_ctx* c, Solve* sv) {
-    if (c->budget) return false;
+    if (c->budget || (c->unstaged && c->unstaged == c->ws_gen)) return false;
     void *x = nullptr, *m = nullptr, *co = nullptr;
     const size_t ne = sv->d.elems();
     const std::string err = c->err;
@@ -927,7 +949,9 @@ bool stage_solve(recon_ctx* c, Solve* sv) {
     if (!rc && cb) rc = ensure(c, "gc", cb, &co, true);
     if (rc) {
         c->err = err;
-        release_staging(c);
+        cudaStreamSynchronize(c->stream);  // this slot's copies only; nothing else uses them
+        drop_staging(c, c->bufs, c->ws_gen);
+        c->unstaged = c->ws_gen;
         return false;
     }
     Solve a = *sv;  // x0 straight from the caller's buffers
