@@ -648,13 +648,16 @@ __global__ void hdiag_kernel(const double2* __restrict__ H, int N1, int N2, int 
 // reduction after the barrier. CTA 0 publishes (alpha_k, beta_{k-1}^2).
 //
 // The last CTA takes no part in the barriers: it takes the largest eigenvalue of the tridiagonal of
-// the first 8, 10, 12, ... published steps and asks CTA 0 to end the iteration once it has not grown
-// by 5e-16 of itself over two steps (the workers are a few steps ahead by then; at the last step the
-// value is taken as it is). lambda_max of Grams of image series stands after ~20-26 steps, that of
-// random series with a 0.2 % top gap after ~40-50; a fixed 64 steps with two barriers each took 805 us
-// at s = 243 (12.6 us a step) on every first iteration. The bound of a step is latency: the barrier,
-// the dependent FP64 chains (64 cycles an operation) and the FP64 issue of the redundant vector work.
-// s = 243 series: 137 us (recon_weight with its own eps 1100 -> 424 us).
+// the first 8, 10, 12, ... published steps and asks CTA 0 to end the iteration once it has not grown by
+// 5e-16 of itself from one check to the next (the workers are a few steps ahead by then; at the last
+// step the value is taken as it is). A check of m steps takes about 0.36 m + 2 us, a step 5.7 at s = 243:
+// checked every second step, matrices that converge slowly waited for the checks, so from 28 steps on it
+// is every fourth one (random series at s = 243: 749 -> 636 us a weight; the steps of larger matrices take
+// longer than the checks, and at s = 315 and 486 the four extra steps cost 20 us). lambda_max of Grams of
+// image series stands after ~20-26 steps, that of random series with a 0.2 % top gap after ~40-50; a fixed
+// 64 steps with two barriers each took 805 us at s = 243 (12.6 us a step) on every first iteration. The
+// bound of a step is latency: the barrier, the dependent FP64 chains (64 cycles an operation) and the FP64
+// issue of the redundant vector work. s = 243 series: 137 us (recon_weight with its own eps 1100 -> 424 us).
 struct LancMat {
     const double2* G;   // s x s column-major, Hermitian
     double2* w;         // G q of a step, two buffers of s
@@ -857,7 +860,7 @@ RECON_DEV void lanczos_check(const LancMat& L, GridBar* gb, const CoopFault& fau
     double theta = 0.0, lower = 0.0;
     bool stands = false;
     int scale = 0;
-    for (unsigned int next = 8;; next += 2) {
+    for (unsigned int next = 8;; next += next < 28 ? 2 : next < 48 ? 4 : 8) {
         // the steps up to the next check, or all there are: never more, so that the value does not
         // depend on how far the workers have got meanwhile
         if (threadIdx.x == 0) {
