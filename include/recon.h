@@ -127,8 +127,8 @@ int recon_solve_batch_host(recon_ctx* c, int n, recon_dims d, const void* const*
  * (grid, frame count and filter support may all differ; the parameters prm are shared), slot i
  * reading kspace[i], masks[i] and writing image_out[i]. Run as recon_solve_batch runs its slots:
  * independent slots by default; with RECON_OPT_BATCH_GROUP = g the whole batch is one CUDA graph
- * and every g consecutive slots share one Lanczos, one eps and one FP64 sweep launch per IRLS
- * iteration, each matrix of its own size s_i = N1 N2 M (the sweep runs as many pivot steps as
+ * and every g consecutive slots share one eps and one FP64 sweep launch per IRLS iteration (Lanczos
+ * on the first one: a launch per solve, side by side), each matrix of its own size s_i = N1 N2 M (the sweep runs as many pivot steps as
  * the largest needs). Results are bitwise identical to solving each problem alone.
  * 1 <= n <= RECON_MAX_BATCH; synchronous. */
 int recon_solve_many(recon_ctx* c, int n, const recon_dims* d, const recon_filter* f,
@@ -186,8 +186,8 @@ int recon_poll(recon_ctx* c, int ticket, int* done);
  *   the FP64 weight of its solves on the sweep path (p = 0, RECON_WEIGHT_AUTO, graphs on).
  *   0: every solve has its own graph and stream, its weight launches its own (independent slots).
  *   g >= 1: the whole batch is one CUDA graph; every IRLS iteration the solves of each group of g
- *   consecutive slots join for ONE Lanczos (first iteration), one eps and ONE sweep launch that
- *   serve all of them (one grid barrier per pivot step for the group), then continue on their
+ *   consecutive slots (on the first one after a Lanczos launch each, side by side) join for one eps
+ *   and ONE sweep launch that serve all of them (one grid barrier per pivot step for the group), then continue on their
  *   own streams; with several groups the groups' weight launches take turns, so each overlaps
  *   the other groups' CG. Results are bitwise identical to solving each problem alone. */
 #define RECON_OPT_BATCH_GROUP 7

@@ -1029,16 +1029,20 @@ int iter_gram(recon_ctx* c, Solve& sv) {
     return RECON_OK;
 }
 
-// The FP64 weight of a group of solves (p = 0 sweep path) in shared launches on the active
-// stream: at n = 0 a Lanczos launch for each lambda_max, then one eps launch and one sweep
-// launch for all. The group leader's scratch holds the barriers of the shared launches.
+// lambda_max of the solve's first Gram (active slot's stream): the solves of a group run theirs side
+// by side, one launch each, before they join: four 128x128x12 solves of one iteration 1880 us, with one
+// after the other on the leader's stream 3000, with one launch for all of them (64 fixed steps) 2600.
+int iter_lanczos(recon_ctx* c, Solve& sv) {
+    ProfScope ps(c, RECON_PROF_LANCZOS);
+    RC_CUDA(recon::launch_lanczos_lmax(sv.d.s(), sv.w.G, sv.w.lanc, sv.w.lmax, sv.w.kerr + 1, c->stream,
+                                       sv.w.fault));
+    return RECON_OK;
+}
+
+// The FP64 weight of a group of solves (p = 0 sweep path, lambda_max known) in shared launches on the
+// active stream: one eps launch and one sweep launch for all. The group leader's scratch holds the
+// barriers of the shared launches.
 int group_weight(recon_ctx* c, Solve* grp, int cnt, int n) {
-    if (n == 0) {
-        ProfScope ps(c, RECON_PROF_LANCZOS);
-        for (int b = 0; b < cnt; ++b)
-            RC_CUDA(recon::launch_lanczos_lmax(grp[b].d.s(), grp[b].w.G, grp[b].w.lanc, grp[b].w.lmax,
-                                               grp[b].w.kerr + 2 * n + 1, c->stream, grp[b].w.fault));
-    }
     {
         const double* lmax[recon::kMaxHpdBatch];
         double* eps[recon::kMaxHpdBatch];
@@ -1101,6 +1105,7 @@ int batch_capture(recon_ctx* c, std::vector<Solve>& sv, int group) {
         for (int i = 0; i < n && !rc; ++i) {
             rc = select_slot(c, i);
             if (!rc) rc = iter_gram(c, sv[i]);
+            if (!rc && it == 0) rc = iter_lanczos(c, sv[i]);
             if (!rc) RC_CUDA(cudaEventRecord(ev(i), c->stream));
         }
         for (int g0 = 0; g0 < n && !rc; g0 += group) {
