@@ -7,6 +7,8 @@
 // sampling mask between a forward and an inverse transform so that A^H A needs one column pass.
 #include <cuda_bf16.h>
 
+#include <utility>
+
 #include "common.cuh"
 #include "kernels.h"
 #include "regfft.cuh"
@@ -338,6 +340,7 @@ col_kernel(const float2* in, float2* out, const uint8_t* __restrict__ mask,
 constexpr int kR256Rows = 4;  // rows per 64-thread CTA, one half-warp per row
 
 // Pass A of a CG step for 256-point rows (same contract as row_fwd_pupdate_kernel).
+template <bool kX>
 __global__ void __launch_bounds__(64)
 row_fwd_pupdate_256_kernel(const float2* __restrict__ r, float2* __restrict__ p,
                            float2* __restrict__ x, const double* __restrict__ alpha,
@@ -354,14 +357,14 @@ row_fwd_pupdate_256_kernel(const float2* __restrict__ r, float2* __restrict__ p,
     const int row = blockIdx.x * kR256Rows + lr;
     const bool ok = row < nrows;
     const size_t base = (size_t)row * 256 + j;
-    float2 u[16], pv[16], xv[16];
+    float2 u[16], pv[16], xv[kX ? 16 : 1];
     if (ok) {
 #pragma unroll
         for (int n1 = 0; n1 < 16; ++n1) u[n1] = r[base + 16 * n1];
         if (!first) {
 #pragma unroll
             for (int n1 = 0; n1 < 16; ++n1) pv[n1] = p[base + 16 * n1];
-            if (alpha) {
+            if constexpr (kX) {
 #pragma unroll
                 for (int n1 = 0; n1 < 16; ++n1) xv[n1] = x[base + 16 * n1];
             }
@@ -380,10 +383,12 @@ row_fwd_pupdate_256_kernel(const float2* __restrict__ r, float2* __restrict__ p,
     __syncthreads();  // tw2, beta
     if (!first) {
         const float beta = beta_s;
-        if (ok && alpha) {
-            const float al = (float)alpha[0];
+        if constexpr (kX) {
+            if (ok) {
+                const float al = (float)alpha[0];
 #pragma unroll
-            for (int n1 = 0; n1 < 16; ++n1) x[base + 16 * n1] = axpy(al, pv[n1], xv[n1]);
+                for (int n1 = 0; n1 < 16; ++n1) x[base + 16 * n1] = axpy(al, pv[n1], xv[n1]);
+            }
         }
 #pragma unroll
         for (int n1 = 0; n1 < 16; ++n1) {
@@ -407,6 +412,7 @@ row_fwd_pupdate_256_kernel(const float2* __restrict__ r, float2* __restrict__ p,
 // 64-thread CTA, 8 lanes per row (row_dft128 in regfft.cuh).
 constexpr int kR128Rows = 8;
 
+template <bool kX>
 __global__ void __launch_bounds__(64)
 row_fwd_pupdate_128_kernel(const float2* __restrict__ r, float2* __restrict__ p,
                            float2* __restrict__ x, const double* __restrict__ alpha,
@@ -423,14 +429,14 @@ row_fwd_pupdate_128_kernel(const float2* __restrict__ r, float2* __restrict__ p,
     const int row = blockIdx.x * kR128Rows + lr;
     const bool ok = row < nrows;
     const size_t base = (size_t)row * 128 + j;
-    float2 u[16], pv[16], xv[16];
+    float2 u[16], pv[16], xv[kX ? 16 : 1];
     if (ok) {
 #pragma unroll
         for (int n1 = 0; n1 < 16; ++n1) u[n1] = r[base + 8 * n1];
         if (!first) {
 #pragma unroll
             for (int n1 = 0; n1 < 16; ++n1) pv[n1] = p[base + 8 * n1];
-            if (alpha) {
+            if constexpr (kX) {
 #pragma unroll
                 for (int n1 = 0; n1 < 16; ++n1) xv[n1] = x[base + 8 * n1];
             }
@@ -449,10 +455,12 @@ row_fwd_pupdate_128_kernel(const float2* __restrict__ r, float2* __restrict__ p,
     __syncthreads();  // tw8, beta
     if (!first) {
         const float beta = beta_s;
-        if (ok && alpha) {
-            const float al = (float)alpha[0];
+        if constexpr (kX) {
+            if (ok) {
+                const float al = (float)alpha[0];
 #pragma unroll
-            for (int n1 = 0; n1 < 16; ++n1) x[base + 8 * n1] = axpy(al, pv[n1], xv[n1]);
+                for (int n1 = 0; n1 < 16; ++n1) x[base + 8 * n1] = axpy(al, pv[n1], xv[n1]);
+            }
         }
 #pragma unroll
         for (int n1 = 0; n1 < 16; ++n1) {
@@ -711,6 +719,7 @@ col_mask_64_kernel(float2* t, const uint8_t* __restrict__ mask, int Q, float sca
 // (rows 8 p1 + p2, p2 = blockIdx.x % 8, 8 lanes per row as in row_fwd_pupdate_128_kernel), then the
 // 16-point DFT over p1 of each of the 128 columns and the twiddle w128^(p2 k1) (P = Q = 128, so the
 // one length-128 table serves both directions); Y[k1][p2] goes to row 8 k1 + p2 of t.
+template <bool kX>
 __global__ void __launch_bounds__(128)
 row_fwd_col1_128_kernel(const float2* __restrict__ r, float2* __restrict__ p,
                         float2* __restrict__ x, const double* __restrict__ alpha,
@@ -727,13 +736,13 @@ row_fwd_col1_128_kernel(const float2* __restrict__ r, float2* __restrict__ p,
     const int p2 = blockIdx.x % 8;
     const size_t sbase = (size_t)(blockIdx.x / 8) * 128 * 128;
     const size_t base = sbase + (size_t)(8 * p1 + p2) * 128 + j;
-    float2 u[16], pv[16], xv[16];
+    float2 u[16], pv[16], xv[kX ? 16 : 1];
 #pragma unroll
     for (int n1 = 0; n1 < 16; ++n1) u[n1] = r[base + 8 * n1];
     if (!first) {
 #pragma unroll
         for (int n1 = 0; n1 < 16; ++n1) pv[n1] = p[base + 8 * n1];
-        if (alpha) {
+        if constexpr (kX) {
 #pragma unroll
             for (int n1 = 0; n1 < 16; ++n1) xv[n1] = x[base + 8 * n1];
         }
@@ -748,7 +757,7 @@ row_fwd_col1_128_kernel(const float2* __restrict__ r, float2* __restrict__ p,
     __syncthreads();  // tw8, beta
     if (!first) {
         const float beta = beta_s;
-        if (alpha) {
+        if constexpr (kX) {
             const float al = (float)alpha[0];
 #pragma unroll
             for (int n1 = 0; n1 < 16; ++n1) x[base + 8 * n1] = axpy(al, pv[n1], xv[n1]);
@@ -1104,36 +1113,64 @@ cudaError_t launch_adjoint(const Dims& d, const Twiddles& tw, const void* b, int
     return row_fft<true>(d.Q, t, x, d.T * d.rows(), 1.0f, tw.twQ, st);
 }
 
+// Pass A of 128- and 256-point rows comes in two kernels, with and without x (kX): its 16 values a thread
+// take 126 registers instead of 94, and fewer CTAs an SM (the other lengths hold eight, 70 registers, and
+// two forms of them gained nothing: CTAs that start ahead of their turn are packed on the SMs that the
+// update pass leaves free, and 56 registers let more of them; 128x32x60 took 18.4 instead of 15.0 us a step).
+template <bool kX>
+cudaError_t row_fwd_pupdate(const Dims& d, const Twiddles& tw, const float2* r, float2* p, float2* x,
+                            const double* alpha, float2* t, const Partials& rr, const double* rr_prev,
+                            double* rr_out, int first, cudaStream_t st) {
+    const int nrows = d.T * d.rows();
+    const double* parts = rr.parts;
+    if (vol_fold(d))  // the row DFT and the first half of the length-P DFT (see vol_fold)
+        return launch_pdl(row_fwd_col1_128_kernel<kX>, dim3(d.T * d.R * 8), dim3(128), 0, st, r, p, x, alpha,
+                          t, parts, rr.n, rr_prev, rr_out, first, tw.twQ);
+    if (d.Q == 256)
+        return launch_pdl(row_fwd_pupdate_256_kernel<kX>, dim3((nrows + kR256Rows - 1) / kR256Rows), dim3(64),
+                          0, st, r, p, x, alpha, t, nrows, parts, rr.n, rr_prev, rr_out, first, tw.twQ);
+    return launch_pdl(row_fwd_pupdate_128_kernel<kX>, dim3((nrows + kR128Rows - 1) / kR128Rows), dim3(64), 0,
+                      st, r, p, x, alpha, t, nrows, parts, rr.n, rr_prev, rr_out, first, tw.twQ);
+}
+
+// CTAs of 128- or 256-point pass A that the chip holds at once.
+template <bool kX>
+int row_fwd_wave(int Q) {
+    static const auto per_sm = [] {
+        std::pair<int, int> n{0, 0};
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n.first, row_fwd_pupdate_128_kernel<kX>, 64, 0) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n.second, row_fwd_pupdate_256_kernel<kX>, 64, 0) != cudaSuccess)
+            n = {0, 0};
+        return n;
+    }();
+    return (Q == 128 ? per_sm.first : per_sm.second) * num_sms();
+}
+
+bool x_with_row_fwd(const Dims& d, bool coils) {
+    const bool two_forms = !coils && (d.Q == 128 || d.Q == 256);
+    if (d.elems() < (size_t)1 << (d.Q == 128 && two_forms && d.R == 1 ? 19 : 18)) return false;
+    if (!two_forms || d.R > 1) return true;
+    const int rows = d.Q == 128 ? kR128Rows : kR256Rows, ctas = (d.T * d.P + rows - 1) / rows;
+    return ctas <= row_fwd_wave<true>(d.Q) || ctas > row_fwd_wave<false>(d.Q);
+}
+
 cudaError_t launch_row_fwd_pupdate(const Dims& d, const Twiddles& tw, const float2* r, float2* p,
                                    float2* x, const double* alpha, float2* t, const Partials& rr,
-                                   const double* rr_prev,
-                                   double* rr_out, int first, cudaStream_t st) {
-    const int nrows = d.T * d.rows();
-    if (vol_fold(d))  // the row DFT and the first half of the length-P DFT (see vol_fold)
-        return launch_pdl(row_fwd_col1_128_kernel, dim3(d.T * d.R * 8), dim3(128), 0, st, r, p, x, alpha, t,
-                          (const double*)rr.parts, rr.n, rr_prev, rr_out, first, tw.twQ);
-    if (d.Q == 256) {
-        const int grid = (nrows + kR256Rows - 1) / kR256Rows;
-        return launch_pdl(row_fwd_pupdate_256_kernel, dim3(grid), dim3(64), 0, st, r, p, x, alpha, t,
-                          nrows,
-                          (const double*)rr.parts, rr.n, rr_prev, rr_out, first, tw.twQ);
-    }
-    if (d.Q == 128) {
-        const int grid = (nrows + kR128Rows - 1) / kR128Rows;
-        return launch_pdl(row_fwd_pupdate_128_kernel, dim3(grid), dim3(64), 0, st, r, p, x, alpha, t,
-                          nrows,
-                          (const double*)rr.parts, rr.n, rr_prev, rr_out, first, tw.twQ);
-    }
+                                   const double* rr_prev, double* rr_out, int first, cudaStream_t st) {
+    if (first) alpha = nullptr;
     switch (d.Q) {
-#define CASE(N)                                                                              \
-    case N: {                                                                                \
-        const int grid = (nrows + row_seqs<N>() - 1) / row_seqs<N>();                        \
-        return launch_pdl(row_fwd_pupdate_kernel<N>, dim3(grid), dim3(row_threads<N>()), 0, st, r, p, \
-                          x, alpha, t, \
-                          nrows, (const double*)rr.parts, rr.n, rr_prev, rr_out, first, tw.twQ); \
-    }
+#define CASE(N)                                                                                            \
+    case N:                                                                                                \
+        return launch_pdl(row_fwd_pupdate_kernel<N>,                                                       \
+                          dim3((d.T * d.rows() + row_seqs<N>() - 1) / row_seqs<N>()), dim3(row_threads<N>()), \
+                          0, st, r, p, x, alpha, t, d.T * d.rows(), (const double*)rr.parts, rr.n, rr_prev, \
+                          rr_out, first, tw.twQ);
         CASE(16) CASE(32) CASE(64) CASE(192) CASE(512)
 #undef CASE
+        case 128:
+        case 256:
+            return alpha ? row_fwd_pupdate<true>(d, tw, r, p, x, alpha, t, rr, rr_prev, rr_out, first, st)
+                         : row_fwd_pupdate<false>(d, tw, r, p, x, alpha, t, rr, rr_prev, rr_out, first, st);
         default: return cudaErrorInvalidValue;
     }
 }

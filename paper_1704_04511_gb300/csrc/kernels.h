@@ -111,6 +111,13 @@ cudaError_t launch_row_fwd_pupdate(const Dims& d, const Twiddles& tw, const floa
                                    float2* x, const double* alpha, float2* t, const Partials& rr,
                                    const double* rr_prev,
                                    double* rr_out, int first, cudaStream_t st);
+// Whether x += alpha p of a step comes with the next pass A, which reads p anyway (9 instead of 10 series
+// of traffic a step besides the transforms). Not below 2^18 elements (2^19 for image series with 128-point
+// rows), where the passes are bound by latency and pass A is the longer chain, and not where it makes two
+// waves of pass A's CTAs of one (128- and 256-point rows). Steps of solves: 192x192x24 26.4 us instead of 28.1,
+// 512x512x16 113 instead of 119, 256x256x16 25.5 instead of 26.1; 192x128x16 19.7 instead of 19.0; where it took
+// a second wave, 256x256x21 32.3 instead of 30.3, 512x128x21 39.8 instead of 37.6.
+bool x_with_row_fwd(const Dims& d, bool coils);
 // CG step, pass B: t = column-IFFT(mask * column-FFT(t)) / (PQ), in place.
 cudaError_t launch_col_mask(const Dims& d, const Twiddles& tw, float2* t, const uint8_t* mask,
                             cudaStream_t st);

@@ -601,12 +601,7 @@ int cg_block(recon_ctx* c, const Dims& d, const Twiddles& tw, Work& w, const uin
     // the update pass; the update pass leaves those of |r|^2 in w.rparts for the next pass A,
     // which also stores the sum in rr[it] (rr[0] comes from the residual carry).
     recon::Partials pq{w.parts, 0}, rr{w.rparts, 0};
-    // x += alpha p of a step comes with the next pass A, which reads p anyway: 9 instead of 10 series of
-    // traffic a step besides the transforms. Series of 2^18 elements or more (15 steps at 192x128x20 436
-    // instead of 455 us, 512x512x16 1185 instead of 1243, 2 x 15 at 128x128x64x12 10.75 instead of
-    // 11.37 ms); the passes of smaller ones are bound by latency, and pass A is the longer chain
-    // (128x128x12, pixel-wise prior: 978 against 972 us).
-    const bool defer = d.elems() >= (size_t)1 << 18;
+    const bool defer = recon::x_with_row_fwd(d, coils != nullptr);
     for (int it = 0; it < n_cg; ++it) {
         const double* rr_prev = it > 0 ? w.rr + it - 1 : w.rr;
         const double* alpha = it > 0 && defer ? w.pq + it - 1 : nullptr;  // the previous step's, for x

@@ -422,3 +422,11 @@ def test_lambda_max_at_the_last_step(R, filt, kind):
     got = {recon.recon_weight(ctx.h, (8, 32, 32), filt, Gd, -1.0, 0.0, S) for _ in range(200)}
     assert len(got) == 1
     assert abs(got.pop() - lam) <= (4 * s * 2.0 ** -53 + 1e-13) * lam
+
+
+@pytest.mark.parametrize("T,P,Q", [(21, 256, 256), (24, 256, 256), (15, 256, 128), (16, 256, 128), (21, 512, 128),
+                                   (24, 256, 192), (5, 512, 512)])
+def test_cg_steps_where_pass_a_takes_x_or_not(R, T, P, Q):
+    """Series of 2^18 elements and more with x in the first pass and without (second waves of CTAs, 128-point
+    rows below 2^19 elements)."""
+    test_cg_steps_around_the_deferred_update(R, T, P, Q, 3)
