@@ -112,9 +112,18 @@ struct RowFft<128> : RowFft16<128> {
 // straight from global memory into registers (each once per run; no copy of the p rows in shared
 // memory). kDiag: the diagonal form where all M windows of a frame exist (for 3 <= M <= 5, where it saves
 // products and the block and its sums fit the registers; the circular lifting always).
-// The loads of a thread's first task (WLoads) are issued before the transform of the rows.
+// kAhead: the loads of a thread's first task (WLoads) were issued before the transform of the rows; for rows
+// of 128 and more elements up to three taps, more do not fit the registers next to the transform's elements
+// (256x256x16, M = 4: 220 bytes of spills at 80 registers).
+// Runs of eight frames for rows of 128 and 256 elements, and for long rows with more than four taps, whose
+// M - 1 frames on either side and M (M + 1) / 2 weights a run are the most of its loads: runs of two took
+// 36.1 us a CG step at 256x256x16, M = 5, eight take 27.0 (M = 6: 39.5 and 29.9; 512x512x16: 176 and 142).
+// Rows of up to 64 elements are bound by latency: more, shorter tasks (128x16x126, M = 5: 15 steps 353 us with
+// runs of two frames, 440 with four).
 template <class F, int M>
-constexpr int kWRun = M > 4 ? 2 : (F::kIn > 8 ? 8 : 4);
+constexpr int kWRun = F::kIn > 8 ? 8 : M <= 4 ? 4 : F::kLanes <= 8 ? 2 : 8;
+template <class F, int M>
+constexpr bool kWAhead = M <= 3 || (F::kIn <= 8 && F::kLanes <= 8);
 template <int M, int FC>
 struct WLoads {
     float2 pw[FC + 2 * (M - 1)];    // p_{f0 - (M - 1) + i}
@@ -135,14 +144,14 @@ RECON_DEV void w_load(WLoads<M, FC>& v, const float2* __restrict__ prow, const f
     for (int i = 0; i < M * (M + 1) / 2; ++i) v.s[i] = Srow[(size_t)i * npix + c];
 }
 
-template <class F, int N, int M, int FC, bool CIRC, bool kDiag>
+template <class F, int N, int M, int FC, bool CIRC, bool kDiag, bool kAhead>
 RECON_DEV void w_phase(WLoads<M, FC>& v, float2* __restrict__ trow, const float2* __restrict__ prow,
                        const float2* __restrict__ Srow, float2* res, float lam, int T, int n0, int n1,
                        size_t npix) {
     const int k = CIRC ? T : T - M + 1;
     const int nrun = (n1 - n0 + FC - 1) / FC;
     for (int e = threadIdx.x; e < N * nrun; e += blockDim.x) {
-        if (e != (int)threadIdx.x) w_load<N, M, FC, CIRC>(v, prow, Srow, e, T, n0, n1, npix);
+        if (!kAhead || e != (int)threadIdx.x) w_load<N, M, FC, CIRC>(v, prow, Srow, e, T, n0, n1, npix);
         const int c = e % N, f0 = n0 + (e / N) * FC, f1 = min(n1, f0 + FC);
         float2 s[M][M];
 #pragma unroll
@@ -184,8 +193,8 @@ RECON_DEV void w_phase(WLoads<M, FC>& v, float2* __restrict__ trow, const float2
 
 // The terms that w_phase left, added per column over the frames in order (Kahan), and over the columns
 // by FP32 warp trees: a warp's sum in its lane 0, FP64, zero elsewhere. Columns c and c + kThreads share
-// an accumulator, so that the sum is that of a CTA of kThreads threads, one column each, whatever the
-// launch shape (CG amplifies the last bits of Re <p, q> on the smallest series).
+// an accumulator, so that the sum of a run is that of a CTA of kThreads threads, one column each, whatever
+// the CTA's threads (CG amplifies the last bits of Re <p, q> on the smallest series).
 template <class F, int N>
 RECON_DEV double w_terms(const float2* res, int T) {
     const int nc = N < kThreads ? N : kThreads;
@@ -241,8 +250,8 @@ InvShape inv_shape(int T) {
 // frames' p from global memory, so the runs are independent), kLanes threads per frame: it
 // inverse-transforms the k-space rows of t (giving A^H A p; the 1/(PQ) scale was applied with the mask;
 // elements in registers, exchange buffers that then hold the transformed rows), adds lam W p, writes q
-// over t and emits a partial of Re <p, q>. Rows of up to 32 elements keep all their frames in one CTA
-// and with it the order of that sum (see w_terms). The pass is bound by latency for image series, by HBM
+// over t and emits a partial of Re <p, q>. Rows of up to 32 elements keep all their frames in one CTA, up
+// to 256 frames of 16-point and 128 of 32-point rows, and with it the order of that sum (see w_terms). The pass is bound by latency for image series, by HBM
 // for volumes. 64x64x21 7.8 -> 4.4 us per launch, 192x192x24 17.4 -> 9.6, 512x512x16 66.6 -> 32.3,
 // against one CTA per row with passes over shared memory and three copies of the row's frames there.
 // Rows of 128 and 256 elements took such copies of p (and of t and S) too, with asynchronous staging
@@ -250,31 +259,51 @@ InvShape inv_shape(int T) {
 // takes 10.5 instead of 11.2 ms, four 256x256x16 solves at once 16.6 instead of 17.9, a single one the
 // same 19.2, 15 steps at 512x128x12 508 instead of 548 us. Registers decide: 80 let two CTAs of 24
 // 256-point frames share an SM (at 128: 671 us for 15 steps at 256x256x24 instead of 633).
-constexpr int kRunThreads = 256;   // most threads of a CTA (512 for rows of up to 32 elements, 384 of 256)
+// Most threads of a CTA. 192-point rows with up to four taps: 16 frames, so that series of 11 to 16 frames
+// need no second run (512x192x11, M = 4: 41.2 us a step with two runs, 37.8 with one); 512-point rows with
+// more: eight frames for the same reason (256x512x5, M = 5: 33.1 us with two runs, 30.4 with one).
+template <int N, int M>
+__host__ __device__ constexpr int run_threads() {
+    return N <= 32 || (N == 512 && M > 4) ? 512 : N == 256 || (N == 192 && M <= 4) ? 384 : 256;
+}
+// CTAs an SM that the registers are held to. More than four taps with 16 elements a thread take 117 to 128
+// registers, one CTA of 256-point rows (256x256x24, M = 5: 41.5 us a step, 43.9 at 80 registers with spills).
+template <int N, int M>
+__host__ __device__ constexpr int run_blocks() {
+    if (N <= 32) return 1;
+    if (M > 4) return N == 192 ? 2 : 1;
+    return N == 256 || N == 192 || (N == 128 && M == 4) ? 2 : 3;
+}
+// Units wanted (CTAs of the shortest runs that fit the chip at once), and frames of the shortest run: eight
+// for 256-point rows and for long rows with more than four taps, as many as a thread of W takes at once; else four.
+// (128x256x5 and x8, M = 3: 14.9 and 14.8 us a step with runs of four frames, 14.0 and 14.3 with one run. With
+// fewer than 128 image rows four: 64x256x24 16.0 us with 256 units, 17.2 with 192.)
 template <int N>
-__host__ __device__ constexpr int run_threads() { return N <= 32 ? 512 : (N == 256 ? 384 : kRunThreads); }
-// Units wanted: four CTAs an SM, two of the larger ones with 16 elements a thread (15 steps at
-// 256x256x16: 480 us, 515 with four).
-template <class F>
-constexpr int kRunUnits = F::kIn > 8 ? 304 : 608;
+constexpr int kRunUnits = N == 256 ? 456 : N == 128 ? 304 : 608;
 struct RunShape {
     int nrun, per, threads, bufs;
 };
-template <class F, int N>
+template <class F, int N, int M>
 RunShape run_shape(int T, int rows) {
     constexpr int L = F::kLanes;
     // Frames of a CTA in whole sequences: 24 threads a frame (192-point rows) do not divide the CTA's
-    // 256, and a share of 256 / 24 frames rounded up would ask for more.
-    constexpr int most_frames = run_threads<N>() / L;
-    static_assert((most_frames * L + 31) / 32 * 32 <= run_threads<N>() && 64 <= run_threads<N>() &&
-                      (F::kIn <= 8 || N <= run_threads<N>()),
+    // threads, and a share of 256 / 24 frames rounded up would ask for more than there are. Series of more
+    // than 16 frames of 192-point rows in runs of ten at most (256x192x24: 32.0 us a step, 34.0 with 12).
+    constexpr int most_frames = run_threads<N, M>() / L;
+    // W's tasks come in rounds of the CTA's threads: half a row more or less, so that no round is nearly
+    // empty (21 frames of 256-point rows: 768 tasks, two rounds of 384 threads or three of 352)
+    constexpr int grain = F::kIn > 8 ? N / 2 : 32;
+    static_assert((most_frames * L + grain - 1) / grain * grain <= run_threads<N, M>() &&
+                      64 <= run_threads<N, M>() && (F::kIn <= 8 || N <= run_threads<N, M>()),
                   "a run's threads exceed the kernel's launch bounds");
     RunShape v;
-    int n = (T + most_frames - 1) / most_frames;
-    if (N > 32) {  // more, shorter runs (of four frames at least) until the units fill the chip
+    const int most = N == 192 && T > 16 && most_frames > 10 ? 10 : most_frames;
+    int n = (T + most - 1) / most;
+    if (N > 32) {  // more, shorter runs until the units fill the chip
         // (rounded down: a few units more than fit at once would take a second round of their own)
-        const int fill = kRunUnits<F> / rows, most = (T + 3) / 4;
-        if (n < fill) n = fill < most ? fill : (n > most ? n : most);
+        const int shortest = (N == 256 && rows >= 128) || (N > 64 && M > 4) ? 8 : 4;
+        const int fill = (N == 256 && rows < 128 ? 304 : kRunUnits<N>) / rows, limit = (T + shortest - 1) / shortest;
+        if (n < fill) n = fill < limit ? fill : (n > limit ? n : limit);
     }
     v.per = (T + n - 1) / n;
     v.nrun = (T + v.per - 1) / v.per;
@@ -284,11 +313,12 @@ RunShape run_shape(int T, int rows) {
     // Rows of 128 and 256 elements: at least a thread per column for W (128x128x12, M = 3: 340 us for 15
     // steps with 64 threads, 326 with 128); warps without a frame have no part in the transform.
     if (F::kIn > 8 && v.threads < N) v.threads = N;
+    v.threads = (v.threads + grain - 1) / grain * grain;
     return v;
 }
 
 template <class F, int N, int M, bool CIRC>
-__global__ void __launch_bounds__(run_threads<N>(), N <= 32 || M > 4 ? 1 : (N == 256 ? 2 : 3))
+__global__ void __launch_bounds__((run_threads<N, M>()), (run_blocks<N, M>()))
 row_inv_w_kernel(float2* t, const float2* __restrict__ p, const float2* __restrict__ S,
                  float lam, int T, int P, int nrun, int per, double* __restrict__ pq_parts,
                  const float2* __restrict__ tw_g) {
@@ -314,7 +344,8 @@ row_inv_w_kernel(float2* t, const float2* __restrict__ p, const float2* __restri
             u[m] = ok ? trow[(size_t)(n0 + fl) * npix + i + m * F::kLanes] : make_float2(0.f, 0.f);
         constexpr int FC = kWRun<F, M>;
         WLoads<M, FC> wl;
-        w_load<N, M, FC, CIRC>(wl, p + (size_t)r1 * N, S + (size_t)r1 * N, threadIdx.x, T, n0, n1, npix);
+        if constexpr (kWAhead<F, M>)
+            w_load<N, M, FC, CIRC>(wl, p + (size_t)r1 * N, S + (size_t)r1 * N, threadIdx.x, T, n0, n1, npix);
         if (!F::kByWarp || n0 + (int)(threadIdx.x & ~31u) / F::kLanes < n1) {
             F::inverse(u, sx, tw, i);
             F::sync();  // the last exchange is read
@@ -325,7 +356,8 @@ row_inv_w_kernel(float2* t, const float2* __restrict__ p, const float2* __restri
             }
         }
         __syncthreads();
-        w_phase<F, N, M, FC, CIRC, true>(wl, trow, p + (size_t)r1 * N, S + (size_t)r1 * N, res, lam, T, n0, n1, npix);
+        w_phase<F, N, M, FC, CIRC, true, kWAhead<F, M>>(wl, trow, p + (size_t)r1 * N, S + (size_t)r1 * N, res,
+                                                         lam, T, n0, n1, npix);
         __syncthreads();  // the terms
         if (un + (int)gridDim.x >= nunit) pdl_trigger();
         tot += w_terms<F, N>(res, n1 - n0);
@@ -418,7 +450,7 @@ coil_row_inv_kernel(float2* t, const float2* __restrict__ p, const float2* __res
         constexpr int FC = M > 4 ? 2 : 4;
         WLoads<M, FC> wl;
         w_load<N, M, FC, false>(wl, p + (size_t)r1 * N, S + (size_t)r1 * N, threadIdx.x, T, 0, T, npix);
-        w_phase<F, N, M, FC, false, false>(wl, trow, p + (size_t)r1 * N, S + (size_t)r1 * N, res, lam, T, 0, T, npix);
+        w_phase<F, N, M, FC, false, false, true>(wl, trow, p + (size_t)r1 * N, S + (size_t)r1 * N, res, lam, T, 0, T, npix);
         __syncthreads();  // the terms
         pdl_trigger();
         const double tot = warps_sum_t0(w_terms<F, N>(res, T), red);
@@ -699,7 +731,7 @@ cudaError_t launch_row_inv_w_NM(const Dims& d, const Twiddles& tw, float2* t, co
     const int rows = d.rows();
     int grid = 0;
     auto k = d.circ ? row_inv_w_kernel<F, N, M, true> : row_inv_w_kernel<F, N, M, false>;
-    const RunShape v = run_shape<F, N>(d.T, rows);
+    const RunShape v = run_shape<F, N, M>(d.T, rows);
     const size_t smem = ((size_t)v.bufs * F::kBuf + N) * sizeof(float2);
     if (smem > kDynSmemFree) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

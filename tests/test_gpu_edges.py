@@ -430,3 +430,20 @@ def test_cg_steps_where_pass_a_takes_x_or_not(R, T, P, Q):
     """Series of 2^18 elements and more with x in the first pass and without (second waves of CTAs, 128-point
     rows below 2^19 elements)."""
     test_cg_steps_around_the_deferred_update(R, T, P, Q, 3)
+
+
+@pytest.mark.parametrize("T,P,Q,M", [(8, 16, 256, 5), (9, 32, 256, 6), (17, 256, 256, 4), (21, 256, 256, 5),
+                                     (6, 16, 256, 6), (33, 16, 256, 4), (25, 64, 128, 5), (21, 128, 128, 4),
+                                     (33, 16, 128, 6), (17, 16, 128, 3)])
+def test_operator_in_frame_runs_of_many_taps(R, T, P, Q, M):
+    """Rows of 128 and 256 elements with four to six taps, whose loads follow the transform, and frame
+    counts that leave a partial round of W's tasks."""
+    test_operator_in_frame_runs(R, T, P, Q, M)
+
+
+@pytest.mark.parametrize("T,P,Q,M", [(11, 512, 192, 4), (16, 64, 192, 4), (17, 64, 192, 3), (17, 64, 192, 6),
+                                     (6, 16, 512, 6), (5, 256, 512, 5), (11, 16, 64, 6), (13, 32, 32, 5),
+                                     (20, 64, 16, 6)])
+def test_operators_of_many_taps(R, T, P, Q, M):
+    """The other row lengths with three to six taps at the edges of their runs of frames."""
+    test_operators_at_run_edges(R, T, P, Q, M)
