@@ -882,12 +882,16 @@ cudaError_t launch_sum_partials(const Partials& in, double* out, cudaStream_t st
     return cudaGetLastError();
 }
 
-// Frames of a run of the residual carry: the longest of 16, 8, 4, 2 that leaves kResFill threads in
-// flight (about 20 warps an SM), 2 for the smallest series.
-constexpr long long kResFill = 100000;
+// Frames of a run of the residual carry: the longest of 16, 8, 4, 2 (no longer than the series needs: the
+// registers are those of the whole run) that leaves enough threads in flight, 2 for the smallest series:
+// about ten warps an SM, and twenty for runs of 16 with up to four taps, whose weights are few to read
+// again (256x256x16, M = 3: two runs 1.3 us less than one; M = 6: one run 4.2 us less than two;
+// 256x512x5, M = 3: runs of 8 37 us a call, of 16 41).
 int resid_run(const Dims& d) {
     int fc = 16;
-    while (fc > 2 && (long long)d.pixels() * ((d.T + fc - 1) / fc) < kResFill) fc /= 2;
+    while (fc > 2 && fc / 2 >= d.T) fc /= 2;
+    auto fill = [&] { return (long long)d.pixels() * ((d.T + fc - 1) / fc); };
+    while (fc > 2 && fill() < (fc == 16 && d.M <= 4 ? 90000 : 50000)) fc /= 2;
     return fc;
 }
 

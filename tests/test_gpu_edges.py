@@ -447,3 +447,11 @@ def test_operator_in_frame_runs_of_many_taps(R, T, P, Q, M):
 def test_operators_of_many_taps(R, T, P, Q, M):
     """The other row lengths with three to six taps at the edges of their runs of frames."""
     test_operators_at_run_edges(R, T, P, Q, M)
+
+
+@pytest.mark.parametrize("first", [False, True])
+@pytest.mark.parametrize("T,P,Q,M", [(4, 512, 512, 3), (5, 256, 512, 5), (16, 256, 256, 6), (8, 256, 128, 6),
+                                     (11, 512, 192, 2), (3, 128, 256, 3), (2, 256, 256, 1)])
+def test_residual_carry_run_lengths(R, T, P, Q, M, first):
+    """Runs no longer than the series, and of 16 frames for many taps."""
+    test_residual_carry(R, T, P, Q, M, first)
