@@ -45,18 +45,27 @@ frame0_max_kernel(const float2* __restrict__ x, size_t npix, unsigned int* __res
 // cycle, and only the steps left over modulo its length are run. The values are bitwise those of
 // running them all; most pixels stand after five steps of 20, a few per cent go round in the last
 // bits. 256x256x16, 20 steps: 31.7 -> 19 us.
+// More than 32 frames (kLong): the times come from the parameters (a constant operand of the unrolled
+// code), the logarithms are formed twice, and four frames beyond T are left out at a time, so that the
+// 64 samples leave registers for five CTAs an SM and 33 frames do not pay for 64. 256x256x33, 20 steps:
+// 73 -> 58 us a call, 5 steps 44 -> 47 (69 with all 64 samples and times in registers, 166 a thread).
 template <int NT>
-__global__ void __launch_bounds__(kT2Threads)
+__global__ void __launch_bounds__(kT2Threads, NT > 32 ? 5 : 0)
 t2fit_kernel(const float2* __restrict__ x, int T, size_t npix, T2Times tm, float frac,
              const unsigned int* __restrict__ amax, int n_gn, float* __restrict__ t2,
              float* __restrict__ amp) {
     const size_t px = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (px >= npix) return;
     const float thr = __fmul_rn(frac, __uint_as_float(amax[0]));
+    constexpr bool kLong = NT > 32;
     float y[NT], tt[NT];
 #pragma unroll
     for (int n = 0; n < NT; ++n) {
         y[n] = n < T ? magnitude_rn(x[(size_t)n * npix + px]) : 0.f;
+        if constexpr (kLong) {
+            tt[n] = tm.t[n];  // 0 beyond T
+            continue;
+        }
         const float t = n < T ? tm.t[n] : 0.f;
         asm volatile("mov.f32 %0, %1;" : "=f"(tt[n]) : "f"(t));  // stays in a register
     }
@@ -70,6 +79,7 @@ t2fit_kernel(const float2* __restrict__ x, int T, size_t npix, T2Times tm, float
     float tbar = 0.f, lbar = 0.f, ly[NT];
 #pragma unroll
     for (int n = 0; n < NT; ++n) {
+        if (kLong && n % 4 == 0 && n >= T) break;
         ly[n] = n < T ? logf(fmaxf(y[n], 1e-30f)) : 0.f;
         tbar += tt[n];  // 0 beyond T
         lbar += ly[n];
@@ -79,8 +89,10 @@ t2fit_kernel(const float2* __restrict__ x, int T, size_t npix, T2Times tm, float
     float sxy = 0.f, sxx = 0.f;
 #pragma unroll
     for (int n = 0; n < NT; ++n) {
+        if (kLong && n % 4 == 0 && n >= T) break;
         const float dt = n < T ? tt[n] - tbar : 0.f;
-        sxy = fmaf(dt, ly[n] - lbar, sxy);
+        const float l = !kLong ? ly[n] : n < T ? logf(fmaxf(y[n], 1e-30f)) : 0.f;
+        sxy = fmaf(dt, l - lbar, sxy);
         sxx = fmaf(dt, dt, sxx);
     }
     float R = fmaxf(-sxy / sxx, kRmin);
@@ -93,6 +105,7 @@ t2fit_kernel(const float2* __restrict__ x, int T, size_t npix, T2Times tm, float
         float a11 = 0.f, a12 = 0.f, a22 = 0.f, g1 = 0.f, g2 = 0.f;
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
+            if (kLong && n % 4 == 0 && n >= T) break;
             const float e = n < T ? expf(-tt[n] * R) : 0.f;
             const float model = A * e;
             const float res = model - y[n];

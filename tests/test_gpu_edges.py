@@ -455,3 +455,9 @@ def test_operators_of_many_taps(R, T, P, Q, M):
 def test_residual_carry_run_lengths(R, T, P, Q, M, first):
     """Runs no longer than the series, and of 16 frames for many taps."""
     test_residual_carry(R, T, P, Q, M, first)
+
+
+@pytest.mark.parametrize("T", [34, 36, 37, 40, 41, 61])
+def test_t2fit_long_series(R, T):
+    """More than 32 frames, on both sides of the groups of four that are left out beyond the last one."""
+    test_t2fit_frame_counts(R, T)
