@@ -223,8 +223,12 @@ coil_row_fwd_kernel(const float2* __restrict__ r, float2* __restrict__ p,
 // slot of the last pass is an input slot of the first one; lengths with a factor of three exchange
 // once more). 192x192x24 9.6 -> 7.3 us per launch, 512x512x16 36.1 -> 29.3, against passes over
 // shared memory. (Four columns per CTA at 512: 30.8 us.)
+template <int N, int C>
+__host__ __device__ constexpr int col_reg_ctas() {  // 64 registers; an SM takes 32 CTAs at most
+    return C * RegFft<N>::kLanes < 32 ? 32 : 1024 / (C * RegFft<N>::kLanes);
+}
 template <int N, int MODE, int C>
-__global__ void __launch_bounds__(C * RegFft<N>::kLanes, 1024 / (C * RegFft<N>::kLanes))  // 64 registers
+__global__ void __launch_bounds__(C * RegFft<N>::kLanes, (col_reg_ctas<N, C>()))
 col_reg_kernel(const void* in_, float2* out, const uint8_t* __restrict__ mask,
                int Q, int mask_frames, float scale, const float2* __restrict__ tw_g) {
     using F = RegFft<N>;
