@@ -47,8 +47,11 @@ def alg_bytes(kind: str, w, n_cg: int) -> float:
     E = w.T * w.P * w.Q * D
     N = w.P * w.Q * D
     npair = w.M * (w.M + 1) // 2
-    # from 2^18 elements on, x += alpha p of every step but the last comes with the next row pass
-    moved = 16.0 * E * (n_cg - 1) / n_cg if E >= 1 << 18 else 0.0  # x read and written there
+    # from 2^18 elements on (2^19 for image series with 128-point rows), x += alpha p of every step but
+    # the last comes with the next row pass (of the workloads here: none is at one of the sizes where
+    # it would take a second wave of CTAs and stays with the update)
+    least = 1 << (19 if D == 1 and w.Q == 128 else 18)
+    moved = 16.0 * E * (n_cg - 1) / n_cg if E >= least else 0.0  # x read and written there
     if kind == "cg_row_fwd":      # read r (+ p), write p and t
         return (24.0 * E + 32.0 * E * (n_cg - 1)) / n_cg + moved
     if kind == "cg_col_mask":     # read t, mask; write t
@@ -751,7 +754,7 @@ def main():
             lockstep["groups"][str(g)] = ent
         recon.recon_set_option(ctx.h, recon.RECON_OPT_BATCH_GROUP, 0)
         lockstep["note"] = ("recon_solve_batch with RECON_OPT_BATCH_GROUP = g: per IRLS iteration "
-                            "one Lanczos / eps / sweep launch per group of g solves; the headline "
+                            "one eps / sweep launch per group of g solves; the headline "
                             "value runs the independent slots (g = 0), measured faster")
 
     # ---- T2 maps of the reconstructed series (recon_t2fit), timed alone with events

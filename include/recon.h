@@ -381,8 +381,9 @@ int recon_apply_normal3(recon_ctx* c, recon_dims3 d, recon_filter3 f, const uint
  *                           (j + M - 1 - m) mod T; Gram, weight and W otherwise as proposed;
  *  RECON_VARIANT_HLR_VOXEL  the pixel-wise Toeplitz prior (Sec. II-D, Eq. MORASA-objective):
  *                           per pixel r the k x M matrix T_r[j][m] = x_{j+M-1-m}(r) (image
- *                           domain), its Gram G_r and weight H_r = (G_r + eps_r I)^(p/2-1) (FP64
- *                           Jacobi eigendecomposition per pixel), eps_r^(0) = eps0_frac *
+ *                           domain), its Gram G_r and weight H_r = (G_r + eps_r I)^(p/2-1) (FP64;
+ *                           p = 0: a Hermitian sweep inverse per pixel, else a Jacobi
+ *                           eigendecomposition), eps_r^(0) = eps0_frac *
  *                           lambda_max(G_r(x0)), eps_r <- eps_r / gamma; W uses S(r) = H_r^T.
  *                           The filter must have N1 = N2 = 1;
  *  RECON_VARIANT_DIRECT     IRLS without the FFT approximations (Sec. IV-A): the exact multi-fold
@@ -403,7 +404,8 @@ int recon_solve_variant(recon_ctx* c, recon_dims d, const void* kspace, const ui
  * HLR_VOXEL: the per-pixel Grams G_r, [P][Q][M][M] complex128 (row-major M x M). */
 int recon_gram_variant(recon_ctx* c, recon_dims d, recon_filter f, int variant, const void* x,
                        void* G_out);
-/* HLR-Voxel weight of x: per pixel G_r, its FP64 eigendecomposition, H_r with eps[r] (device
+/* HLR-Voxel weight of x: per pixel G_r, its FP64 eigendecomposition (p = 0 without lmax_out: the
+ * sweep inverse of G_r + eps[r] I), H_r with eps[r] (device
  * [P][Q] doubles, > 0) and S(r) = H_r^T into S_out (npair x P x Q complex64, the pair layout of
  * recon_weight); lmax_out (device [P][Q] doubles, may be NULL) receives lambda_max(G_r). */
 int recon_voxel_weight(recon_ctx* c, recon_dims d, int M, const void* x, const double* eps,

@@ -214,7 +214,7 @@ RECON_DEV void last_block_sum(double partial, double* parts, unsigned int* count
 
 // Deterministic sum of n doubles in global memory by warp 0 alone (FP64 in 32 lanes only);
 // the result is valid in every lane of warp 0. (The plain loop: in the CG passes, whose own
-// loads are in flight meanwhile, lane_sum's batched loads measured slower.)
+// loads are in flight meanwhile, loads in batches of eight before the additions measured slower.)
 RECON_DEV double warp0_sum_array(const double* a, int n) {
     double v = 0.0;
     for (int i = threadIdx.x; i < n; i += 32) v += a[i];

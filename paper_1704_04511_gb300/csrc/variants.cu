@@ -3,7 +3,7 @@
 //
 // HLR-Voxel (Sec. II-D, Eq. MORASA-objective): one k x M Toeplitz matrix of the temporal signal
 // per pixel, T_r[j][m] = x_{j+M-1-m}(r). voxel_weight_kernel forms, per pixel and in FP64, the
-// Gram G_r = T_r^H T_r, its eigendecomposition by cyclic complex Jacobi rotations, the weight
+// Gram G_r = T_r^H T_r, its eigendecomposition by cyclic complex Jacobi rotations (at p = 0 a Hermitian sweep inverse), the weight
 // H_r = U diag((lambda + eps)^(p/2-1)) U^H and the banded-W matrix S(r) = H_r^T (so that
 // Re <x, W x> = sum_r Tr(H_r G_r)); the CG then runs on the proposed path's kernels. The penalty
 // sum_r ||T_r||_p is one objective with one smoothing eps, scheduled as in Sec. III-C from the
