@@ -48,7 +48,8 @@ frame0_max_kernel(const float2* __restrict__ x, size_t npix, unsigned int* __res
 // More than 32 frames (kLong): the times come from the parameters (a constant operand of the unrolled
 // code), the logarithms are formed twice, and four frames beyond T are left out at a time, so that the
 // 64 samples leave registers for five CTAs an SM and 33 frames do not pay for 64. 256x256x33, 20 steps:
-// 73 -> 58 us a call, 5 steps 44 -> 47 (69 with all 64 samples and times in registers, 166 a thread).
+// 73 us a call by the loop over T, 77 with all 64 samples and times in registers (166 a thread), now 54; 5 steps
+// 44, 68 and 47.
 template <int NT>
 __global__ void __launch_bounds__(kT2Threads, NT > 32 ? 5 : 0)
 t2fit_kernel(const float2* __restrict__ x, int T, size_t npix, T2Times tm, float frac,
